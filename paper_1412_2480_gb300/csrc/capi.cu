@@ -318,17 +318,19 @@ void drop_graph(pic_sim* s) {
     }
 }
 
-// The step in five parts: [step_begin, J = 0, (overflow push)] [dominant particle
+// The step in five parts: [step begin, J = 0, (overflow push)] [dominant particle
 // kernel] [migration] [field solve: rhs, PCG loop, E/B update] [step_end].
 void enqueue_part(pic_sim* s, int part, cudaStream_t st) {
     const FieldArgs a = field_args(s, 0, 0);
     const bool fp64 = s->prm.precision == PIC_FP64;
     switch (part) {
     case kPartPre:
+        if (!fp64) {
+            mixed_enqueue(s->mixed, st, 0);
+            break;
+        }
         launch_step_begin(a, st);
-        if (fp64) cudaMemsetAsync(s->J64, 0, 3 * s->ntot * sizeof(double), st);
-        else cudaMemsetAsync(s->Jfix, 0, 3 * s->ntot * sizeof(long long), st);
-        if (!fp64) mixed_enqueue(s->mixed, st, 0);
+        cudaMemsetAsync(s->J64, 0, 3 * s->ntot * sizeof(double), st);
         break;
     case kPartPush:
         if (!fp64) {
@@ -358,7 +360,7 @@ void enqueue_part(pic_sim* s, int part, cudaStream_t st) {
         break;
     case kPartPost:
         if (!fp64) {
-            mixed_enqueue(s->mixed, st, 2);  // the injector's pairs, then the bin swap
+            mixed_enqueue(s->mixed, st, 2);  // the injector's pairs
         } else if (s->hgrids[0].inject) {
             Fp64InjectArgs in{};
             in.grids = s->dgrids;
@@ -379,7 +381,8 @@ void enqueue_part(pic_sim* s, int part, cudaStream_t st) {
         }
         break;
     case kPartEnd:
-        launch_step_end(a, st);
+        if (fp64) launch_step_end(a, st);
+        else mixed_enqueue(s->mixed, st, 3);
         break;
     default:
         break;
@@ -535,10 +538,10 @@ int build_graph(pic_sim* s) {
 // the same count from the step's structure for direct launches.
 long long step_kernels(pic_sim* s, bool graph) {
     if (graph && s->graph_kernels >= 0) return s->graph_kernels;
-    // step begin and end; field part: explicit half step, update_E, explicit_B, or
-    // zero_x, rhs, update_E, update_B (+ the cooperative solve)
-    long long k = (s->prm.flags & PIC_EXPLICIT) ? 5 : 6;
-    if (!(s->prm.flags & PIC_EXPLICIT) && s->prm.precision == PIC_MIXED32) k -= 1;  // k_rhs_dw zeroes x itself
+    // field part: explicit half step, update_E, explicit_B, or rhs, update_E, update_B
+    // (+ the cooperative solve)
+    long long k = 3;
+    if (s->prm.precision == PIC_FP64) k += (s->prm.flags & PIC_EXPLICIT) ? 2 : 3;  // step begin, end, zero_x
     if (s->prm.precision == PIC_MIXED32) {
         k += mixed_step_kernels(s->mixed);
     } else {
@@ -841,7 +844,7 @@ int init_handle(const pic_params* prm, int n, pic_sim** out) {
     if (prm[0].precision == PIC_FP64) {
         A(dalloc(&s->J64, n3));
     } else {
-        A(dalloc(&s->Jfix, n3));
+        A(dalloc(&s->Jfix, n3 + 1));  // whole pairs of words (k_mixed_begin)
         A(dalloc(&s->bvec, n3));
         A(dalloc(&s->r32, n3));
         A(dalloc(&s->p32, n3));

@@ -11,20 +11,20 @@
 // slots sit at its own offsets.
 //
 // Per step (inside the captured step graph):
-//   0. k_mixed_begin / k_push_overflow: particles parked in the overflow list (no room
+//   0. k_mixed_begin clears the current and the next buffer's counts; k_push_overflow: particles parked in the overflow list (no room
 //      in a bin; normally none) are pushed straight from global memory;
 //   1. k_push_tile<P>, one persistent launch per shape order P present: each CTA takes
-//      the next tile of that order from a device work counter (tiles listed largest
-//      first, so uneven simulations balance across the SMs), stages the FP32 field window
+//      the next tile of that order, or part of a tile, from a device work counter (tiles
+//      listed largest first, so uneven simulations balance across the SMs), stages the FP32 field window
 //      (tile + 2 cells below, 3 above, in x and y) into shared memory and zeroes a
 //      fixed-point current window of the same size. Its particles are its own stayer segment plus the eight
 //      neighbours' outboxes addressed to it. Warps run independently (no block barrier in
 //      the particle loop): each gathers E^n, B^n, pushes (Boris), moves and deposits
 //      J^{n+1/2} (Esirkepov) with native integer shared-memory atomics, then writes each
 //      particle to the next buffer's stayer segment or to the outbox of the neighbour it
-//      moved into, taking slots from warp-aggregated shared-memory counters. The current
+//      moved into, taking slots from warp-aggregated counters. The current
 //      window is added to the global fixed-point current at the end;
-//   2. k_mixed_swap: the buffers swap.
+//   2. k_mixed_end, after the field update: the buffers swap.
 // No global atomics are needed in steady state and no migration kernel runs. A particle
 // found outside its tile is pushed with the same arithmetic and the same current
 // rounding on global memory, so results never depend on bin capacity; a particle that
@@ -43,6 +43,7 @@
 namespace pic {
 
 constexpr int kTileThreads = 256;
+constexpr double kBinSlack = 1.25;  // stayer capacity over the expected particles of a tile
 constexpr int kNbr = 8;          // outboxes per bin, one per neighbouring tile
 constexpr int kSegs = 1 + kNbr;  // count slots per bin: [0] stayers, [1 + o] outbox o
 
@@ -68,9 +69,9 @@ __host__ __device__ __forceinline__ size_t aos(long long k, int f) {
 struct MixedArgs {
     const GridDev* grids;
     const int* tile_grid;  // simulation of each global tile
-    const int* tlist;      // tiles of this launch's shape order, largest first
-    int ntl;               // entries of tlist
-    int* work;             // next entry of tlist to take (zeroed every step)
+    const int2* items;     // work of this launch's shape order: (tile, part), largest tiles first
+    int nitems;
+    int* work;             // next item to take (zeroed every step)
     long long ntot;
     const float* F32;
     long long* Jfix;
@@ -99,10 +100,14 @@ struct MixedState {
     long long nslots = 0, ovf_cap = 0;
     int ntiles_total = 0;
     int* tile_grid = nullptr;     // device [ntiles_total]
-    int* tlist = nullptr;         // device: tiles grouped by shape order, largest first
-    int* work = nullptr;          // device [4]: work counter of each order's launch
+    std::vector<int> host_tile_grid;
+    std::vector<int> tlist;       // tiles grouped by shape order, largest first
     int order_first[4] = {0, 0, 0, 0}, order_n[4] = {0, 0, 0, 0};
+    int2* items = nullptr;        // device: (tile, part) of each order's launch, in tlist's order
+    int item_first[4] = {0, 0, 0, 0}, item_n[4] = {0, 0, 0, 0};
+    int* work = nullptr;          // device [4]: work counter of each order's launch
     size_t smem[4] = {0, 0, 0, 0};  // dynamic shared memory of each order's launch
+    int resident[4] = {0, 0, 0, 0}; // CTAs of each order's launch the device holds at once
     int pblocks[4] = {0, 0, 0, 0};  // persistent CTAs of each order's launch
     std::vector<long long> n;     // live particles [2 g + species]
     unsigned long long* injected = nullptr;  // device [2 ngrids]: pairs added by the injector
@@ -461,6 +466,14 @@ __device__ __forceinline__ void to_overflow(unsigned* op, int* ogs, long long ov
 // ---------------------------------------------------------------------------------
 // 1. Tile kernel
 // ---------------------------------------------------------------------------------
+// Cell of a window node on a periodic axis of n cells: k lies in [-2, n + window), so one
+// wrap does unless the grid is smaller than the window's margins.
+__device__ __forceinline__ int wrap_window(int k, int n) {
+    if (k < 0) k += n;
+    while (k >= n) k -= n;
+    return k;
+}
+
 // Resident CTAs per SM the order-2 tile kernel is compiled for (register budget).
 #ifndef PIC_TILE_MIN_BLOCKS_P2
 #define PIC_TILE_MIN_BLOCKS_P2 3
@@ -487,8 +500,9 @@ k_push_tile(const MixedArgs a) {
         if (threadIdx.x == 0) s_item = atomicAdd(a.work, 1);
         __syncthreads();
         const int item = s_item;
-        if (item >= a.ntl) break;
-        const int t = __ldg(a.tlist + item);  // global tile
+        if (item >= a.nitems) break;
+        const int2 tp = __ldg(a.items + item);
+        const int t = tp.x, part = tp.y;      // global tile, part of its particles
         const int g = __ldg(a.tile_grid + t);
         const GridDev& G = a.grids[g];
         const int lt = t - G.tile_first;      // tile within its simulation
@@ -498,6 +512,7 @@ k_push_tile(const MixedArgs a) {
         const int nx = G.nx, ny = G.ny;
         const int WX = G.wx, NW = G.wx * G.wy;
         const long long cap = G.cap, capo = G.capo, stride = bin_stride(G);
+        const int parts = G.parts;
         int* jw = reinterpret_cast<int*>(smem_raw);  // [0, 3 NW) hi words, [3 NW, 6 NW) lo words
         float* fw = reinterpret_cast<float*>(smem_raw + (size_t)6 * NW * sizeof(int));
         if (threadIdx.x < 2 * kSegs) {
@@ -509,31 +524,9 @@ k_push_tile(const MixedArgs a) {
             s_sent[s][k] = sent;
             s_start[s][k + 1] = (int)min((long long)sent, k == 0 ? cap : capo);  // prefix-summed below
             s_base[s][k] = G.bin_off + b * stride + off;
-            if (threadIdx.x == 0) {
-                int* oin = par ? a.ovf_in[1] : a.ovf_in[0];
-                s_sent[0][kSegs] = oin[t];
-                oin[t] = 0;  // read; the overflow kernel of the next step counts into it again
-            }
+            if (threadIdx.x == 0) s_sent[0][kSegs] = (par ? a.ovf_in[1] : a.ovf_in[0])[t];
             s_out[s][k] = 0;
         }
-        const float* Fg = a.F32 + G.cell_off;
-        for (int idx = threadIdx.x; idx < 6 * NW; idx += blockDim.x) {
-            const int c = idx / NW;
-            const int w = idx - c * NW;
-            const int wy = w / WX;
-            const int wx = w - wy * WX;
-            int gx = ((X0 - 2 + wx) % nx + nx) % nx, s = 1;
-            if (G.walls) {  // conductor images: Ex, By, Bz even, Ey, Ez, Bx odd
-                const bool half = c == 0 || c == 4 || c == 5;
-                gx = wall_col(X0 - 2 + wx, nx, half, !half, s);
-            }
-            const int gy = ((Y0 - 2 + wy) % ny + ny) % ny;
-            // (Ex, By) pairs, (Ey, Bx) pairs, Ez, Bz
-            const int dst = c == 0 ? 2 * w : c == 4 ? 2 * w + 1 : c == 1 ? 2 * NW + 2 * w
-                          : c == 3 ? 2 * NW + 2 * w + 1 : c == 2 ? 4 * NW + w : 5 * NW + w;
-            fw[dst] = s == 0 ? 0.f : (float)s * Fg[c * a.ntot + (long long)gy * nx + gx];
-        }
-        for (int idx = threadIdx.x; idx < 6 * NW; idx += blockDim.x) jw[idx] = 0;
         __syncthreads();
         if (threadIdx.x < 2) {
             const int s = threadIdx.x;
@@ -546,19 +539,62 @@ k_push_tile(const MixedArgs a) {
             s_pop = n;
         }
         __syncthreads();
+        // this item's range [lo, hi) of the tile's particles: species 0, padded to whole
+        // chunks, then species 1; the last part takes what is left
+        const int v1 = (s_start[0][kSegs] + 31) & ~31;
+        const int vend = v1 + s_start[1][kSegs];
+        const int lo = part * G.pchunk;
+        const int hi = part == parts - 1 ? vend : min(vend, lo + G.pchunk);
+        if (lo >= hi) continue;  // (uniform over the CTA) nothing to push, no current to add
+        // The window, one node per thread and round: its wrapped (or mirrored) cell once for
+        // all six components, whose loads are all in flight together.
+        const float* Fg = a.F32 + G.cell_off;
+        for (int w = threadIdx.x; w < NW; w += blockDim.x) {
+            const int wy = w / WX, wx = w - wy * WX;
+            const float* R = Fg + (long long)wrap_window(Y0 - 2 + wy, ny) * nx;
+            float ex, ey, ez, bx, by, bz;
+            if (!G.walls) {
+                R += wrap_window(X0 - 2 + wx, nx);
+                ex = R[0];
+                ey = R[a.ntot];
+                ez = R[2 * a.ntot];
+                bx = R[3 * a.ntot];
+                by = R[4 * a.ntot];
+                bz = R[5 * a.ntot];
+            } else {  // conductor images: Ex, By, Bz even, Ey, Ez, Bx odd
+                int sh, si;
+                const float* Rh = R + wall_col(X0 - 2 + wx, nx, true, false, sh);
+                const float* Ri = R + wall_col(X0 - 2 + wx, nx, false, true, si);
+                const float fh = (float)sh, fi = (float)si;
+                ex = fh * Rh[0];
+                by = fh * Rh[4 * a.ntot];
+                bz = fh * Rh[5 * a.ntot];
+                ey = si == 0 ? 0.f : fi * Ri[a.ntot];
+                ez = si == 0 ? 0.f : fi * Ri[2 * a.ntot];
+                bx = si == 0 ? 0.f : fi * Ri[3 * a.ntot];
+            }
+            reinterpret_cast<float2*>(fw)[w] = make_float2(ex, by);
+            reinterpret_cast<float2*>(fw + 2 * NW)[w] = make_float2(ey, bx);
+            fw[4 * NW + w] = ez;
+            fw[5 * NW + w] = bz;
+#pragma unroll
+            for (int c = 0; c < 6; c++) jw[c * NW + w] = 0;
+        }
+        __syncthreads();
         const FixedScale fs = fixed_scale(G, s_pop);
         const WinMem W{fw, jw, jw + 3 * NW, WX, NW, fs.js, fs.jlb};
         const GlobalMem M{a.F32 + G.cell_off, reinterpret_cast<unsigned long long*>(a.Jfix + G.cell_off),
                           a.ntot, nx, ny, fs, fs.js, G.walls};
         const unsigned* cur = par ? a.buf[1] : a.buf[0];
         unsigned* nxt = par ? a.buf[0] : a.buf[1];
+        int* cnxt = (nxp ? a.cnt[1] : a.cnt[0]) + (long long)t * 2 * kSegs;
         float ek = 0.f;
         for (int s = 0; s < 2; s++) {
             const PushConst K = push_const(G, s);
-            const int total = s_start[s][kSegs];
+            const int first = max(lo - (s ? v1 : 0), 0), total = min(hi - (s ? v1 : 0), s_start[s][kSegs]);
             const long long own = G.bin_off + ((long long)lt * 2 + s) * stride;
             const int st1 = s_start[s][1];  // end of the stayer segment
-            for (int c0 = warp * 32; c0 < total; c0 += nwarp * 32) {
+            for (int c0 = first + warp * 32; c0 < total; c0 += nwarp * 32) {
                 const int v = c0 + lane;
                 const bool valid = v < total;
                 int dest = -1, cnew = 0;
@@ -604,7 +640,10 @@ k_push_tile(const MixedArgs a) {
                     const int leader = __ffs(grp) - 1;
                     const int rank = __popc(grp & ((1u << lane) - 1u));
                     int b0 = 0;
-                    if (lane == leader && dest >= 0) b0 = atomicAdd(&s_out[s][dest], __popc(grp));
+                    // slots of the next buffer: the tile's counters, in shared memory while
+                    // one CTA pushes the whole tile
+                    if (lane == leader && dest >= 0)
+                        b0 = atomicAdd(parts == 1 ? &s_out[s][dest] : cnxt + s * kSegs + dest, __popc(grp));
                     b0 = __shfl_sync(grp, b0, leader) + rank;
                     long long slot = -1;
                     if (dest == 0 && b0 < cap) slot = own + b0;
@@ -622,26 +661,23 @@ k_push_tile(const MixedArgs a) {
             }
         }
         __syncthreads();
-        if (threadIdx.x < 2 * kSegs) {
-            const int s = threadIdx.x / kSegs, k = threadIdx.x - (threadIdx.x / kSegs) * kSegs;
-            int* cnxt = nxp ? a.cnt[1] : a.cnt[0];
-            cnxt[((long long)t * 2 + s) * kSegs + k] = s_out[s][k];  // sent, parked ones included
-        }
+        if (parts == 1 && threadIdx.x < 2 * kSegs)
+            cnxt[threadIdx.x] = (&s_out[0][0])[threadIdx.x];  // sent, parked ones included
         // add the current window into the global fixed-point current
         unsigned long long* Jg = reinterpret_cast<unsigned long long*>(a.Jfix + G.cell_off);
-        for (int idx = threadIdx.x; idx < 3 * NW; idx += blockDim.x) {
-            const int hi = jw[idx], lo = jw[3 * NW + idx];
-            if ((hi | lo) == 0) continue;
-            const unsigned long long v = (unsigned long long)fixed_value(hi, lo, fs);
-            const int c = idx / NW;
-            const int w = idx - c * NW;
-            const int wy = w / WX;
-            const int wx = w - wy * WX;
-            int gx = ((X0 - 2 + wx) % nx + nx) % nx, s = 1;
-            if (G.walls) gx = wall_col(X0 - 2 + wx, nx, c == 0, c == 0, s);  // mirror: Jx odd
-            if (s == 0) continue;
-            const int gy = ((Y0 - 2 + wy) % ny + ny) % ny;
-            atomicAdd(Jg + c * a.ntot + (long long)gy * nx + gx, s > 0 ? v : 0ull - v);
+        for (int w = threadIdx.x; w < NW; w += blockDim.x) {
+            const int wy = w / WX, wx = w - wy * WX;
+            unsigned long long* R = Jg + (long long)wrap_window(Y0 - 2 + wy, ny) * nx;
+            const int gx = G.walls ? 0 : wrap_window(X0 - 2 + wx, nx);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const int hi = jw[c * NW + w], lw = jw[(3 + c) * NW + w];
+                if ((hi | lw) == 0) continue;
+                const unsigned long long v = (unsigned long long)fixed_value(hi, lw, fs);
+                int col = gx, sg = 1;
+                if (G.walls) col = wall_col(X0 - 2 + wx, nx, c == 0, c == 0, sg);  // mirror: Jx odd
+                if (sg != 0) atomicAdd(R + c * a.ntot + col, sg > 0 ? v : 0ull - v);
+            }
         }
         const double sum = block_sum((double)ek, s_red);  // begins with a block barrier
         if (threadIdx.x == 0 && sum != 0.0) atomicAdd(&a.cg[g].uk, 0.5 * G.w * sum);
@@ -653,9 +689,27 @@ k_push_tile(const MixedArgs a) {
 // 0. Overflow particles: global-memory push; they stay in the overflow list until the
 // host re-sorts after the pic_step call.
 // ---------------------------------------------------------------------------------
-__global__ void k_mixed_begin(DevStatus* st, int* work) {
+// Start of a step, over the whole device: the deferred stop flag and step counter, the
+// kinetic-energy accumulators and the work counters (block 0); J = 0; the next buffer's
+// count slots and overflow count (a stopped step reads none of them again). One launch in
+// place of four small ones: on small grids a step is made of launches.
+__global__ void __launch_bounds__(256)
+k_mixed_begin(const MixedArgs a, int ngrids, long long nj2, int ncnt, int* work) {
+    DevStatus* st = a.st;
+    const int nxp = (int)(st->parity ^ 1u);
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    longlong2* J = reinterpret_cast<longlong2*>(a.Jfix);  // (allocated with room for whole pairs)
+    for (long long k = t; k < nj2; k += nt) J[k] = make_longlong2(0, 0);
+    int* c = nxp ? a.cnt[1] : a.cnt[0];
+    for (int k = (int)t; k < ncnt; k += (int)nt) c[k] = 0;
+    if (blockIdx.x != 0) return;
     if (threadIdx.x < 4) work[threadIdx.x] = 0;
-    if (threadIdx.x == 0 && !st->stop) st->ovf_count[st->parity ^ 1u] = 0ull;
+    if (threadIdx.x == 0) {
+        if (st->stop_next) st->stop = 1u;
+        if (!st->stop) st->steps_done += 1ull;
+        st->ovf_count[nxp] = 0ull;
+    }
+    for (int g = threadIdx.x; g < ngrids; g += blockDim.x) a.cg[g].uk = 0.0;
 }
 
 template <int P>
@@ -755,8 +809,16 @@ __global__ void k_inject_mixed(const MixedArgs a, const int* inj_grid, const lon
     }
 }
 
-__global__ void k_mixed_swap(DevStatus* st) {
-    if (threadIdx.x == 0 && !st->stop) st->parity ^= 1u;
+// End of a step: the buffers swap; PCG statistics.
+__global__ void k_mixed_end(DevStatus* st, int ngrids, CgState* cg) {
+    if (st->stop) return;
+    if (threadIdx.x == 0) st->parity ^= 1u;
+    for (int g = threadIdx.x; g < ngrids; g += blockDim.x) {
+        CgState& s = cg[g];
+        s.last_iters = s.iters;
+        s.max_iters = s.iters > s.max_iters ? s.iters : s.max_iters;
+        s.total_iters += s.iters;
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1050,8 +1112,8 @@ MixedArgs make_args(MixedState* m, int order) {
     MixedArgs a{};
     a.grids = m->dgrids;
     a.tile_grid = m->tile_grid;
-    a.tlist = m->tlist + m->order_first[order];
-    a.ntl = m->order_n[order];
+    a.items = m->items + m->item_first[order];
+    a.nitems = m->item_n[order];
     a.work = m->work + order;
     a.ntot = m->ntot;
     a.F32 = m->F32;
@@ -1209,6 +1271,59 @@ int gather_species(MixedState* m, int g, int par, int s, PartArrays& S, long lon
     return PIC_OK;
 }
 
+// The tile kernels' work items. An item is a tile, or one of `parts` equal parts of its
+// particles where whole tiles are too few, or too long, to fill the device evenly. Each
+// part stages the field window and adds its own current window, and the parts of a tile
+// take their slots of the next buffer from the tile's counters in global memory. The
+// current is an integer sum and its rounding follows the tile's population, so the result
+// does not depend on the split.
+//
+// The split minimises (rounds + 0.4) (n / parts + 500) [x 1.04 if parts > 1], rounds =
+// tiles x parts / resident CTAs (1 in all where they fit at once): an item costs its n /
+// parts particles and its window, worth about 500 particles (8 us of one CTA, measured
+// from 4 to 8 parts of 2048 x 512 cells); a launch of several rounds ends, on average, in
+// a partly empty one; counters in global memory cost 4%. Measured (tile kernel per step,
+// us, one part / the chosen split / twice it): 128 x 128 cells, 100 per cell 1046 / 158
+// (14) / 171; 64 x 64, 8 per cell 75 / 21 (32) / 21; 1413 x 247, 50 per cell 989 / 971
+// (5) / 978; twelve scan simulations 1347 / 1176 (3) / 1243; 2048 x 512, 32 per cell 2698
+// (1, chosen) / 2666 (2) / 2881 (4).
+int plan_items(MixedState* m, std::string& err) {
+    std::vector<int2> items;
+    for (int P = 1; P <= 3; P++) {
+        m->item_first[P] = (int)items.size();
+        const double tiles = m->order_n[P], resident = std::max(m->resident[P], 1);
+        double mean = 0.0;  // particles per tile that the bins are sized for
+        for (int g = 0; g < m->ngrids; g++)
+            if (m->G[g].order == P) mean += m->G[g].cap * (2.0 / kBinSlack) * m->G[g].ntiles / tiles;
+        double part = mean, best = -1.0;  // particles per item
+        for (int p = 1; p <= 256 && (p == 1 || mean / p >= kTileThreads); p++) {
+            const double rounds = tiles * p / resident;
+            const double cost = (rounds <= 1.0 ? 1.0 : rounds + 0.4) * (mean / p + 500.0) * (p > 1 ? 1.04 : 1.0);
+            if (best < 0.0 || cost < best) {
+                best = cost;
+                part = mean / p;
+            }
+        }
+        for (int g = 0; g < m->ngrids; g++) {
+            GridDev& G = m->G[g];
+            if (G.order != P) continue;
+            const double n = G.cap * (2.0 / kBinSlack);
+            G.parts = (int)std::max(1.0, std::min(256.0, std::floor(n / part + 0.5)));
+            G.pchunk = ((int)std::ceil(n / G.parts) + kTileThreads - 1) / kTileThreads * kTileThreads;
+        }
+        for (int q = m->order_first[P]; q < m->order_first[P] + m->order_n[P]; q++)
+            for (int part = 0; part < m->G[m->host_tile_grid[m->tlist[q]]].parts; part++)
+                items.push_back(make_int2(m->tlist[q], part));
+        m->item_n[P] = (int)items.size() - m->item_first[P];
+        m->pblocks[P] = std::min(m->item_n[P], m->resident[P]);
+    }
+    if (m->items) cudaFree(m->items);
+    m->items = nullptr;
+    MCK(dalloc(&m->items, items.size()));
+    MCK(cudaMemcpy(m->items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    return PIC_OK;
+}
+
 // (Re)allocate both bin buffers with per-simulation stayer capacity cap[g] and outbox
 // capacity capo[g] (contents are not preserved; all counts are zeroed).
 int alloc_bins(MixedState* m, const std::vector<long long>& cap, const std::vector<long long>& capo,
@@ -1227,6 +1342,7 @@ int alloc_bins(MixedState* m, const std::vector<long long>& cap, const std::vect
         off += (long long)G.ntiles * 2 * bin_stride(G);
     }
     m->nslots = off;
+    if (int rc = plan_items(m, err)) return rc;
     for (int p = 0; p < 2; p++) {
         cudaError_t e = dalloc(&m->buf[p], (size_t)m->nslots * kFields);
         if (e != cudaSuccess) {
@@ -1341,14 +1457,15 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         D.wy = D.ty + 5;
         const size_t sm = (size_t)6 * D.wx * D.wy * sizeof(int) + (size_t)6 * D.wx * D.wy * sizeof(float);
         m->smem[D.order] = std::max(m->smem[D.order], sm);
-        const double slack = q.bin_slack > 0 ? q.bin_slack : 1.25;
+        const double slack = q.bin_slack > 0 ? q.bin_slack : kBinSlack;
         cap[g] = round32((double)q.ppc * D.tx * D.ty * slack + 64.0);
         capo[g] = round32((double)q.ppc * std::max(D.tx, D.ty) * 1.5 + 32.0);
         expect += 2ll * q.ppc * (long long)q.nx * q.ny;
     }
     m->ntiles_total = ntiles;
     // per-order tile lists, largest expected work first
-    std::vector<int> tg(ntiles), tl;
+    std::vector<int> tg(ntiles);
+    std::vector<int>& tl = m->tlist;
     std::vector<std::pair<long long, int>> order_tiles[4];
     for (int g = 0; g < ngrids; g++) {
         const GridDev& D = G[g];
@@ -1369,6 +1486,7 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         m->order_n[P] = (int)order_tiles[P].size();
         for (auto& e : order_tiles[P]) tl.push_back(e.second);
     }
+    m->host_tile_grid = tg;
     m->ovf_cap = std::max<long long>(65536, expect / 8);
     m->ovf_cap = (m->ovf_cap + 31) / 32 * 32;
     cudaError_t e = cudaSuccess;
@@ -1402,16 +1520,10 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         }
     }
     if (e == cudaSuccess) e = dalloc(&m->tile_grid, (size_t)ntiles);
-    if (e == cudaSuccess) e = dalloc(&m->tlist, (size_t)ntiles);
     if (e == cudaSuccess) e = dalloc(&m->work, 4);
     if (e == cudaSuccess) e = cudaMemcpy(m->tile_grid, tg.data(), ntiles * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(m->tlist, tl.data(), ntiles * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(m->work, 0, 4 * sizeof(int));
     int rc = PIC_OK;
-    if (e == cudaSuccess) {
-        rc = alloc_bins(m, cap, capo, 0, err);
-        if (rc == PIC_OK) e = cudaDeviceSynchronize();
-    }
     // Shared-memory opt-in: only ever raised, since the attribute belongs to the kernel
     // and other handles in the process may need more than this one.
     int dev = 0, nsm = 152;
@@ -1427,12 +1539,16 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         if (r == cudaSuccess)
             r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kTileThreads, m->smem[P]);
         if (r == cudaSuccess && nb < 1) r = cudaErrorInvalidConfiguration;
-        m->pblocks[P] = std::min(m->order_n[P], nb * nsm);
+        m->resident[P] = nb * nsm;
         return r;
     };
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<1>, 1);
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<2>, 2);
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<3>, 3);
+    if (rc == PIC_OK && e == cudaSuccess) {
+        rc = alloc_bins(m, cap, capo, 0, err);
+        if (rc == PIC_OK) e = cudaDeviceSynchronize();
+    }
     if (rc == PIC_OK && e == cudaSuccess) {
         e = cudaMemcpy((void*)dgrids, G, ngrids * sizeof(GridDev), cudaMemcpyHostToDevice);
     }
@@ -1456,7 +1572,7 @@ void mixed_destroy(MixedState* m) {
         for (void* q : ps)
             if (q) cudaFree(q);
     }
-    void* ps[] = {m->tile_grid, m->tlist, m->work, m->injected, m->inj_grid, m->inj_first};
+    void* ps[] = {m->tile_grid, m->items, m->work, m->injected, m->inj_grid, m->inj_first};
     for (void* q : ps)
         if (q) cudaFree(q);
     delete m;
@@ -1522,7 +1638,10 @@ int mixed_load(MixedState* m, int g, int s, const double* x, const double* y, co
 
 void mixed_enqueue(MixedState* m, cudaStream_t st, int part) {
     if (part == 0) {
-        k_mixed_begin<<<1, 32, 0, st>>>(m->st, m->work);
+        const long long nj2 = (3 * m->ntot + 1) / 2;
+        const int ncnt = m->ntiles_total * (2 * kSegs + 1);
+        const unsigned nb = (unsigned)std::min<long long>(8 * 152, std::max<long long>(1, (nj2 + 255) / 256));
+        k_mixed_begin<<<nb, 256, 0, st>>>(make_args(m, 0), m->ngrids, nj2, ncnt, m->work);
         k_push_overflow<<<152, kTileThreads, 0, st>>>(make_args(m, 0));
     } else if (part == 1) {
         for (int P = 1; P <= 3; P++) {
@@ -1535,18 +1654,19 @@ void mixed_enqueue(MixedState* m, cudaStream_t st, int part) {
             default: k_push_tile<3><<<nb, kTileThreads, m->smem[3], st>>>(a); break;
             }
         }
-    } else {
+    } else if (part == 2) {
         if (m->inject_grids)
             k_inject_mixed<<<(unsigned)((m->inject_threads + 255) / 256), 256, 0, st>>>(
                 make_args(m, 0), m->inj_grid, m->inj_first, m->inject_grids, m->injected);
-        k_mixed_swap<<<1, 32, 0, st>>>(m->st);
+    } else {
+        k_mixed_end<<<1, 128, 0, st>>>(m->st, m->ngrids, m->cg);
     }
 }
 
 int mixed_before_steps(MixedState*, cudaStream_t, std::string&) { return PIC_OK; }
 
 int mixed_step_kernels(const MixedState* m) {
-    int k = 3;  // k_mixed_begin, k_push_overflow, k_mixed_swap
+    int k = 3;  // k_mixed_begin, k_push_overflow, k_mixed_end
     for (int P = 1; P <= 3; P++) k += m->order_n[P] > 0 ? 1 : 0;
     return k + (m->inject_grids ? 1 : 0);
 }

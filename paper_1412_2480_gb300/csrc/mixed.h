@@ -24,14 +24,15 @@ void mixed_destroy(MixedState* m);
 // host or device).
 int mixed_load(MixedState* m, int g, int sp, const double* x, const double* y, const double* ux,
                const double* uy, const double* uz, long long n, cudaStream_t s, std::string& err);
-// Enqueue one part of the particle half of a step (the fixed-point current already
-// zeroed): part 0 = overflow-list push, 1 = tile kernels, 2 = buffer swap.
+// Enqueue one part of a step: part 0 = its start (stop flag, counters, J = 0) and the
+// overflow-list push, 1 = tile kernels, 2 = the injector's pairs, 3 = its end (buffer
+// swap, PCG statistics).
 void mixed_enqueue(MixedState* m, cudaStream_t s, int part);
 // Host bookkeeping around a pic_step call (re-bin when bins overflowed).
 int mixed_before_steps(MixedState* m, cudaStream_t s, std::string& err);
 int mixed_after_steps(MixedState* m, cudaStream_t s, std::string& err);
 
-// Kernels mixed_enqueue launches per step (all three parts together).
+// Kernels mixed_enqueue launches per step (all parts together).
 int mixed_step_kernels(const MixedState* m);
 long long mixed_count(MixedState* m, int g, int sp);
 // Add simulation g's node density into rho (device, ncell values; may be null), each
