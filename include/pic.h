@@ -341,7 +341,7 @@ PIC_API int pic_particles(pic_sim* s, int32_t species, double* out5xn, int64_t n
  * The library cannot see the lengths of F, J and dB: they must hold at least the counts
  * above (the Python binding checks them). Returns PIC_OK, PIC_EINVAL (sizes beyond the
  * maximum, bad parameters, or a pointer that is not memory of the current device),
- * PIC_ECUDA, or PIC_ECG_NOCONV.
+ * PIC_ECUDA, PIC_ECG_NOCONV, or PIC_ETIMEOUT (a grid-wide wait of the solve ran out).
  *
  * The first call on a device does a one-time set-up on that device (it looks up the
  * device address of the scratch array); make that first call before any stream capture

@@ -49,6 +49,7 @@ struct pic_sim {
     bool quads = false;  // every simulation's nx is a multiple of 4
     double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
     double* part = nullptr;
+    double* cg_part = nullptr;  // FP64: the PCG's partial sums
     CgState* cg = nullptr;
     unsigned int* done = nullptr;
     DevStatus* st = nullptr;
@@ -222,7 +223,13 @@ void fill_grid(const pic_params& p, GridDev& G) {
         G.pk_fx[s] = (float)(G.qw[s] * G.dx / (G.dt * area));
         G.pk_fy[s] = (float)(G.qw[s] * G.dy / (G.dt * area));
         G.pk_fz[s] = (float)(G.qw[s] / area);
+        G.p64_h[s] = 0.5 * G.qm[s] * G.dt;
+        G.p64_fx[s] = G.qw[s] * G.dx / (G.dt * area);
+        G.p64_fy[s] = G.qw[s] * G.dy / (G.dt * area);
+        G.p64_fz[s] = G.qw[s] / area;
     }
+    G.p64_dtx = G.dt * G.idx;
+    G.p64_dty = G.dt * G.idy;
     G.pk_dtx = (float)(G.dt * G.idx);
     G.pk_dty = (float)(G.dt * G.idy);
     G.js40 = (float)(G.jscale * std::ldexp(1.0, -40));
@@ -280,6 +287,7 @@ FieldArgs field_args(pic_sim* s, int use_cond, cudaGraphConditionalHandle cond) 
     a.q = s->q;
     a.cg = s->cg;
     a.part = s->part;
+    a.cg_part = s->cg_part;
     a.done = s->done;
     a.st = s->st;
     a.cond = cond;
@@ -431,9 +439,10 @@ cudaError_t add_while(cudaStream_t st, cudaGraphConditionalHandle h, cudaStream_
     return e;
 }
 
-// Capture the parts in `mask` (in order) into one graph. The field-solve part becomes
-// rhs -> WHILE(any simulation active){PCG iteration} -> E/B update, the WHILE condition
-// being set on the device by the rhs and PCG kernels.
+// Capture the parts in `mask` (in order) into one graph. The field-solve part is rhs ->
+// one cooperative solve kernel -> E/B update, or, for MIXED32 handles without it, rhs ->
+// WHILE(any simulation active){refinement} -> E/B update, the WHILE condition being set
+// on the device by the rhs and PCG kernels.
 int capture(pic_sim* s, int mask, cudaGraph_t* gout, cudaGraphExec_t* xout) {
     cudaStream_t st = s->stream;
     CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
@@ -446,6 +455,13 @@ int capture(pic_sim* s, int mask, cudaGraph_t* gout, cudaGraphExec_t* xout) {
         }
         if (s->prm.flags & PIC_EXPLICIT) {
             launch_explicit_fields(field_args(s, 0, 0), st);
+            launch_nodal(field_args(s, 0, 0), st);
+            continue;
+        }
+        if (s->prm.precision == PIC_FP64) {  // rhs -> one cooperative kernel for the whole PCG -> update
+            launch_rhs(field_args(s, 0, 0), st);
+            e = launch_cg(field_args(s, 0, 0), s->hgrids[0].ncell, s->device, st);
+            if (e == cudaSuccess) launch_field_update(field_args(s, 0, 0), st);
             launch_nodal(field_args(s, 0, 0), st);
             continue;
         }
@@ -471,10 +487,7 @@ int capture(pic_sim* s, int mask, cudaGraph_t* gout, cudaGraphExec_t* xout) {
             launch_learned_guess(s->guess, s->dgrids, s->cg, s->ntot, s->bvec, nullptr, s->x, nullptr, st);
             launch_guess_residual(field_args(s, 1, h), st);
         }
-        if (e == cudaSuccess && s->prm.precision == PIC_FP64) {
-            e = add_while(st, h, s->body_stream,
-                          [&](cudaStream_t bs) { launch_cg_iteration(field_args(s, 1, h), bs); return cudaSuccess; });
-        } else if (e == cudaSuccess) {
+        if (e == cudaSuccess) {
             // mixed precision: WHILE(outer) { inner begin; WHILE(inner) { FP32 iteration };
             // x += e, r = b - A x }
             e = add_while(st, h, s->body_stream, [&](cudaStream_t bs) {
@@ -549,7 +562,7 @@ long long step_kernels(pic_sim* s, bool graph) {
         k += s->hgrids[0].inject ? 1 : 0;
     }
     if (s->learned) k += 2;  // k_guess, k_guess_residual
-    if (s->use_coop) k += 1;
+    if (s->use_coop || (s->prm.precision == PIC_FP64 && !(s->prm.flags & PIC_EXPLICIT))) k += 1;
     if (s->any_nodal) k += 1;  // k_nodal
     return k;
 }
@@ -557,11 +570,11 @@ long long step_kernels(pic_sim* s, bool graph) {
 // Kernels the PCG loop launched for the given loop-counter increments (none with the
 // cooperative solve: its iterations run inside one launch).
 long long loop_kernels(const pic_sim* s, unsigned long long d_iters, unsigned long long d_refine) {
-    if (s->use_coop) return 0;
-    return 2 * (long long)d_iters + (s->prm.precision == PIC_MIXED32 ? 3 * (long long)d_refine : 0);
+    if (s->use_coop || s->prm.precision == PIC_FP64) return 0;
+    return 2 * (long long)d_iters + 3 * (long long)d_refine;
 }
 
-// Direct launches (PIC_NO_GRAPH): the PCG loop is driven from the host.
+// Direct launches (PIC_NO_GRAPH): the MIXED32 PCG loop is driven from the host.
 int run_step_direct(pic_sim* s) {
     cudaStream_t st = s->stream;
     enqueue_part(s, kPartPre, st);
@@ -585,8 +598,8 @@ int run_step_direct(pic_sim* s) {
             launch_guess_residual(a, st);
         }
     }
-    if (s->use_coop) {
-        CK(launch_mp_coop(s->coop, a, st));
+    if (s->use_coop || s->prm.precision == PIC_FP64) {
+        CK(s->use_coop ? launch_mp_coop(s->coop, a, st) : launch_cg(a, s->hgrids[0].ncell, s->device, st));
         launch_field_update(a, st);
         launch_nodal(a, st);
         enqueue_part(s, kPartEnd, st);
@@ -597,19 +610,15 @@ int run_step_direct(pic_sim* s) {
     CK(cudaMemcpyAsync(&nact, &s->st->n_active, sizeof nact, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     while (nact > 0) {
-        if (s->prm.precision == PIC_FP64) {
-            launch_cg_iteration(a, st);
-        } else {
-            launch_mp_inner_begin(a, st);
+        launch_mp_inner_begin(a, st);
+        CK(cudaMemcpyAsync(&nin, &s->st->n_in_active, sizeof nin, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        while (nin > 0) {
+            launch_mp_inner_iteration(a, st);
             CK(cudaMemcpyAsync(&nin, &s->st->n_in_active, sizeof nin, cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
-            while (nin > 0) {
-                launch_mp_inner_iteration(a, st);
-                CK(cudaMemcpyAsync(&nin, &s->st->n_in_active, sizeof nin, cudaMemcpyDeviceToHost, st));
-                CK(cudaStreamSynchronize(st));
-            }
-            launch_mp_refine(a, st);
         }
+        launch_mp_refine(a, st);
         CK(cudaMemcpyAsync(&nact, &s->st->n_active, sizeof nact, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
     }
@@ -696,6 +705,15 @@ int charge_density(pic_sim* s, double* rho, double* mom = nullptr, int which = P
     }
     CK(cudaGetLastError());
     return PIC_OK;
+}
+
+// Whether p is memory of the handle's device that its kernels can write.
+bool on_device(const pic_sim* s, const void* p) {
+    cudaPointerAttributes at{};
+    const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                    at.device == s->device;
+    cudaGetLastError();
+    return ok;
 }
 
 int check_species(pic_sim* s, int sp) {
@@ -843,6 +861,7 @@ int init_handle(const pic_params* prm, int n, pic_sim** out) {
     A(dalloc(&s->dsegs, 2));
     if (prm[0].precision == PIC_FP64) {
         A(dalloc(&s->J64, n3));
+        A(dalloc(&s->cg_part, kCgPartials));
     } else {
         A(dalloc(&s->Jfix, n3 + 1));  // whole pairs of words (k_mixed_begin)
         A(dalloc(&s->bvec, n3));
@@ -1435,15 +1454,23 @@ int pic_particles(pic_sim* s, int32_t sp, double* out, int64_t n) {
         return rc;
     }
     const GridDev& G = s->hgrids[0];
+    // positions in physical units: straight into a caller's array on this device, else
+    // through a temporary of the library's pool
     double* t = nullptr;
-    CK(dalloc(&t, 2 * (size_t)n));
-    k_unload_fp64<<<(unsigned)((n + 255) / 256), 256, 0, s->stream>>>(n, s->pa[sp][0], s->pa[sp][1],
-                                                                      G.dx, G.dy, t, t + n);
-    cudaError_t e = cudaMemcpyAsync(out, t, 2 * n * sizeof(double), cudaMemcpyDefault, s->stream);
+    cudaError_t e = cudaSuccess;
+    const bool direct = on_device(s, out);
+    if (!direct) e = temp_alloc((void**)&t, 2 * (size_t)n * sizeof(double), s->stream);
+    double* pos = direct ? out : t;
+    if (e == cudaSuccess) {
+        k_unload_fp64<<<(unsigned)((n + 255) / 256), 256, 0, s->stream>>>(n, s->pa[sp][0], s->pa[sp][1], G.dx, G.dy,
+                                                                          pos, pos + n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(out, t, 2 * n * sizeof(double), cudaMemcpyDefault, s->stream);
     for (int a = 2; a < 5 && e == cudaSuccess; a++)
         e = cudaMemcpyAsync(out + a * n, s->pa[sp][a], n * sizeof(double), cudaMemcpyDefault, s->stream);
+    temp_free(t, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    cudaFree(t);
     if (e != cudaSuccess) return fail(s, PIC_ECUDA, std::string("pic_particles: ") + cudaGetErrorString(e));
     return PIC_OK;
 }
@@ -1634,7 +1661,7 @@ void pic_free(pic_sim* s) {
     cnn_free_guess(&s->guess);
     coop_free(&s->coop);
     void* ptrs[] = {s->dgrids, s->dblk_grid, s->F, s->J64, s->Jfix, s->F32, s->Fn, s->x, s->r, s->p, s->q,
-                    s->part, s->cg, s->done, s->st, s->tmp, s->dsegs, s->dblk_seg[0], s->dblk_seg[1],
+                    s->part, s->cg_part, s->cg, s->done, s->st, s->tmp, s->dsegs, s->dblk_seg[0], s->dblk_seg[1],
                     s->bvec, s->r32, s->p32, s->q32, s->e32, s->r32b, s->z32};
     for (void* p : ptrs) dfree(p);
     for (int sp = 0; sp < 2; sp++)

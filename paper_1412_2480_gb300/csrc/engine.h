@@ -9,6 +9,11 @@
 
 namespace pic {
 
+// Blocks of the FP64 PCG's cooperative kernel at most, and its partial sums (two sets, then
+// its arrival counter).
+constexpr int kCgMaxBlocks = 640;
+constexpr int kCgPartials = 2 * kCgMaxBlocks + 1;
+
 // Device buffers and launch geometry of the grid (field-solve) kernels.
 struct FieldArgs {
     const GridDev* grids;   // [ngrids]
@@ -27,6 +32,7 @@ struct FieldArgs {
     double *x, *r, *p, *q;  // 3 * ntot each: dB (solution), residual, direction, A p
     CgState* cg;            // [ngrids]
     double* part;           // 4 * nblk block partials
+    double* cg_part;        // kCgPartials, partial sums and counter of the FP64 PCG, or nullptr
     unsigned int* done;     // [ngrids] block-completion counters
     DevStatus* st;
     cudaGraphConditionalHandle cond;  // WHILE-node handle of the PCG loop
@@ -54,8 +60,9 @@ void launch_guess_residual(const FieldArgs& a, cudaStream_t s);
 // The same in FP32 for the cooperative solve, from the guess's FP32 copy in a.e32 into
 // a.r32 (which holds the FP32 copy of b): the first inner solve needs no more.
 void launch_guess_residual32(const FieldArgs& a, cudaStream_t s);
-// One PCG iteration: A-product and direction update, then solution/residual update.
-void launch_cg_iteration(const FieldArgs& a, cudaStream_t s);
+// The FP64 PCG after launch_rhs, for the one simulation (of ncell cells) that a.grids
+// holds, on device `dev`: one cooperative kernel, nothing allocated.
+cudaError_t launch_cg(const FieldArgs& a, int ncell, int dev, cudaStream_t s);
 // E, B from Eqs. (5)-(6) with dB; FP32 copies when a.F32 is set.
 void launch_field_update(const FieldArgs& a, cudaStream_t s);
 // Explicit FDTD field step, Eqs. (3)-(4) (PIC_EXPLICIT): three kernels, no solve.

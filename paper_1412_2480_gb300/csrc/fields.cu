@@ -5,11 +5,15 @@
 // One thread per cell handles the three components of every vector. Reductions use
 // per-block partials and a "last block finishes" step per simulation (fixed summation
 // order, so results do not depend on block scheduling); the last simulation to finish
-// sets the WHILE condition of the captured PCG loop, so the loop runs exactly as many
-// iterations as the slowest simulation needs, with no host round trip.
+// sets the WHILE condition of the captured MIXED32 PCG loop, so the loop runs exactly as
+// many iterations as the slowest simulation needs, with no host round trip. The FP64 PCG
+// is one cooperative kernel.
 //
 // Staggering (Sec. 2, Fig. 1; index k = j*nx + i): Ez at (i,j); Ex, By at (i+1/2,j);
 // Ey, Bx at (i,j+1/2); Bz at (i+1/2,j+1/2). J shares the E lattices.
+#include <algorithm>
+#include <mutex>
+
 #include "dword.cuh"
 #include "engine.h"
 
@@ -87,34 +91,54 @@ __device__ __forceinline__ double dld(const T* p, long long k1, long long k2, do
     else return (p[k1] - p[k2]) * s;
 }
 
+// Simulation-wide sums of its blocks' partials, in every thread of the finishing block:
+// warp a sums value a, the four chains of a lane in parallel.
+template <int NV>
+__device__ __forceinline__ void finish_sums(const GridDev& G, const double* part, int nblk_total, double tot[NV]) {
+    __shared__ double s_tot[NV];
+    if (threadIdx.x < 32 * NV) {
+        const int lane = threadIdx.x & 31;
+        const double* p = part + (threadIdx.x >> 5) * nblk_total + G.blk_first;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = lane; b < G.nblk; b += 128)
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (b + 32 * u < G.nblk) acc[u] += __ldcg(p + b + 32 * u);
+        const double s = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+        if (lane == 0) s_tot[threadIdx.x >> 5] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < NV; a++) tot[a] = s_tot[a];
+}
+
 // Sum `nv` values per thread over the block, store them as this block's partials, and
 // return true in every thread of the block that completes its simulation last. The
 // finishing block then holds the simulation-wide sums in `tot`.
 template <int NV>
 __device__ bool reduce_and_finish(const GridDev& G, int g, double v[NV], double* part,
                                   int nblk_total, unsigned int* done, double tot[NV]) {
-    __shared__ double scratch[32];
+    __shared__ double s_v[NV][kFieldThreads];
     __shared__ bool last;
 #pragma unroll
-    for (int a = 0; a < NV; a++) {
-        const double s = block_sum(v[a], scratch);
-        if (threadIdx.x == 0) part[a * nblk_total + blockIdx.x] = s;
+    for (int a = 0; a < NV; a++) s_v[a][threadIdx.x] = v[a];
+    __syncthreads();
+    if (threadIdx.x < 32 * NV) {  // warp a sums value a
+        const double s = warp_of_block_sum(s_v[threadIdx.x >> 5]);
+        if ((threadIdx.x & 31) == 0) {
+            part[(threadIdx.x >> 5) * nblk_total + blockIdx.x] = s;
+            __threadfence();
+        }
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         const unsigned t = atomicAdd(&done[g], 1u);
         last = (t == (unsigned)G.nblk - 1u);
     }
     __syncthreads();
     if (!last) return false;
     __threadfence();
-#pragma unroll
-    for (int a = 0; a < NV; a++) {
-        double acc = 0.0;
-        for (int b = threadIdx.x; b < G.nblk; b += blockDim.x)
-            acc += __ldcg(&part[a * nblk_total + G.blk_first + b]);
-        tot[a] = block_sum(acc, scratch);
-    }
+    finish_sums<NV>(G, part, nblk_total, tot);
     if (threadIdx.x == 0) done[g] = 0u;
     return true;
 }
@@ -252,7 +276,6 @@ template <int NV>
 __device__ bool reduce_and_finish_dw(const GridDev& G, int g, DW v[NV], double* part, int nblk_total,
                                      unsigned int* done, double tot[NV]) {
     __shared__ DW wsum[NV][32];
-    __shared__ double scratch[32];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -276,13 +299,7 @@ __device__ bool reduce_and_finish_dw(const GridDev& G, int g, DW v[NV], double* 
     __syncthreads();
     if (!last) return false;
     __threadfence();
-#pragma unroll
-    for (int a = 0; a < NV; a++) {
-        double acc = 0.0;
-        for (int b = threadIdx.x; b < G.nblk; b += blockDim.x)
-            acc += __ldcg(&part[a * nblk_total + G.blk_first + b]);
-        tot[a] = block_sum(acc, scratch);
-    }
+    finish_sums<NV>(G, part, nblk_total, tot);
     if (threadIdx.x == 0) done[g] = 0u;
     return true;
 }
@@ -385,13 +402,15 @@ k_rhs_dw(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, in
     finish_all_grids(ngrids, ngrids, cg, st, cond, use_cond);
 }
 
-// Zero the solution where the warm start is off (x0 = 0), for the FP64 path. Separate
-// from k_rhs because k_rhs reads x at neighbours when warm starting.
+// Zero the solution where the warm start is off (x0 = 0) and the solve's arrival counter,
+// for the FP64 path. Separate from k_rhs because k_rhs reads x at neighbours when warm
+// starting.
 __global__ void __launch_bounds__(kFieldThreads)
 k_zero_x(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, long long ntot,
-         double* __restrict__ x) {
+         double* __restrict__ x, unsigned int* __restrict__ count) {
     const int g = blk_grid[blockIdx.x];
     const GridDev& G = grids[g];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0u;
     if (G.warm == 1) return;
     FOR_CELLS(G, g, c) {
         x[c.k] = 0.0;
@@ -400,87 +419,210 @@ k_zero_x(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, lo
     }
 }
 
-// ---- PCG iteration, part 1 ------------------------------------------------------
-// With the Jacobi preconditioner of a constant-coefficient operator (diagonal c0), the
-// preconditioned iterates equal plain CG's, so z = r is used. The A-product of the new
-// direction p = r + beta p_old is formed as A r + beta (A p_old): A is linear, so this
-// equals A p while touching only r at neighbours.
-__global__ void __launch_bounds__(kFieldThreads)
-k_cg_direction(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids,
-               int nblk_total, long long ntot, const double* __restrict__ r,
-               double* __restrict__ p, double* __restrict__ q, CgState* cg, double* part,
-               unsigned int* done) {
-    const int g = blk_grid[blockIdx.x];
-    if (!cg[g].active) return;
-    const GridDev& G = grids[g];
-    const double beta = cg[g].beta;
-    double v[1] = {0.0};
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot;
-            const double* R = r + o;
-            const double rc = R[c.k];
-            const double Ar = G.c0 * rc - G.cx * nbx(R, c, a) - G.cy * (R[c.kn] + R[c.ks]);
-            double pn, qn;
-            if (beta == 0.0) {
-                pn = rc;
-                qn = Ar;
-            } else {
-                pn = rc + beta * p[o + c.k];
-                qn = Ar + beta * q[o + c.k];
+// ---- FP64 PCG -----------------------------------------------------------------------
+// The whole CG of one simulation as one cooperative kernel. With the Jacobi preconditioner
+// of a constant-coefficient operator (diagonal c0), the preconditioned iterates equal
+// plain CG's, so z = r is used. The A-product of the new direction p = r + beta p_old is
+// formed as A r + beta (A p_old): A is linear, so this equals A p while touching only r at
+// neighbours. Per iteration:
+//   q = A r + beta q, p = r + beta p, (p, q) -> alpha;  x += alpha p, r -= alpha q,
+//   (r, r) -> beta and the test ||r|| <= rtol ||b||.
+// What bounds it on a small grid is the latency of the two grid-wide sums of an iteration
+// (grid_sum below), and on a large one the FP64 pipe (33 operations per cell and
+// iteration). Up to two cells per thread, p, q, x and the own r stay in registers (C = 1, 2)
+// and only r goes through L2 for the neighbours; larger grids keep the vectors in memory
+// (C = 0). As two kernels per iteration in a WHILE node an iteration took 30 us on 32768
+// cells (18 us of it in the kernels), 31 us with host-driven launches on 65536; now 9.3 and 11.5.
+
+// Sum of v over all threads of the grid, the same bits in every block, and a grid-wide
+// barrier: writes before it are visible to loads (of L2) after it. Every block leaves its
+// partial sum, adds one to a counter that only grows, and when the counter says that all
+// have, one warp of each block adds the partials in a fixed order. It leaves the sum S and
+// the quotient S / scale (inv: scale / S) in out[0..1] (shared memory): a division repeated
+// by every thread costs as much here as the rest of an iteration. The partials alternate
+// between two sets, as a block can be at most one sum ahead of another. (Slots that carry
+// the epoch, read by all blocks instead of a counter, took 5.7 us on 152 blocks, their
+// polls in each other's way; the counter's barrier alone takes 1.3 us.)
+// false: the others did not arrive within `limit` polls.
+__device__ bool grid_sum(double v, double scale, bool inv, double out[2], double* part, unsigned int* count,
+                         unsigned int epoch, unsigned int limit, unsigned int* timeout) {
+    __shared__ double s_part[kFieldThreads];
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, lane = tid & 31;
+    double* set = part + (epoch & 1u) * kCgMaxBlocks;
+    s_part[tid] = v;
+    __syncthreads();
+    if (tid < 32) {
+        const double b = warp_of_block_sum(s_part);
+        int ok = 1;
+        if (lane == 0) {
+            set[blockIdx.x] = b;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+            unsigned int seen;
+            for (unsigned int it = 0;;) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+                if (seen >= epoch * gridDim.x) break;
+                if (++it > limit) {
+                    ok = 0;
+                    atomicExch(timeout, 1u);
+                    break;
+                }
             }
-            p[o + c.k] = pn;
-            q[o + c.k] = qn;
-            v[0] += pn * qn;
+            s_ok = ok;
+        }
+        __syncwarp();
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        for (unsigned int k = lane; k < gridDim.x; k += 128)
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if (k + 32 * u < gridDim.x) t[u] += __ldcg(set + k + 32 * u);
+        const double sum = warp_sum((t[0] + t[1]) + (t[2] + t[3]));
+        const double quo = inv ? scale / sum : sum / scale;
+        if (lane == 0) {
+            out[0] = sum;
+            out[1] = quo;
         }
     }
-    double tot[1];
-    if (!reduce_and_finish<1>(G, g, v, part, nblk_total, done, tot)) return;
-    if (threadIdx.x == 0) cg[g].alpha = cg[g].rr / tot[0];
+    __syncthreads();
+    return s_ok != 0;
 }
 
-// ---- PCG iteration, part 2 ------------------------------------------------------
-// x += alpha p; r -= alpha A p; convergence test ||r|| <= rtol ||b||.
-__global__ void __launch_bounds__(kFieldThreads)
-k_cg_update(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids,
-            int nblk_total, long long ntot, double* __restrict__ x, double* __restrict__ r,
-            const double* __restrict__ p, const double* __restrict__ q, CgState* cg,
-            double* part, unsigned int* done, DevStatus* st, cudaGraphConditionalHandle cond,
-            int use_cond) {
-    const int g = blk_grid[blockIdx.x];
-    const unsigned n_part = st->n_active;  // simulations iterating in this launch
-    if (!cg[g].active) return;
-    const GridDev& G = grids[g];
-    const double alpha = cg[g].alpha;
-    double v[1] = {0.0};
-    FOR_CELLS(G, g, c) {
+// Neighbour sums as nbx() forms them, from L2 (other blocks write r during the solve).
+__device__ __forceinline__ double nbx_cg(const double* V, const Cell& c, int a, double vc) {
+    if (a == 0) return (c.ew ? 0.0 : __ldcg(V + c.ke)) + (c.ww ? -__ldcg(V + c.k + 1) : __ldcg(V + c.kw));
+    return (c.ew ? vc : __ldcg(V + c.ke)) + (c.ww ? vc : __ldcg(V + c.kw));
+}
+
+template <int C>
+__global__ void __launch_bounds__(kFieldThreads, C == 2 ? 2 : 3)
+k_cg_coop(const GridDev* __restrict__ grids, long long ntot, double* __restrict__ x, double* r, double* __restrict__ p,
+          double* __restrict__ q, CgState* cg, double* part, unsigned int* count, DevStatus* st, int per) {
+    // (the same in every block: block 0 writes the state only after the last grid_sum)
+    if (!cg->active) return;
+    const GridDev& G = grids[0];
+    const double c0 = G.c0, cx = G.cx, cy = G.cy, rtol = G.rtol, bb = cg->bb;
+    const int maxit = G.maxit, ncell = G.ncell;
+    const unsigned int limit = st->spin_limit ? st->spin_limit : (1u << 22);
+    __shared__ double s_pq[2], s_rr[2];  // (p, q), alpha; (r, r), beta
+    const double rr0 = cg->rr;
+    const double near_bb = rtol * rtol * bb * (1.0 + 1e-12);
+    double alpha = 0.0, beta = 0.0;
+    constexpr int N = C > 0 ? C : 1;
+    // this block's cells: `per` of them (C > 0), or every gridDim-th row of threads
+    const int first = (int)(blockIdx.x * (C > 0 ? per : kFieldThreads) + threadIdx.x);
+    const int stride = C > 0 ? kFieldThreads : (int)(gridDim.x * kFieldThreads);
+    const int last = C > 0 ? min(ncell, (int)(blockIdx.x + 1) * per) : ncell;
+    double rv[N][3], pv[N][3], qv[N][3], xv[N][3];
+    if constexpr (C > 0) {
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot + c.k;
-            x[o] += alpha * p[o];
-            const double rn = r[o] - alpha * q[o];
-            r[o] = rn;
-            v[0] += rn * rn;
-        }
+        for (int n = 0; n < N; n++)
+            if (first + n * stride < last) {
+                const long long k = G.cell_off + first + n * stride;
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    rv[n][a] = __ldcg(r + a * ntot + k);
+                    xv[n][a] = x[a * ntot + k];
+                }
+            }
     }
-    double tot[1];
-    if (!reduce_and_finish<1>(G, g, v, part, nblk_total, done, tot)) return;
-    if (threadIdx.x == 0) {
-        CgState& s = cg[g];
-        s.beta = tot[0] / s.rr;
-        s.rr = tot[0];
-        s.iters += 1;
-        s.rel = sqrt(tot[0] / s.bb);
-        if (s.rel <= G.rtol) {
-            s.active = 0;
-        } else if (s.iters >= G.maxit) {
-            s.active = 0;
-            atomicAdd(&st->cg_noconv, 1u);
-            st->stop_next = 1u;
+    unsigned int epoch = 0;
+    int iters = 0, conv = 0;
+    bool ok = true;
+    for (;;) {
+        double acc = 0.0;
+        // direction of one component at a cell: rc in, p and q updated
+        const auto dir = [&](const Cell& c, int a, double rc, double& pn, double& qn) {
+            const double* R = r + a * ntot;
+            const double Ar = c0 * rc - cx * nbx_cg(R, c, a, rc) - cy * (__ldcg(R + c.kn) + __ldcg(R + c.ks));
+            pn = iters == 0 ? rc : rc + beta * pn;  // (p and q of the last solve are not used)
+            qn = iters == 0 ? Ar : Ar + beta * qn;
+            acc += pn * qn;
+        };
+        if constexpr (C > 0) {
+#pragma unroll
+            for (int n = 0; n < N; n++)
+                if (first + n * stride < last) {
+                    const Cell c = cell_at(G, 0, first + n * stride);
+#pragma unroll
+                    for (int a = 0; a < 3; a++) dir(c, a, rv[n][a], pv[n][a], qv[n][a]);
+                }
+        } else {
+            for (int l = first; l < last; l += stride) {
+                const Cell c = cell_at(G, 0, l);
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const long long o = a * ntot + c.k;
+                    double pn = 0.0, qn = 0.0;
+                    if (iters > 0) {
+                        pn = p[o];
+                        qn = q[o];
+                    }
+                    dir(c, a, __ldcg(r + o), pn, qn);
+                    p[o] = pn;
+                    q[o] = qn;
+                }
+            }
         }
+        const double rr = iters == 0 ? rr0 : s_rr[0];
+        if (!(ok = grid_sum(acc, rr, true, s_pq, part, count, ++epoch, limit, &st->sync_timeout))) break;
+        alpha = s_pq[1];  // (r, r) / (p, q)
+        acc = 0.0;
+        if constexpr (C > 0) {
+#pragma unroll
+            for (int n = 0; n < N; n++)
+                if (first + n * stride < last) {
+                    const long long k = G.cell_off + first + n * stride;
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        xv[n][a] += alpha * pv[n][a];
+                        rv[n][a] -= alpha * qv[n][a];
+                        r[a * ntot + k] = rv[n][a];
+                        acc += rv[n][a] * rv[n][a];
+                    }
+                }
+        } else {
+            for (int l = first; l < last; l += stride) {
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    const long long o = a * ntot + G.cell_off + l;
+                    x[o] += alpha * p[o];
+                    const double rn = __ldcg(r + o) - alpha * q[o];
+                    r[o] = rn;
+                    acc += rn * rn;
+                }
+            }
+        }
+        if (!(ok = grid_sum(acc, rr, false, s_rr, part, count, ++epoch, limit, &st->sync_timeout))) break;
+        beta = s_rr[1];
+        iters += 1;
+        // ||r|| <= rtol ||b||: on the squares, and in the last bits as the quotient's root says
+        conv = s_rr[0] <= near_bb;
+        if (conv) conv = sqrt(s_rr[0] / bb) <= rtol;
+        if (conv || iters >= maxit) break;
     }
-    finish_all_grids(ngrids, (int)n_part, cg, st, cond, use_cond, 0);
+    if constexpr (C > 0) {
+#pragma unroll
+        for (int n = 0; n < N; n++)
+            if (first + n * stride < last) {
+                const long long k = G.cell_off + first + n * stride;
+#pragma unroll
+                for (int a = 0; a < 3; a++) x[a * ntot + k] = xv[n][a];
+            }
+    }
+    if (threadIdx.x != 0) return;
+    if (!ok) st->stop_next = 1u;
+    if (blockIdx.x != 0 || !ok) return;
+    cg->rr = s_rr[0];
+    cg->beta = beta;
+    cg->rel = sqrt(s_rr[0] / bb);
+    cg->iters = iters;
+    cg->active = 0;
+    st->n_active = 0;
+    st->loop_iters[0] += (unsigned long long)iters;
+    if (!conv) {
+        st->cg_noconv += 1u;
+        st->stop_next = 1u;
+    }
 }
 
 // ---- Field update, Eqs. (5)-(6) --------------------------------------------------
@@ -1145,7 +1287,9 @@ void launch_step_end(const FieldArgs& a, cudaStream_t s) {
 }
 
 void launch_rhs(const FieldArgs& a, cudaStream_t s) {
-    if (!a.Jfix) k_zero_x<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.x);  // (k_rhs_dw zeroes x itself)
+    if (!a.Jfix)  // (k_rhs_dw zeroes x itself)
+        k_zero_x<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.x,
+                                                   reinterpret_cast<unsigned int*>(a.cg_part + 2 * kCgMaxBlocks));
     if (a.Jfix)
         k_rhs_dw<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk, a.ntot, a.F, a.Jfix, a.x,
                                                   a.coop ? nullptr : a.r, a.cg, a.part, a.done, a.st, a.cond,
@@ -1190,12 +1334,62 @@ void launch_explicit_fields(const FieldArgs& a, cudaStream_t s) {
     k_explicit_B<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.F, a.x, a.st, a.F32);
 }
 
-void launch_cg_iteration(const FieldArgs& a, cudaStream_t s) {
-    k_cg_direction<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk,
-                                                    a.ntot, a.r, a.p, a.q, a.cg, a.part, a.done);
-    k_cg_update<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk, a.ntot,
-                                                 a.x, a.r, a.p, a.q, a.cg, a.part, a.done, a.st,
-                                                 a.cond, a.use_cond);
+namespace {
+// SMs of device `dev` (out[3]) and blocks of each form of k_cg_coop it holds at once.
+cudaError_t cg_resident(int dev, int out[4]) {
+    static std::mutex mu;
+    static int known[64][4] = {};
+    std::lock_guard<std::mutex> lk(mu);
+    cudaError_t e = dev >= 0 && dev < 64 ? cudaSuccess : cudaErrorInvalidDevice;
+    if (e == cudaSuccess && known[dev][0] == 0) {
+        int nsm = 0, occ[3] = {0, 0, 0};
+        e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], k_cg_coop<0>, kFieldThreads, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], k_cg_coop<1>, kFieldThreads, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[2], k_cg_coop<2>, kFieldThreads, 0);
+        if (e == cudaSuccess) {
+            for (int c = 0; c < 3; c++) known[dev][c] = std::min(std::max(occ[c], 1) * nsm, kCgMaxBlocks);
+            known[dev][3] = nsm;
+        }
+    }
+    if (e == cudaSuccess)
+        for (int c = 0; c < 4; c++) out[c] = known[dev][c];
+    return e;
+}
+}  // namespace
+
+cudaError_t launch_cg(const FieldArgs& a, int ncell, int dev, cudaStream_t s) {
+    int res[4];
+    cudaError_t e = cg_resident(dev, res);
+    if (e != cudaSuccess) return e;
+    // one cell per thread while the device holds that many threads, then two, then memory;
+    // the cells spread evenly over a whole number of blocks per SM (256 x 256: 224 cells in
+    // each of 293 blocks rather than two full blocks on 104 SMs and one on the others)
+    int form = 0, per = kFieldThreads, nb = std::min((ncell + per - 1) / per, res[0]);
+    for (int c = 1; c <= 2 && !form; c++) {
+        if ((long long)ncell > (long long)res[c] * kFieldThreads * c) continue;
+        form = c;
+        const int rounds = (int)((ncell + (long long)res[3] * kFieldThreads * c - 1) / ((long long)res[3] * kFieldThreads * c));
+        per = std::min(((ncell + rounds * res[3] - 1) / (rounds * res[3]) + 31) / 32 * 32, kFieldThreads * c);
+        nb = (ncell + per - 1) / per;
+        if (nb > res[c]) form = 0;
+    }
+    if (!form) {
+        per = kFieldThreads;
+        nb = std::min((ncell + per - 1) / per, res[0]);
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)nb);
+    cfg.blockDim = dim3(kFieldThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const auto kern = form == 0 ? k_cg_coop<0> : (form == 1 ? k_cg_coop<1> : k_cg_coop<2>);
+    return cudaLaunchKernelEx(&cfg, kern, a.grids, a.ntot, a.x, a.r, a.p, a.q, a.cg, a.cg_part,
+                              reinterpret_cast<unsigned int*>(a.cg_part + 2 * kCgMaxBlocks), a.st, per);
 }
 
 void launch_field_update(const FieldArgs& a, cudaStream_t s) {

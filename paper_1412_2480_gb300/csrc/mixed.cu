@@ -1067,16 +1067,10 @@ cudaMemPool_t temp_pool(cudaError_t* e) {
 
 template <typename T>
 cudaError_t talloc(T** p, size_t n, cudaStream_t st) {
-    *p = nullptr;
-    cudaError_t e = cudaSuccess;
-    cudaMemPool_t pool = temp_pool(&e);
-    if (!pool) return e == cudaSuccess ? cudaErrorMemoryAllocation : e;
-    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T), pool, st);
+    return temp_alloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T), st);
 }
 
-void tfree(void* p, cudaStream_t st) {
-    if (p) cudaFreeAsync(p, st);
-}
+void tfree(void* p, cudaStream_t st) { temp_free(p, st); }
 
 void free_parts(PartArrays& A, cudaStream_t st) {
     void* ps[] = {A.cij, A.ox, A.oy, A.ux, A.uy, A.uz, A.gs};
@@ -1421,6 +1415,18 @@ std::vector<long long> current_caps(MixedState* m, bool outboxes) {
 }  // namespace
 
 // =====================================================================================
+
+cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st) {
+    *p = nullptr;
+    cudaError_t e = cudaSuccess;
+    cudaMemPool_t pool = temp_pool(&e);
+    if (!pool) return e == cudaSuccess ? cudaErrorMemoryAllocation : e;
+    return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, st);
+}
+
+void temp_free(void* p, cudaStream_t st) {
+    if (p) cudaFreeAsync(p, st);
+}
 
 int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
                  const GridDev* dgrids, long long ntot, float* F32, long long* Jfix, CgState* cg,

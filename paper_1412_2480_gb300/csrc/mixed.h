@@ -14,6 +14,10 @@ namespace pic {
 
 struct MixedState;
 
+// Temporaries of the library's stream-ordered pool (mixed.cu).
+cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st);
+void temp_free(void* p, cudaStream_t st);
+
 // Choose tiles and allocate bins for ngrids simulations (fills the tile fields of the
 // host descriptors G[0..ngrids), which the caller then copies to dgrids).
 int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,

@@ -8,6 +8,7 @@
 // same kernels as the solve inside pic_step.
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <mutex>
 
 #include "engine.h"
@@ -31,7 +32,8 @@ constexpr size_t kOffCg = kOffGrid + up256(sizeof(GridDev));
 constexpr size_t kOffDone = kOffCg + up256(sizeof(CgState));
 constexpr size_t kOffSt = kOffDone + up256(sizeof(unsigned int));
 constexpr size_t kOffBlk = kOffSt + up256(sizeof(DevStatus));
-constexpr size_t kScratchBytes = kOffBlk + up256((size_t)kNaMaxBlocks * sizeof(int));
+constexpr size_t kOffCgPart = kOffBlk + up256((size_t)kNaMaxBlocks * sizeof(int));
+constexpr size_t kScratchBytes = kOffCgPart + up256((size_t)kCgPartials * sizeof(double));
 
 // Shared by every call on a device and kept until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -140,44 +142,41 @@ extern "C" PIC_API int pic_field_solve_noalloc(int32_t nx, int32_t ny, double dx
     a.cg = reinterpret_cast<CgState*>(base + kOffCg);
     a.done = reinterpret_cast<unsigned int*>(base + kOffDone);
     a.st = reinterpret_cast<DevStatus*>(base + kOffSt);
+    a.cg_part = reinterpret_cast<double*>(base + kOffCgPart);
     a.use_cond = 0;
-    // the array keeps the previous call's contents: clear what must start at zero
-    cudaError_t e = cudaMemcpyAsync(base + kOffGrid, &G, sizeof G, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffBlk, 0, (size_t)G.nblk * sizeof(int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffCg, 0, sizeof(CgState), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffDone, 0, sizeof(unsigned int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffSt, 0, sizeof(DevStatus), s);
+    // the array keeps the previous call's contents: one copy sets the descriptor and clears
+    // what must start at zero behind it (state, counters, status); the block table is zero
+    // from the start and nothing writes it
+    unsigned char head[kOffBlk - kOffGrid] = {0};
+    memcpy(head, &G, sizeof G);
+    cudaError_t e = cudaMemcpyAsync(base + kOffGrid, head, sizeof head, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
         set_err(errbuf, errlen, cudaGetErrorString(e));
         return PIC_ECUDA;
     }
     launch_rhs(a, s);
-    // PCG iterations in batches; kernels of a converged solve return at once
-    unsigned int n_active = 1;
-    int launched = 0;
-    while (n_active && launched < cg_max_iter) {
-        const int batch = (cg_max_iter - launched) < 4 ? (cg_max_iter - launched) : 4;
-        for (int k = 0; k < batch; k++) launch_cg_iteration(a, s);
-        launched += batch;
-        e = cudaMemcpyAsync(&n_active, &a.st->n_active, sizeof n_active, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) {
-            set_err(errbuf, errlen, cudaGetErrorString(e));
-            return PIC_ECUDA;
-        }
+    e = launch_cg(a, (int)N, dev, s);
+    if (e != cudaSuccess) {
+        set_err(errbuf, errlen, cudaGetErrorString(e));
+        return PIC_ECUDA;
     }
-    CgState c{};
-    DevStatus st{};
-    e = cudaMemcpyAsync(&c, a.cg, sizeof c, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&st, a.st, sizeof st, cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(head, base + kOffGrid, sizeof head, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_err(errbuf, errlen, cudaGetErrorString(e));
         return PIC_ECUDA;
     }
+    CgState c{};
+    DevStatus st{};
+    memcpy(&c, head + (kOffCg - kOffGrid), sizeof c);
+    memcpy(&st, head + (kOffSt - kOffGrid), sizeof st);
     if (iters) *iters = c.iters;
     if (rel_resid) *rel_resid = c.rel;
+    if (st.sync_timeout) {
+        set_err(errbuf, errlen, "a grid-wide wait of the PCG timed out");
+        return PIC_ETIMEOUT;
+    }
     if (st.cg_noconv || c.active) {
         set_err(errbuf, errlen, "PCG reached cg_max_iter before cg_rtol");
         return PIC_ECG_NOCONV;

@@ -13,6 +13,7 @@ namespace pic {
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kFieldThreads = 256;  // threads per block of the grid (field) kernels
 constexpr int kPushThreads = 256;   // threads per block of the FP64 particle kernel
+static_assert(kFieldThreads == 256 && kPushThreads == 256, "warp_of_block_sum");
 // Largest tile window (cells) of the MIXED32 kernel: 48 bytes of shared memory per cell
 // (six FP32 field words and six fixed-point current words) within the 227 KB of a CTA.
 constexpr int kMaxWinCells = 4800;
@@ -61,6 +62,9 @@ struct GridDev {
     // fz = q/(dx dy); dt/dx, dt/dy; js40 = jscale 2^-40 (a tile's window scale is js40 2^k)
     float pk_h[2], pk_fx[2], pk_fy[2], pk_fz[2];
     float pk_dtx, pk_dty, js40;
+    // FP64 push constants, likewise: h = (q/m) dt/2, fx = q dx/(dt dx dy), fy = q dy/(dt dx dy),
+    // fz = q/(dx dy); dt/dx, dt/dy
+    double p64_h[2], p64_fx[2], p64_fy[2], p64_fz[2], p64_dtx, p64_dty;
     // MIXED32 field constants as FP32 pairs (h, l), formed once on the host: the
     // right-hand side's theta dt^2/dx^2, theta dt^2/dy^2, 4 pi theta dt^2 jinv/dx and /dy,
     // dt/dx, dt/dy; A's c0, cx, cy; the E update's 4 pi dt jinv and theta
@@ -252,6 +256,15 @@ __device__ __forceinline__ T block_sum(T v, T* scratch) {
     T r = (lane < nw) ? scratch[lane] : T(0);
     r = warp_sum(r);
     return r;
+}
+
+// Sum of 256 values in shared memory by one warp (every lane gets it): eight
+// values per lane, then the lanes, 12 FP64 additions in all. Eight warps of shuffles would
+// issue 45, and every FP64 instruction of a warp takes about 25 cycles of an SM's FP64 pipe
+// here whatever its active lanes.
+__device__ __forceinline__ double warp_of_block_sum(const double* v) {
+    v += threadIdx.x & 31;
+    return warp_sum(((v[0] + v[32]) + (v[64] + v[96])) + ((v[128] + v[160]) + (v[192] + v[224])));
 }
 
 }  // namespace pic
