@@ -299,6 +299,7 @@ FieldArgs field_args(pic_sim* s, int use_cond, cudaGraphConditionalHandle cond) 
     a.e32 = s->e32;
     a.r32b = s->r32b;
     a.z32 = s->z32;
+    a.bar = s->use_coop ? s->coop.bar : nullptr;
     return a;
 }
 

@@ -42,6 +42,7 @@ struct FieldArgs {
     float *r32, *p32, *q32, *e32;      // 3 * ntot each, inner FP32 CG vectors
     float *r32b, *z32;                 // 3 * ntot each: second residual buffer, z = M r
     cudaGraphConditionalHandle cond_in;  // WHILE-node handle of the inner loop
+    unsigned int* bar;                   // the cooperative solve's barrier counter, or nullptr
 };
 
 // Mixed-precision PCG pieces (see fields.cu): inner start, one inner iteration, and the
@@ -79,12 +80,16 @@ constexpr int kCoopMaxGrids = 64;
 struct CoopSolve {
     int2* gchunk = nullptr;       // per simulation: first chunk, chunk count
     int* chunk_grid = nullptr;    // per chunk: simulation
-    int* tile_grid = nullptr;     // per 32 x 64 Chebyshev tile: simulation
+    int* tile_grid = nullptr;     // per Chebyshev tile: simulation
     int2* tile_xy = nullptr;      // per tile: first cell (x, y)
-    double* part = nullptr;       // 2 buffers x 2 values x nchunks chunk partial sums
-    unsigned int* bar = nullptr;  // grid barrier: arrivals, generation
-    int nchunks = 0, nblocks = 0, ngrids = 0, ntiles = 0, cg_inner = 0;
-    int cheb = 0;                 // some simulation takes the Chebyshev inner solve
+    double* part = nullptr;       // chunk partial sums
+    double* cheb_t = nullptr;     // per simulation: Chebyshev solve or not, T_k(sigma)
+    unsigned int* bar = nullptr;  // grid barrier: arrivals
+    int nchunks = 0, nblocks = 0, ngrids = 0, ntiles = 0;
+    int cheb = 0, cg_any = 0;     // some simulation takes the Chebyshev inner solve, the CG
+    int vec = 0;                  // every nx is a multiple of 4: quads of cells
+    int tile_y = 0;               // height of the Chebyshev tiles
+    int rsplit = 1;               // items per chunk of the pair residual
 };
 // PIC_OK, PIC_EINVAL (not applicable: keep the WHILE-node solve) or PIC_ECUDA. cg_inner:
 // the inner solve is always the CG (PIC_CG_INNER).

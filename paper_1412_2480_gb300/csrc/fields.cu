@@ -320,9 +320,11 @@ __global__ void __launch_bounds__(kFieldThreads)
 k_rhs_dw(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids, int nblk_total,
          long long ntot, const double* __restrict__ F, const long long* __restrict__ J, double* __restrict__ x,
          double* __restrict__ r, CgState* cg, double* part, unsigned int* done, DevStatus* st,
-         cudaGraphConditionalHandle cond, int use_cond, double* __restrict__ bout, float* __restrict__ r32) {
+         cudaGraphConditionalHandle cond, int use_cond, double* __restrict__ bout, float* __restrict__ r32,
+         unsigned int* bar) {
     const int g = blk_grid[blockIdx.x];
     const GridDev& G = grids[g];
+    if (bar && blockIdx.x == 0 && threadIdx.x == 0) *bar = 0u;  // for the cooperative solve that follows
     float v[4] = {0.f, 0.f, 0.f, 0.f};  // b.b, r.r, |E|^2, |B|^2
     const DW AX = dwp(G.dw_ax), AY = dwp(G.dw_ay), KJX = dwp(G.dw_kjx), KJY = dwp(G.dw_kjy);
     const DW DTX = dwp(G.dw_dtx), DTY = dwp(G.dw_dty), C0 = dwp(G.dw_c0), CX = dwp(G.dw_cx), CY = dwp(G.dw_cy);
@@ -1293,7 +1295,7 @@ void launch_rhs(const FieldArgs& a, cudaStream_t s) {
     if (a.Jfix)
         k_rhs_dw<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk, a.ntot, a.F, a.Jfix, a.x,
                                                   a.coop ? nullptr : a.r, a.cg, a.part, a.done, a.st, a.cond,
-                                                  a.use_cond, a.b, a.r32);
+                                                  a.use_cond, a.b, a.r32, a.bar);
     else
         k_rhs<double><<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk,
                                                        a.ntot, a.F, a.J64, a.x, a.r, a.cg,

@@ -56,22 +56,28 @@ constexpr int kPerThread = kChunkCells / kCoopThreads;
 constexpr int kInnerMax = 64;  // inner iterations per refinement, as in the WHILE-node solve
 constexpr int kCoopMaxChunks = 4096;  // two partials per chunk staged in shared memory: 64 KB
 
-// Chebyshev inner solve: interior tile (32 x 64 cells), most steps per solve (the
-// window's halo is kChebMaxIt - 1 cells on every side, whatever the steps), the window
-// (56 x 88 cells: 4 strips of 22 rows, one column per thread, 224 threads), its row
-// pitch and height in shared memory with a ring of zero ghost cells, one buffer's size.
+// Chebyshev inner solve: interior tile (32 x TY cells, TY = 64, 32 or 16), most steps per
+// solve (the window's halo is kChebMaxIt - 1 cells on every side, whatever the steps), the
+// window (56 x (TY + 24) cells: 4 strips of rows, one column per thread, 224 threads), its
+// row pitch and height in shared memory with a ring of zero ghost cells, one buffer's size.
+// The height follows from how many CTAs the tiles can fill (coop_create): a step takes a
+// thread through its strip row by row, 22 rows of a 64-row tile or 10 of a 16-row one, so
+// on a grid of few tiles shorter ones shorten the solve, and on a large one their halos
+// cost more than they save.
 constexpr int kChebTileX = 32;
-constexpr int kChebTileY = 64;
 constexpr int kChebMaxIt = 13;
 constexpr int kChebHalo = kChebMaxIt - 1;
 constexpr int kChebW = kChebTileX + 2 * kChebHalo;
-constexpr int kChebH = kChebTileY + 2 * kChebHalo;
 constexpr int kChebStrips = 4;
-constexpr int kChebRows = kChebH / kChebStrips;
 constexpr int kChebPitch = kChebW + 2;
-constexpr int kChebCells = kChebPitch * (kChebH + 2);
-constexpr int kChebTileCells = kChebTileX * kChebTileY;  // the interior, staged for the x update
-static_assert(kChebRows * kChebStrips == kChebH && kChebW * kChebStrips <= kCoopThreads, "window layout");
+template <int TY>
+struct ChebTile {
+    static constexpr int kH = TY + 2 * kChebHalo;
+    static constexpr int kRows = kH / kChebStrips;
+    static constexpr int kCells = kChebPitch * (kH + 2);
+    static constexpr int kInterior = kChebTileX * TY;  // staged for the x update
+    static_assert(kRows * kChebStrips == kH && kChebW * kChebStrips <= kCoopThreads, "window layout");
+};
 constexpr double kChebFloor = 1e-7;
 constexpr double kChebRtolMin = 1e-13;  // the FP32-pair residual resolves about 1e-14 of ||b||
 constexpr double kChebWorst = 1e-3;
@@ -85,6 +91,9 @@ struct CoopArgs {
     const int* tile_grid;   // Chebyshev tiles: simulation, first cell (x, y)
     const int2* tile_xy;
     int ntiles;
+    const double* cheb_t;   // [ngrids][kChebMaxIt + 1]: [0] whether the simulation takes the
+                            // Chebyshev solve, [k] T_k(sigma)
+    int rsplit;             // 3: the Chebyshev path's residual one component at a time
     long long ntot;
     const double* b;
     double* x;
@@ -94,14 +103,15 @@ struct CoopArgs {
     float* p32;
     float* q32;
     float* e32;
-    double* part;           // 2 buffers x 2 values x nchunks, alternating between phases
-    unsigned int* bar;      // [0] arrivals, [1] generation
+    double* part;           // CG: 2 buffers x 2 values x nchunks, alternating between phases
+    double* part_dw;        // pair residual: 2 buffers x 3 components x nchunks, likewise
+    unsigned int* bar;      // arrivals at the grid barriers of this launch (from zero)
     CgState* cg;
     DevStatus* st;
 };
 
 struct GState {
-    double rr, bb, scale, rr_in0, rr_in, rz, alpha, beta, tol_in, rel, rtol;
+    double rr, bb, scale, rr_in0, rr_in, rz, alpha, beta, tol_in, rtol;
     int active, in_active, iters, in_iters, outer, maxit;
     int cheb, m;  // inner solve by the Chebyshev iteration; its steps this refinement
     int dw;       // x is held as FP32 pairs in (p32, q32) until the final join
@@ -115,40 +125,87 @@ struct GState {
 };
 
 // Grid-wide barrier of a cooperative launch (all CTAs resident): arrivals on one counter
-// (word 0), release by advancing the generation (word 1). Bounded: false if the other
-// CTAs did not arrive within `limit` polls; the CTA then leaves the kernel, and so do
-// the others at their next barrier (none waits for ever). (A two-level tree of
-// counters was slower here.)
-constexpr int kBarWords = 2;
-
-__device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned int* timeout, unsigned int limit) {
+// that only grows; the epoch-th barrier is passed when it reaches epoch * nblocks. Bounded:
+// false if the other CTAs did not arrive within `limit` polls; the CTA then leaves the
+// kernel, and so do the others at their next barrier (none waits for ever). 1.3 us on 152
+// CTAs (measured); a counter that is reset, with a generation word and a sleep between
+// polls, took about twice that, a two-level tree of counters more.
+__device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned int epoch, unsigned int* timeout,
+                             unsigned int limit) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned int* gen = bar + 1;
-        const unsigned int g0 = *gen;
         int ok = 1;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == nblocks - 1u) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            unsigned int it = 0;
-            while (*gen == g0) {
-                if (++it > limit) {
-                    atomicExch(timeout, 1u);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
+        unsigned int seen;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        for (unsigned int it = 0;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+            if (seen >= epoch * nblocks) break;
+            if (++it > limit) {
+                atomicExch(timeout, 1u);
+                ok = 0;
+                break;
             }
         }
-        __threadfence();
         s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+// Sum of a simulation's n partials: value k goes to slot k mod 256, the slots are added in
+// a fixed tree. By a whole block (one slot per thread, the result in warp 0) or by one warp
+// (eight slots per lane), with the same bits.
+__device__ __forceinline__ double slot_tree(const double v[8]) {
+    return warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
+}
+__device__ __forceinline__ double partials_block(const double* p, int n, double* s_slot) {
+    const int tid = threadIdx.x;
+    double t = 0.0;
+    for (int k = tid; k < n; k += 4 * kCoopThreads) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u] = k + u * kCoopThreads < n ? __ldcg(p + k + u * kCoopThreads) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (k + u * kCoopThreads < n) t += v[u];
+    }
+    s_slot[tid] = t;
+    __syncthreads();
+    if (tid >= 32) return 0.0;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) v[j] = s_slot[32 * j + tid];
+    return slot_tree(v);
+}
+__device__ __forceinline__ double partials_warp(const double* p, int n) {
+    const int lane = threadIdx.x & 31;
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = lane; k < n; k += kCoopThreads) {
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+            if (k + 32 * j < n) v[j] += __ldcg(p + k + 32 * j);
+    }
+    return slot_tree(v);
+}
+
+// Block sums of N values per thread in FP32-pair arithmetic (off the FP64 pipe), as FP64 in
+// out[0..N) of thread 0's choice: warp c finishes value c.
+template <int N>
+__device__ __forceinline__ void block_sums_dw(const float (&v)[N], double* out) {
+    __shared__ DW s_w[N][kCoopThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int c = 0; c < N; c++) {
+        const DW w = warp_sum_dw(DW{v[c], 0.f});
+        if (lane == 0) s_w[c][warp] = w;
+    }
+    __syncthreads();
+    if (warp < N) {
+        const DW w = warp_sum_dw(lane < kCoopThreads / 32 ? s_w[warp][lane] : DW{0.f, 0.f});
+        if (lane == 0) out[warp] = dw_join(w);
+    }
+    __syncthreads();
 }
 
 // Sum of one simulation's chunk partials (staged in shared memory), by one warp, in a
@@ -177,17 +234,48 @@ __device__ __forceinline__ void stage_partials(const double* part, int n, double
     __syncthreads();
 }
 
-enum Phase { kBegin, kDirection, kUpdate, kX, kResidual, kJoin, kResidualDW };
+enum Phase { kBegin, kDirection, kUpdate, kX, kResidual, kJoin };
 
 // Per-chunk constants, in registers.
 struct ChunkC {
     int nx, ny, ncell, l0, walls, rb;  // rb: residual buffer holding the current r
-    int dw;                            // x lives as FP32 pairs (a.p32, a.q32): the Chebyshev path
     long long off, ntot;
     double c0, cx, cy, inv;
     float c0f, cxf, cyf, betaf, alphaf, pc0f, pcxf, pcyf, scf;
     DW C0, CX, CY;
 };
+
+// Constants of chunk ch of simulation g (FP64 -> FP32 conversions run on the slow FP64 pipe:
+// once per simulation, not per cell).
+__device__ __forceinline__ ChunkC chunk_consts(const CoopArgs& a, const GState& s, int g, int ch, int rb) {
+    const GridDev* Gp = a.grids + g;
+    ChunkC q;
+    q.nx = __ldg(&Gp->nx);
+    q.ny = __ldg(&Gp->ny);
+    q.ncell = __ldg(&Gp->ncell);
+    q.walls = __ldg(&Gp->walls);
+    q.off = __ldg(&Gp->cell_off);
+    q.ntot = a.ntot;
+    q.rb = rb;
+    q.c0 = __ldg(&Gp->c0);
+    q.cx = __ldg(&Gp->cx);
+    q.cy = __ldg(&Gp->cy);
+    q.c0f = s.c0f;
+    q.cxf = s.cxf;
+    q.cyf = s.cyf;
+    q.pc0f = s.pc0f;
+    q.pcxf = s.pcxf;
+    q.pcyf = s.pcyf;
+    q.C0 = s.C0;
+    q.CX = s.CX;
+    q.CY = s.CY;
+    q.betaf = s.betaf;
+    q.alphaf = s.alphaf;
+    q.scf = s.scf;
+    q.inv = s.inv;
+    q.l0 = (ch - __ldg(&a.gchunk[g].x)) * kChunkCells;
+    return q;
+}
 
 // M v for the four cells of a quad: centre quad v, north and south quads, west and east
 // scalars (images already applied).
@@ -342,37 +430,6 @@ __device__ __forceinline__ void chunk_cells(const CoopArgs& a, const ChunkC& q, 
                                       dw_join({h.w, lo.w})};
                 st4d(a.x + o, xv);
             }
-        } else if constexpr (PH == kResidualDW) {  // on the pairs: r = b - A x, its FP32 copy, (r, r)
-            const DW C0 = q.C0, CX = q.CX, CY = q.CY;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const float* XH = a.p32 + c * ntot;
-                const float* XL = a.q32 + c * ntot;
-                const float4 hc = ld4(XH + k), lc = ld4(XL + k), hn = ld4(XH + kn), ln = ld4(XL + kn);
-                const float4 hs = ld4(XH + ks), ls = ld4(XL + ks);
-                DW xw{__ldcg(XH + kwv), __ldcg(XL + kwv)}, xe{__ldcg(XH + kev), __ldcg(XL + kev)};
-                double bv[4];
-                ld4d(a.b + c * ntot + k, bv);
-                const DW xc[4] = {{hc.x, lc.x}, {hc.y, lc.y}, {hc.z, lc.z}, {hc.w, lc.w}};
-                const DW xn[4] = {{hn.x, ln.x}, {hn.y, ln.y}, {hn.z, ln.z}, {hn.w, ln.w}};
-                const DW xs[4] = {{hs.x, ls.x}, {hs.y, ls.y}, {hs.z, ls.z}, {hs.w, ls.w}};
-                if (q.walls) {
-                    if (i == 0) xw = c == 0 ? dw_neg(xc[1]) : xc[0];
-                    if (i + 4 == q.nx) xe = c == 0 ? DW{0.f, 0.f} : xc[3];
-                }
-                float rf[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const DW w = u == 0 ? xw : xc[u - 1];
-                    const DW e = u == 3 ? xe : xc[u + 1];
-                    const DW off = dw_add(dw_mul(CX, dw_add(w, e)), dw_mul(CY, dw_add(xn[u], xs[u])));
-                    const DW Ax = dw_add(dw_mul(C0, xc[u]), dw_neg(off));
-                    const DW r = dw_add(dw_from(bv[u]), dw_neg(Ax));
-                    rf[u] = r.h;
-                    acc1 = fmaf(r.h, r.h, acc1);
-                }
-                st4(a.r32[0] + c * ntot + k, make_float4(rf[0], rf[1], rf[2], rf[3]));
-            }
         } else {  // kResidual: r = b - A x in FP64
 #pragma unroll
             for (int c = 0; c < 3; c++) {
@@ -463,33 +520,41 @@ __device__ __forceinline__ void direction_full(const CoopArgs& a, const ChunkC& 
     }
 }
 
-// The pair residual on a full chunk, component by component with the loads of both
-// quads issued before any arithmetic (as direction_full, for the same reason).
-__device__ __forceinline__ void residual_dw_full(const CoopArgs& a, const ChunkC& q, float& acc1) {
-    int k[kQuads], kn[kQuads], ks[kQuads], kw[kQuads], ke[kQuads], ii[kQuads];
+// The pair residual r = b - A x of component c on a chunk: its FP32 copy and the thread's
+// part of (r, r). A x from the pairs' five points.
+__device__ __forceinline__ DW pair_residual(const ChunkC& q, DW xc, DW xw, DW xe, DW xn, DW xs, double b) {
+    const DW off = dw_add(dw_mul(q.CX, dw_add(xw, xe)), dw_mul(q.CY, dw_add(xn, xs)));
+    return dw_add(dw_from(b), dw_neg(dw_add(dw_mul(q.C0, xc), dw_neg(off))));
+}
+
+// nx a multiple of 4: components c0 .. c0 + NC - 1 on NQ quads of cells from quad q0 of the
+// thread, with vector loads, those of all quads issued before any arithmetic (as
+// direction_full, for the same reason); acc gets the sums of squares added.
+template <int NC, int NQ>
+__device__ __forceinline__ void residual_quads(const CoopArgs& a, const ChunkC& q, int c0, int q0, float (&acc)[NC]) {
+    int k[NQ], kn[NQ], ks[NQ], kw[NQ], ke[NQ], ii[NQ];
 #pragma unroll
-    for (int qq = 0; qq < kQuads; qq++) {
-        const int l = q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x);
-        const int j = l / q.nx, i = l - j * q.nx;
-        const int row = j * q.nx;
+    for (int qq = 0; qq < NQ; qq++) {
+        const int l = q.l0 + 4 * ((q0 + qq) * kCoopThreads + (int)threadIdx.x);
+        const int j = l / q.nx, i = l - j * q.nx, row = j * q.nx;
         ii[qq] = i;
-        k[qq] = row + i;
+        k[qq] = l;
         kw[qq] = row + (i == 0 ? q.nx - 1 : i - 1);
         ke[qq] = row + (i + 4 == q.nx ? 0 : i + 4);
         kn[qq] = (j + 1 == q.ny ? 0 : j + 1) * q.nx + i;
         ks[qq] = (j == 0 ? q.ny - 1 : j - 1) * q.nx + i;
     }
-    const DW C0 = q.C0, CX = q.CX, CY = q.CY;
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
+    for (int cc = 0; cc < NC; cc++) {
+        const int c = c0 + cc;
         const long long o = c * q.ntot + q.off;
         const float* XH = a.p32 + o;
         const float* XL = a.q32 + o;
-        float4 hc[kQuads], lc[kQuads], hn[kQuads], ln[kQuads], hs[kQuads], ls[kQuads];
-        float hw[kQuads], lw[kQuads], he[kQuads], le[kQuads];
-        double bv[kQuads][4];
+        float4 hc[NQ], lc[NQ], hn[NQ], ln[NQ], hs[NQ], ls[NQ];
+        float hw[NQ], lw[NQ], he[NQ], le[NQ];
+        double bv[NQ][4];
 #pragma unroll
-        for (int qq = 0; qq < kQuads; qq++) {
+        for (int qq = 0; qq < NQ; qq++) {
             hc[qq] = ld4(XH + k[qq]);
             lc[qq] = ld4(XL + k[qq]);
             hn[qq] = ld4(XH + kn[qq]);
@@ -503,7 +568,7 @@ __device__ __forceinline__ void residual_dw_full(const CoopArgs& a, const ChunkC
             ld4d(a.b + o + k[qq], bv[qq]);
         }
 #pragma unroll
-        for (int qq = 0; qq < kQuads; qq++) {
+        for (int qq = 0; qq < NQ; qq++) {
             const DW xc[4] = {{hc[qq].x, lc[qq].x}, {hc[qq].y, lc[qq].y}, {hc[qq].z, lc[qq].z}, {hc[qq].w, lc[qq].w}};
             const DW xn[4] = {{hn[qq].x, ln[qq].x}, {hn[qq].y, ln[qq].y}, {hn[qq].z, ln[qq].z}, {hn[qq].w, ln[qq].w}};
             const DW xs[4] = {{hs[qq].x, ls[qq].x}, {hs[qq].y, ls[qq].y}, {hs[qq].z, ls[qq].z}, {hs[qq].w, ls[qq].w}};
@@ -515,17 +580,100 @@ __device__ __forceinline__ void residual_dw_full(const CoopArgs& a, const ChunkC
             float rf[4];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
-                const DW w = u == 0 ? xw : xc[u - 1];
-                const DW e = u == 3 ? xe : xc[u + 1];
-                const DW off = dw_add(dw_mul(CX, dw_add(w, e)), dw_mul(CY, dw_add(xn[u], xs[u])));
-                const DW Ax = dw_add(dw_mul(C0, xc[u]), dw_neg(off));
-                const DW r = dw_add(dw_from(bv[qq][u]), dw_neg(Ax));
+                const DW r = pair_residual(q, xc[u], u == 0 ? xw : xc[u - 1], u == 3 ? xe : xc[u + 1], xn[u], xs[u], bv[qq][u]);
                 rf[u] = r.h;
-                acc1 = fmaf(r.h, r.h, acc1);
+                acc[cc] = fmaf(r.h, r.h, acc[cc]);
             }
             st4(a.r32[0] + o + k[qq], make_float4(rf[0], rf[1], rf[2], rf[3]));
         }
     }
+}
+
+// Any nx: one cell per thread and step, kCellsAhead in flight. Neighbouring cells of a
+// warp's row come from the same lines, so the scalar loads cost issue slots and not traffic.
+constexpr int kCellsAhead = 2;  // (four spill)
+template <int NC>
+__device__ __forceinline__ void residual_cells(const CoopArgs& a, const ChunkC& q, int c0, float (&acc)[NC]) {
+#pragma unroll 1
+    for (int q0 = 0; q0 < kPerThread; q0 += kCellsAhead) {
+        int k[kCellsAhead], kw[kCellsAhead], ke[kCellsAhead], kn[kCellsAhead], ks[kCellsAhead], ii[kCellsAhead];
+#pragma unroll
+        for (int u = 0; u < kCellsAhead; u++) {
+            // (a cell beyond the grid repeats its last one, and counts for nothing)
+            const int l = q.l0 + (q0 + u) * kCoopThreads + (int)threadIdx.x, lc = min(l, q.ncell - 1);
+            const int j = lc / q.nx, i = lc - j * q.nx, row = j * q.nx;
+            ii[u] = i;
+            k[u] = lc;
+            kw[u] = row + (i == 0 ? q.nx - 1 : i - 1);
+            ke[u] = row + (i + 1 == q.nx ? 0 : i + 1);
+            kn[u] = (j + 1 == q.ny ? 0 : j + 1) * q.nx + i;
+            ks[u] = (j == 0 ? q.ny - 1 : j - 1) * q.nx + i;
+        }
+#pragma unroll
+        for (int cc = 0; cc < NC; cc++) {
+            const int c = c0 + cc;
+            const long long o = c * q.ntot + q.off;
+            const float* XH = a.p32 + o;
+            const float* XL = a.q32 + o;
+            DW xc[kCellsAhead], xw[kCellsAhead], xe[kCellsAhead], xn[kCellsAhead], xs[kCellsAhead];
+            double bv[kCellsAhead];
+#pragma unroll
+            for (int u = 0; u < kCellsAhead; u++) {
+                xc[u] = DW{__ldcg(XH + k[u]), __ldcg(XL + k[u])};
+                xw[u] = DW{__ldcg(XH + kw[u]), __ldcg(XL + kw[u])};
+                xe[u] = DW{__ldcg(XH + ke[u]), __ldcg(XL + ke[u])};
+                xn[u] = DW{__ldcg(XH + kn[u]), __ldcg(XL + kn[u])};
+                xs[u] = DW{__ldcg(XH + ks[u]), __ldcg(XL + ks[u])};
+                bv[u] = __ldcg(a.b + o + k[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kCellsAhead; u++) {
+                if (q.walls) {
+                    if (ii[u] == 0) xw[u] = c == 0 ? dw_neg(xe[u]) : xc[u];
+                    if (ii[u] + 1 == q.nx) xe[u] = c == 0 ? DW{0.f, 0.f} : xc[u];
+                }
+                const DW r = pair_residual(q, xc[u], xw[u], xe[u], xn[u], xs[u], bv[u]);
+                if (q.l0 + (q0 + u) * kCoopThreads + (int)threadIdx.x < q.ncell) {
+                    a.r32[0][o + k[u]] = r.h;
+                    acc[cc] = fmaf(r.h, r.h, acc[cc]);
+                }
+            }
+        }
+    }
+}
+
+// Components c0 .. c0 + NC - 1 of a chunk's pair residual and their partial sums.
+template <bool VEC, int NC>
+__device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, int g, int ch, int c0, double* part) {
+    const ChunkC q = chunk_consts(a, s, g, ch, 0);
+    float acc[NC];
+#pragma unroll
+    for (int cc = 0; cc < NC; cc++) acc[cc] = 0.f;
+    if constexpr (VEC) {
+        if (q.l0 + kChunkCells <= q.ncell) {
+            residual_quads<NC, kQuads>(a, q, c0, 0, acc);
+        } else {
+#pragma unroll 1
+            for (int qq = 0; qq < kQuads; qq++)
+                if (q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x) < q.ncell) residual_quads<NC, 1>(a, q, c0, qq, acc);
+        }
+    } else {
+        residual_cells<NC>(a, q, c0, acc);
+    }
+    block_sums_dw<NC>(acc, part + c0);
+}
+
+// x = h + l (FP64) on a chunk of any nx.
+__device__ __forceinline__ void join_cells(const CoopArgs& a, const ChunkC& q) {
+#pragma unroll
+    for (int c = 0; c < 3; c++)
+#pragma unroll
+        for (int u = 0; u < kPerThread; u++) {
+            const int l = q.l0 + u * kCoopThreads + (int)threadIdx.x;
+            if (l >= q.ncell) continue;
+            const long long o = c * q.ntot + q.off + l;
+            a.x[o] = dw_join({__ldcg(a.p32 + o), __ldcg(a.q32 + o)});
+        }
 }
 
 template <int PH>
@@ -534,9 +682,6 @@ __device__ __forceinline__ void chunk_phase(const CoopArgs& a, const ChunkC& q, 
     const bool full = q.l0 + kChunkCells <= q.ncell;
     if constexpr (PH == kDirection) {
         if (full) return direction_full(a, q, acc1);
-    }
-    if constexpr (PH == kResidualDW) {
-        if (full) return residual_dw_full(a, q, acc1);
     }
     if (full) chunk_cells<PH, true>(a, q, acc1, acc2, accd);
     else chunk_cells<PH, false>(a, q, acc1, acc2, accd);
@@ -563,6 +708,11 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+template <int BYTES>  // 4 or 8, aligned likewise
+__device__ __forceinline__ void cp_async_small(void* smem, const void* gmem) {
+    const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
@@ -570,7 +720,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // new e to dst (distinct buffers).
 // WALL: this column is a wall column (wl or wr set); the other columns take the form
 // without the image selects.
-template <bool WALL>
+template <bool WALL, int kChebRows>
 __device__ __forceinline__ void cheb_step(const float* __restrict__ src, float* __restrict__ dst, int base,
                                           float (&e)[kChebRows], float (&d)[kChebRows],
                                           const float (&rs)[kChebRows], float c0f, float cxf, float cyf,
@@ -600,7 +750,11 @@ __device__ __forceinline__ void cheb_step(const float* __restrict__ src, float* 
     }
 }
 
+// VEC: nx and the simulations' offsets are multiples of 4 cells.
+template <bool VEC, int kChebTileY>
 __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, int g, int t, int c, float* ew) {
+    constexpr int kChebRows = ChebTile<kChebTileY>::kRows, kChebCells = ChebTile<kChebTileY>::kCells;
+    constexpr int kChebTileCells = ChebTile<kChebTileY>::kInterior;
     const GridDev* Gp = a.grids + g;
     const int nx = __ldg(&Gp->nx), ny = __ldg(&Gp->ny), walls = __ldg(&Gp->walls);
     const long long off = __ldg(&Gp->cell_off);
@@ -630,12 +784,25 @@ __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, in
     float* ea = ew;
     float* eb = ew + kChebCells;
     // the interior's x, staged asynchronously during the steps: pairs (h rows, then l
-    // rows) or, in the solve's first refinement, FP64 values; rows of kChebTileX, 16-byte
-    // chunks (nx, the offsets and X0 are multiples of 4 cells, so chunks stay aligned)
+    // rows) or, in the solve's first refinement, FP64 values; rows of kChebTileX, in 16-byte
+    // chunks with VEC (nx, the offsets and X0 are multiples of 4 cells then, so chunks stay
+    // aligned), one value at a time without
     float* xst = ew + 2 * kChebCells;
     const int nrow = Y1 - Y0, ncol = X1 - X0;
     const long long ob = c * a.ntot + off + (long long)Y0 * nx + X0;
-    if (s.dw) {
+    if constexpr (!VEC) {
+        for (int q = tid; q < kChebTileCells; q += kCoopThreads) {
+            const int y = q / kChebTileX, xx = q - y * kChebTileX;
+            if (y >= nrow || xx >= ncol) continue;
+            const long long k = ob + (long long)y * nx + xx;
+            if (s.dw) {
+                cp_async_small<4>(xst + q, a.p32 + k);
+                cp_async_small<4>(xst + kChebTileCells + q, a.q32 + k);
+            } else {
+                cp_async_small<8>(reinterpret_cast<double*>(xst) + q, a.x + k);
+            }
+        }
+    } else if (s.dw) {
         for (int q = tid; q < 2 * kChebTileY * (kChebTileX / 4); q += kCoopThreads) {
             const int arr = q / (kChebTileY * (kChebTileX / 4)), rem = q - arr * (kChebTileY * (kChebTileX / 4));
             const int y = rem / (kChebTileX / 4), x4 = 4 * (rem - y * (kChebTileX / 4));
@@ -666,8 +833,8 @@ __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, in
         const float ca = rn * rho, cb = 2.f * rn / delta;
         rho = rn;
         if (act) {
-            if (wl || wr) cheb_step<true>(ea, eb, base, e, d, rs, c0f, cxf, cyf, ca, cb, wl, wr, c == 0);
-            else cheb_step<false>(ea, eb, base, e, d, rs, c0f, cxf, cyf, ca, cb, false, false, false);
+            if (wl || wr) cheb_step<true, kChebRows>(ea, eb, base, e, d, rs, c0f, cxf, cyf, ca, cb, wl, wr, c == 0);
+            else cheb_step<false, kChebRows>(ea, eb, base, e, d, rs, c0f, cxf, cyf, ca, cb, false, false, false);
         }
         __syncthreads();
         float* tmp = ea;
@@ -714,11 +881,13 @@ __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, in
 // CG inner solve: 4 CTAs per SM (64 registers), 608 resident CTAs, so a 2048 x 512
 // grid (512 chunks) gives every CTA at most one chunk per phase. With Chebyshev tiles
 // (CHEB): 2 CTAs per SM, so that a thread holds its column strip in registers.
-template <bool CHEB>
-__global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const CoopArgs a) {
+// CHEB, CG: some simulation takes the Chebyshev solve, the CG; VEC: every simulation's nx is a multiple of
+// 4 (the CG needs it); TY: tile height.
+template <bool CHEB, bool CG, bool VEC, int TY>
+__global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __grid_constant__ CoopArgs a) {
     __shared__ GState gs[kCoopMaxGrids];
-    __shared__ double red[32];
-    extern __shared__ __align__(16) double sp[];  // 2 x nchunks staged partial sums
+    __shared__ double red[32], s_slot[kCoopThreads];
+    extern __shared__ __align__(16) double sp[];  // Chebyshev window; staged partial sums of the CG
     DevStatus* st = a.st;
     if (st->stop) return;  // the same for every CTA: stop changes only between launches
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -729,7 +898,6 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
         GState s{};
         s.rr = c.rr;
         s.bb = c.bb;
-        s.rel = c.rel;
         s.active = c.active;
         s.iters = 0;
         s.outer = 0;
@@ -737,9 +905,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
         s.maxit = a.grids[g].maxit;
         const double c0 = a.grids[g].c0, dl = 2.0 * (a.grids[g].cx + a.grids[g].cy);
         const double sig = dl > 0.0 ? c0 / dl : 0.0;
-        // Chebyshev when 13 steps reduce the error by kChebWorst at least (T_13(sigma) =
-        // cosh(13 acosh sigma) >= 1 / kChebWorst) and the tiles cover the simulation
-        s.cheb = CHEB && sig > 1.0 && kChebMaxIt * acosh(sig) >= acosh(1.0 / kChebWorst) && s.rtol >= kChebRtolMin;
+        s.cheb = CHEB && a.cheb_t[g * (kChebMaxIt + 1)] != 0.0;
         s.dw = 0;
         s.sig = (float)sig;
         s.m = 0;
@@ -756,12 +922,14 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
         gs[g] = s;
     }
     __syncthreads();
-    // window of the Chebyshev tiles after the staged partial sums: two e buffers whose
-    // ghost rings stay zero (the steps write window cells only)
-    float* ew = reinterpret_cast<float*>(sp + 2 * a.nchunks);
+    // window of the Chebyshev tiles: two e buffers whose ghost rings stay zero (the steps
+    // write window cells only), and the staged interior; the CG's partial sums after it
+    float* ew = reinterpret_cast<float*>(sp);
     if constexpr (CHEB)
-        for (int k = tid; k < 2 * kChebCells; k += blockDim.x) ew[k] = 0.f;
-    int buf = 0;
+        for (int k = tid; k < 2 * ChebTile<TY>::kCells; k += blockDim.x) ew[k] = 0.f;
+    double* const spart = CHEB ? reinterpret_cast<double*>(ew + 2 * ChebTile<TY>::kCells + 2 * ChebTile<TY>::kInterior) : sp;
+    unsigned int epoch = 0;  // grid barriers passed
+    int buf = 0, pbuf = 0;   // partial-sum buffers in use: the CG's, the pair residual's
     int rb = 0;  // residual buffer holding the current inner r (the same in every CTA)
     bool ok = true;
     const auto two = [](Phase ph) { return ph == kBegin || ph == kUpdate; };  // phases with two sums
@@ -772,7 +940,21 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
         if (ph == kDirection || ph == kUpdate) return s.active && s.in_active;
         if (ph == kBegin || ph == kX) return s.active && !s.cheb;
         if (ph == kJoin) return s.dw != 0;
-        return s.active != 0;
+        return s.active && !s.dw;  // kResidual (the pairs' residual has its own pass)
+    };
+    // The pair residual of the simulations on pairs: the items are the chunks, or their
+    // three components where the chunks alone would leave CTAs idle; one partial per chunk
+    // and component either way, from one accumulator per thread and component.
+    auto pair_pass = [&]() {
+        double* part = a.part_dw + (size_t)pbuf * 3 * a.nchunks;
+        const int nitems = a.nchunks * a.rsplit;
+        for (int it = blockIdx.x; it < nitems; it += nb) {
+            const int ch = it / a.rsplit;
+            const int g = __ldg(a.chunk_grid + ch);
+            if (!(gs[g].active && gs[g].dw)) continue;  // uniform over the CTA
+            if (a.rsplit == 3) pair_chunk<VEC, 1>(a, gs[g], g, ch, it - 3 * ch, part + 3 * (size_t)ch);
+            else pair_chunk<VEC, 3>(a, gs[g], g, ch, 0, part + 3 * (size_t)ch);
+        }
     };
     // One pass over this CTA's chunks of the simulations taking part in `ph`, with
     // per-chunk partial sums into buffer `buf` where the phase reduces.
@@ -782,56 +964,27 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
             const int g = __ldg(a.chunk_grid + ch);
             const GState& s = gs[g];
             if (!takes(ph, s)) continue;  // uniform over the CTA
-            // per-chunk constants in registers (FP64 -> FP32 conversions run on the slow
-            // FP64 pipe: once per chunk, not per cell)
-            const GridDev* Gp = a.grids + g;
-            ChunkC q;
-            q.nx = __ldg(&Gp->nx);
-            q.ny = __ldg(&Gp->ny);
-            q.ncell = __ldg(&Gp->ncell);
-            q.walls = __ldg(&Gp->walls);
-            q.off = __ldg(&Gp->cell_off);
-            q.ntot = a.ntot;
-            q.rb = rb;
-            q.c0 = __ldg(&Gp->c0);
-            q.cx = __ldg(&Gp->cx);
-            q.cy = __ldg(&Gp->cy);
-            q.c0f = s.c0f;
-            q.cxf = s.cxf;
-            q.cyf = s.cyf;
-            q.pc0f = s.pc0f;
-            q.pcxf = s.pcxf;
-            q.pcyf = s.pcyf;
-            q.C0 = s.C0;
-            q.CX = s.CX;
-            q.CY = s.CY;
-            q.betaf = s.betaf;
-            q.alphaf = s.alphaf;
-            q.scf = s.scf;
-            q.inv = s.inv;
-            q.dw = s.dw;
-            q.l0 = (ch - __ldg(&a.gchunk[g].x)) * kChunkCells;
+            const ChunkC q = chunk_consts(a, gs[g], g, ch, rb);
             float acc1 = 0.f, acc2 = 0.f;
             double accd = 0.0;
-            switch (ph) {
-            case kBegin: chunk_phase<kBegin>(a, q, acc1, acc2, accd); break;
-            case kDirection: chunk_phase<kDirection>(a, q, acc1, acc2, accd); break;
-            case kUpdate: chunk_phase<kUpdate>(a, q, acc1, acc2, accd); break;
-            case kX: chunk_phase<kX>(a, q, acc1, acc2, accd); break;
-            case kJoin:
-                if constexpr (CHEB) chunk_phase<kJoin>(a, q, acc1, acc2, accd);
-                break;
-            default:
-                if constexpr (CHEB)
-                    if (q.dw) {
-                        chunk_phase<kResidualDW>(a, q, acc1, acc2, accd);
-                        break;
-                    }
-                chunk_phase<kResidual>(a, q, acc1, acc2, accd);
-                break;
+            if constexpr (!CG) {  // (no other phase is reached without CG)
+                if constexpr (VEC) chunk_phase<kJoin>(a, q, acc1, acc2, accd);
+                else join_cells(a, q);
+                continue;
+            } else {
+                switch (ph) {
+                case kBegin: chunk_phase<kBegin>(a, q, acc1, acc2, accd); break;
+                case kDirection: chunk_phase<kDirection>(a, q, acc1, acc2, accd); break;
+                case kUpdate: chunk_phase<kUpdate>(a, q, acc1, acc2, accd); break;
+                case kX: chunk_phase<kX>(a, q, acc1, acc2, accd); break;
+                case kJoin:
+                    if constexpr (CHEB) chunk_phase<kJoin>(a, q, acc1, acc2, accd);
+                    break;
+                default: chunk_phase<kResidual>(a, q, acc1, acc2, accd); break;
+                }
             }
             if (ph != kX && ph != kJoin) {
-                const double t1 = block_sum(ph == kResidual && !q.dw ? accd : (double)acc1, red);
+                const double t1 = block_sum(ph == kResidual ? accd : (double)acc1, red);
                 if (tid == 0) part[ch] = t1;
                 __syncthreads();  // red is reused next
                 if (two(ph)) {
@@ -842,16 +995,58 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
             }
         }
     };
+    // The residual's sum t of simulation s: the outer test, on the squares (and in the last
+    // bits as the quotient's root says).
+    auto judge = [&](GState& s, double t) {
+        s.rr = t;
+        s.outer += 1;
+        bool conv = t <= s.rtol * s.rtol * s.bb * (1.0 + 1e-12);
+        if (conv) conv = sqrt(t / s.bb) <= s.rtol;
+        if (conv) {
+            s.active = 0;
+        } else if (s.iters >= s.maxit || s.outer >= s.maxit) {
+            s.active = 0;
+            if (blockIdx.x == 0) {
+                atomicAdd(&st->cg_noconv, 1u);
+                st->stop_next = 1u;
+            }
+        }
+    };
+    // After the pair residual's barrier: every CTA forms the sums alike (by the whole block
+    // for a few simulations, by one warp each for many).
+    auto pair_reduce = [&]() {
+        const double* part = a.part_dw + (size_t)pbuf * 3 * a.nchunks;
+        if (a.ngrids <= 4) {
+            for (int g = 0; g < a.ngrids; g++) {
+                GState& s = gs[g];
+                if (!(s.active && s.dw)) continue;  // uniform over the CTA
+                const int2 gc = a.gchunk[g];
+                const double t = partials_block(part + 3 * (size_t)gc.x, 3 * gc.y, s_slot);
+                if (tid == 0) judge(s, t);
+                __syncthreads();
+            }
+        } else {
+            for (int g = warp; g < a.ngrids; g += kCoopThreads / 32) {
+                GState& s = gs[g];
+                if (!(s.active && s.dw)) continue;
+                const int2 gc = a.gchunk[g];
+                const double t = partials_warp(part + 3 * (size_t)gc.x, 3 * gc.y);
+                __syncwarp();
+                if (lane == 0) judge(s, t);
+            }
+            __syncthreads();
+        }
+    };
     // After a barrier: every CTA forms the sums of the phase for all simulations taking
     // part, then updates their scalars identically.
     auto reduce = [&](Phase ph) {
         const double* part = a.part + (size_t)buf * 2 * a.nchunks;
-        stage_partials(part, two(ph) ? 2 * a.nchunks : a.nchunks, sp);
+        stage_partials(part, two(ph) ? 2 * a.nchunks : a.nchunks, spart);
         for (int g = warp; g < a.ngrids; g += kCoopThreads / 32) {
             GState& s = gs[g];
             if (!takes(ph, s)) continue;
-            const double t = chunk_sum(sp, a.gchunk[g]);
-            const double t2 = two(ph) ? chunk_sum(sp + a.nchunks, a.gchunk[g]) : 0.0;
+            const double t = chunk_sum(spart, a.gchunk[g]);
+            const double t2 = two(ph) ? chunk_sum(spart + a.nchunks, a.gchunk[g]) : 0.0;
             if (lane != 0) continue;
             if (ph == kBegin) {
                 s.rr_in0 = t;
@@ -876,18 +1071,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
                     !(t2 > 0.0))
                     s.in_active = 0;
             } else if (ph == kResidual) {
-                s.rr = t;
-                s.rel = sqrt(t / s.bb);
-                s.outer += 1;
-                if (s.rel <= s.rtol) {
-                    s.active = 0;
-                } else if (s.iters >= s.maxit || s.outer >= s.maxit) {
-                    s.active = 0;
-                    if (blockIdx.x == 0) {
-                        atomicAdd(&st->cg_noconv, 1u);
-                        st->stop_next = 1u;
-                    }
-                }
+                judge(s, t);
             }
         }
         __syncthreads();
@@ -904,24 +1088,30 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
         return n > 0;
     };
 
+    const auto barrier = [&]() { return grid_barrier(a.bar, nb, ++epoch, &st->sync_timeout, lim); };
     while (ok && any(false)) {
         for (int g = tid; g < a.ngrids; g += blockDim.x)
             if (gs[g].active) {
                 GState& s = gs[g];
-                // r32 of about unit RMS: the power of two in [s/2, s), s = sqrt(3 ncell / (r, r))
-                int ex;
-                frexp(sqrt(3.0 * a.grids[g].ncell / s.rr), &ex);
-                s.scale = ldexp(1.0, ex - 1);
-                s.inv = ldexp(1.0, 1 - ex);
+                // r32 of about unit RMS: the power of two in (s/2, s], s = sqrt(3 ncell / (r, r)),
+                // from the quotient's exponent (its root's is half of it, rounded down)
+                const long long n = __double_as_longlong(3.0 * a.grids[g].ncell), d = __double_as_longlong(s.rr);
+                const long long man = (1ll << 52) - 1;
+                const int e2 = (int)(n >> 52) - (int)(d >> 52) - ((n & man) < (d & man) ? 1 : 0);
+                const int ex = e2 >> 1;
+                s.scale = ldexp(1.0, ex);
+                s.inv = ldexp(1.0, -ex);
                 s.scf = (float)s.scale;
                 s.invf = (float)s.inv;
                 s.in_active = 0;
                 if (s.cheb) {
-                    // the reduction this refinement needs (the CG's inner tolerance), in
-                    // Chebyshev steps: 1 / T_m(sigma) <= tgt
-                    const double tgt = fmax(kChebFloor, 0.5 * s.rtol * sqrt(s.bb / fmax(s.rr, 1e-300)));
-                    const int m = (int)ceil(acosh(1.0 / tgt) / acosh((double)s.sig));
-                    s.m = max(1, min(kChebMaxIt, m));
+                    // steps m for the reduction tgt = max(floor, rtol ||b|| / (2 ||r||)) that
+                    // this refinement needs (the CG's inner tolerance): 1 / T_m(sigma) <= tgt
+                    const double* T = a.cheb_t + g * (kChebMaxIt + 1);
+                    const double want = 0.25 * s.rtol * s.rtol * s.bb;
+                    int m = 1;
+                    while (m < kChebMaxIt && T[m] * kChebFloor < 1.0 && T[m] * T[m] * want < s.rr) m++;
+                    s.m = m;
                 }
             }
         __syncthreads();
@@ -931,7 +1121,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
                 const int t = it / 3, c = it - 3 * (it / 3);
                 const int g = __ldg(a.tile_grid + t);
                 if (!(gs[g].active && gs[g].cheb)) continue;  // uniform over the CTA
-                if constexpr (CHEB) cheb_tile(a, gs[g], g, t, c, ew);
+                if constexpr (CHEB) cheb_tile<VEC, TY>(a, gs[g], g, t, c, ew);
             }
             for (int g = tid; g < a.ngrids; g += blockDim.x)
                 if (gs[g].active && gs[g].cheb) {
@@ -946,42 +1136,53 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
             }
             __syncthreads();
         }
-        if (!any_mode(0)) {
-            ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
+        if constexpr (CHEB) {
+            if (!any_mode(0)) {
+                ok = barrier();
+                if (!ok) break;
+                pair_pass();
+                ok = barrier();
+                if (!ok) break;
+                pair_reduce();
+                pbuf ^= 1;
+                if (blockIdx.x == 0 && tid == 0) st->loop_iters[1] += 1ull;
+                continue;
+            }
+        }
+        if constexpr (CG) {
+            pass(kBegin);
+            rb = 1;  // the first pass wrote the scaled residual into buffer 1
+            ok = barrier();
             if (!ok) break;
+            reduce(kBegin);
+            while (any(true)) {
+                pass(kDirection);
+                ok = barrier();
+                if (!ok) break;
+                reduce(kDirection);
+                pass(kUpdate);
+                rb ^= 1;  // the update pass wrote r' into the other buffer
+                ok = barrier();
+                if (!ok) break;
+                reduce(kUpdate);
+                if (blockIdx.x == 0 && tid == 0) st->loop_iters[0] += 1ull;
+            }
+            if (!ok) break;
+            pass(kX);
+            ok = barrier();
+            if (!ok) break;
+            // the residuals in FP64 (CG) and of the pairs (Chebyshev)
             pass(kResidual);
-            ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
+            if constexpr (CHEB) pair_pass();
+            ok = barrier();
             if (!ok) break;
+            if constexpr (CHEB) pair_reduce();
+            pbuf ^= 1;
             reduce(kResidual);
             if (blockIdx.x == 0 && tid == 0) st->loop_iters[1] += 1ull;
-            continue;
+        } else {
+            break;  // not reached: every simulation takes the Chebyshev solve
         }
-        pass(kBegin);
-        rb = 1;  // the first pass wrote the scaled residual into buffer 1
-        ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
-        if (!ok) break;
-        reduce(kBegin);
-        while (any(true)) {
-            pass(kDirection);
-            ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
-            if (!ok) break;
-            reduce(kDirection);
-            pass(kUpdate);
-            rb ^= 1;  // the update pass wrote r' into the other buffer
-            ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
-            if (!ok) break;
-            reduce(kUpdate);
-            if (blockIdx.x == 0 && tid == 0) st->loop_iters[0] += 1ull;
-        }
-        if (!ok) break;
-        pass(kX);
-        ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
-        if (!ok) break;
-        pass(kResidual);
-        ok = grid_barrier(a.bar, nb, &st->sync_timeout, lim);
-        if (!ok) break;
-        reduce(kResidual);
-        if (blockIdx.x == 0 && tid == 0) st->loop_iters[1] += 1ull;
     }
     if (!ok) {
         if (tid == 0) st->stop_next = 1u;
@@ -993,7 +1194,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
             CgState& c = a.cg[g];
             const GState& s = gs[g];
             c.rr = s.rr;
-            c.rel = s.rel;
+            if (s.outer) c.rel = sqrt(s.rr / s.bb);
             c.active = 0;
             c.iters = s.iters;
             c.outer = s.outer;
@@ -1004,48 +1205,109 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const Co
 
 }  // namespace
 
-size_t coop_smem(const CoopSolve& cs) {
-    return 2 * (size_t)cs.nchunks * sizeof(double) +
-           (cs.cheb ? (2 * (size_t)kChebCells + 2 * (size_t)kChebTileCells) * sizeof(float) : 0);
+namespace {
+
+size_t window_floats(int ty) {
+    switch (ty) {
+    case 16: return 2 * (size_t)ChebTile<16>::kCells + 2 * (size_t)ChebTile<16>::kInterior;
+    case 32: return 2 * (size_t)ChebTile<32>::kCells + 2 * (size_t)ChebTile<32>::kInterior;
+    default: return 2 * (size_t)ChebTile<64>::kCells + 2 * (size_t)ChebTile<64>::kInterior;
+    }
 }
 
-// Whether simulation g can take the Chebyshev inner solve (as the kernel decides).
-bool cheb_ok(const GridDev& G) {
+using CoopKernel = void (*)(const CoopArgs);
+CoopKernel coop_kernel(const CoopSolve& cs) {
+    if (cs.cg_any) return cs.cheb ? k_mp_coop<true, true, true, 64> : k_mp_coop<false, true, true, 64>;
+    switch (cs.tile_y) {
+    case 16: return cs.vec ? k_mp_coop<true, false, true, 16> : k_mp_coop<true, false, false, 16>;
+    case 32: return cs.vec ? k_mp_coop<true, false, true, 32> : k_mp_coop<true, false, false, 32>;
+    default: return cs.vec ? k_mp_coop<true, false, true, 64> : k_mp_coop<true, false, false, 64>;
+    }
+}
+
+// sigma = c0 / (2 (cx + cy)) of A's spectrum interval, and whether simulation G can take
+// the Chebyshev inner solve: 13 steps reduce the error by kChebWorst at least (T_13(sigma) =
+// cosh(13 acosh sigma) >= 1 / kChebWorst) and its tolerance is within the pair residual's.
+double cheb_sigma(const GridDev& G) {
     const double dl = 2.0 * (G.cx + G.cy);
-    const double sig = dl > 0.0 ? G.c0 / dl : 0.0;
-    return sig > 1.0 && kChebMaxIt * std::acosh(sig) >= std::acosh(1.0 / kChebWorst);
+    return dl > 0.0 ? G.c0 / dl : 0.0;
+}
+bool cheb_ok(const GridDev& G) {
+    const double sig = cheb_sigma(G);
+    return sig > 1.0 && kChebMaxIt * std::acosh(sig) >= std::acosh(1.0 / kChebWorst) && G.rtol >= kChebRtolMin;
+}
+
+}  // namespace
+
+size_t coop_smem(const CoopSolve& cs) {
+    return (cs.cheb ? window_floats(cs.tile_y) * sizeof(float) : 0) +
+           (cs.cg_any ? 2 * (size_t)cs.nchunks * sizeof(double) : 0);
 }
 
 int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std::string& err) {
     coop_free(cs);
     if (ngrids > kCoopMaxGrids) return PIC_EINVAL;  // the caller keeps the WHILE-node solve
-    for (int g = 0; g < ngrids; g++)
-        if (hg[g].nx % 4) return PIC_EINVAL;  // quads of 4 cells along x
+    std::vector<double> tk((size_t)ngrids * (kChebMaxIt + 1), 0.0);
+    cs->vec = 1;
+    for (int g = 0; g < ngrids; g++) {
+        if (hg[g].nx % 4) cs->vec = 0;  // no quads of 4 cells along x
+        double* T = tk.data() + (size_t)g * (kChebMaxIt + 1);
+        if (cg_inner || !cheb_ok(hg[g])) {
+            cs->cg_any = 1;
+            continue;
+        }
+        cs->cheb = 1;
+        T[0] = 1.0;
+        const double ash = std::acosh((double)(float)cheb_sigma(hg[g]));
+        for (int k = 1; k <= kChebMaxIt; k++) T[k] = std::cosh(k * ash);
+    }
+    if (!cs->vec && cs->cg_any) {  // the CG's passes run on quads
+        *cs = CoopSolve{};
+        return PIC_EINVAL;
+    }
     std::vector<int2> gc(ngrids);
     std::vector<int> cg;
-    std::vector<int> tg;
-    std::vector<int2> txy;
     for (int g = 0; g < ngrids; g++) {
         const int n = (hg[g].ncell + kChunkCells - 1) / kChunkCells;
         gc[g] = make_int2((int)cg.size(), n);
         cg.insert(cg.end(), n, g);
-        for (int y = 0; y < hg[g].ny; y += kChebTileY)
-            for (int x = 0; x < hg[g].nx; x += kChebTileX) {
-                tg.push_back(g);
-                txy.push_back(make_int2(x, y));
-            }
     }
+    if ((int)cg.size() > kCoopMaxChunks) {
+        *cs = CoopSolve{};
+        return PIC_EINVAL;
+    }
+    cs->nchunks = (int)cg.size();
     int dev = 0, nsm = 0, occ = 0, coop = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if ((int)cg.size() > kCoopMaxChunks) return PIC_EINVAL;
-    cs->nchunks = (int)cg.size();
-    cs->cg_inner = cg_inner ? 1 : 0;
-    cs->cheb = 0;
-    for (int g = 0; g < ngrids && !cg_inner; g++) cs->cheb |= cheb_ok(hg[g]) ? 1 : 0;
+    // tile height: the rounds of items (three components of every tile) over two CTAs per SM,
+    // times a strip's rows and the loads and the x update, worth about six rows (the 2048 x
+    // 512 solve spends 0.4 us per row and 2 us on those in each round)
+    std::vector<int> tg;
+    std::vector<int2> txy;
+    double best = 0.0;
+    for (int ty : {64, 32, 16}) {
+        if (ty < 64 && cs->cg_any) break;
+        long long tiles = 0;
+        for (int g = 0; g < ngrids; g++)
+            tiles += (long long)((hg[g].nx + kChebTileX - 1) / kChebTileX) * ((hg[g].ny + ty - 1) / ty);
+        const double cost = std::ceil(3.0 * tiles / (2.0 * std::max(nsm, 1))) * ((ty + 2 * kChebHalo) / kChebStrips + 6);
+        if (cs->tile_y == 0 || cost < best) {
+            best = cost;
+            cs->tile_y = ty;
+        }
+    }
+    for (int g = 0; g < ngrids; g++)
+        for (int y = 0; y < hg[g].ny; y += cs->tile_y)
+            for (int x = 0; x < hg[g].nx; x += kChebTileX) {
+                tg.push_back(g);
+                txy.push_back(make_int2(x, y));
+            }
+    // the pair residual one component at a time while that leaves no CTA two items
+    cs->rsplit = 3 * cs->nchunks <= 2 * nsm ? 3 : 1;
     const size_t smem = coop_smem(*cs);
-    const auto kern = cs->cheb ? k_mp_coop<true> : k_mp_coop<false>;
+    const CoopKernel kern = coop_kernel(*cs);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kCoopThreads, smem);
     if (e == cudaSuccess && (!coop || occ < 1)) {
@@ -1056,13 +1318,15 @@ int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std
     if (e == cudaSuccess) e = cudaMalloc(&cs->chunk_grid, cg.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&cs->tile_grid, tg.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&cs->tile_xy, txy.size() * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMalloc(&cs->part, 4 * cg.size() * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&cs->bar, kBarWords * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMalloc(&cs->part, (4 + 6) * cg.size() * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&cs->cheb_t, tk.size() * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&cs->bar, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemcpy(cs->gchunk, gc.data(), ngrids * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(cs->chunk_grid, cg.data(), cg.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(cs->tile_grid, tg.data(), tg.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(cs->tile_xy, txy.data(), txy.size() * sizeof(int2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(cs->bar, 0, kBarWords * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemcpy(cs->cheb_t, tk.data(), tk.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(cs->bar, 0, sizeof(unsigned int));
     if (e != cudaSuccess) {
         err = std::string("cooperative solve set-up failed: ") + cudaGetErrorString(e);
         cudaGetLastError();
@@ -1073,13 +1337,13 @@ int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std
     cs->ntiles = (int)tg.size();
     // enough CTAs for the chunks (and the Chebyshev tiles' three components), no more
     // than are resident at once
-    const int items = cs->cheb ? std::max(cs->nchunks, 3 * cs->ntiles) : cs->nchunks;
+    const int items = cs->cheb ? std::max(cs->rsplit * cs->nchunks, 3 * cs->ntiles) : cs->nchunks;
     cs->nblocks = std::max(1, std::min(items, occ * nsm));
     return PIC_OK;
 }
 
 void coop_free(CoopSolve* cs) {
-    void* ps[] = {cs->gchunk, cs->chunk_grid, cs->tile_grid, cs->tile_xy, cs->part, cs->bar};
+    void* ps[] = {cs->gchunk, cs->chunk_grid, cs->tile_grid, cs->tile_xy, cs->part, cs->cheb_t, cs->bar};
     for (void* p : ps)
         if (p) cudaFree(p);
     *cs = CoopSolve{};
@@ -1106,6 +1370,9 @@ cudaError_t launch_mp_coop(const CoopSolve& cs, const FieldArgs& f, cudaStream_t
     a.q32 = f.q32;
     a.e32 = f.e32;
     a.part = cs.part;
+    a.part_dw = cs.part + 4 * (size_t)cs.nchunks;
+    a.cheb_t = cs.cheb_t;
+    a.rsplit = cs.rsplit;
     a.bar = cs.bar;
     a.cg = f.cg;
     a.st = f.st;
@@ -1119,11 +1386,8 @@ cudaError_t launch_mp_coop(const CoopSolve& cs, const FieldArgs& f, cudaStream_t
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    // barrier counters from zero on every launch (a launch that gave up on a barrier
-    // leaves arrivals behind)
-    cudaError_t e = cudaMemsetAsync(cs.bar, 0, kBarWords * sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
-    return cs.cheb ? cudaLaunchKernelEx(&cfg, k_mp_coop<true>, a) : cudaLaunchKernelEx(&cfg, k_mp_coop<false>, a);
+    // (the right-hand side's kernel zeroed the barrier's counter)
+    return cudaLaunchKernelEx(&cfg, coop_kernel(cs), a);
 }
 
 }  // namespace pic
