@@ -760,6 +760,56 @@ __global__ void k_fix_to_f64(long long n, const long long* a, double jinv, doubl
     if (k < n) b[k] = (double)a[k] * jinv;
 }
 
+// Gauss's law on the nodes: the charge, and the residual div E - 4 pi rho (off the wall
+// column with walls, where the conductor holds the surface charge) as its largest magnitude
+// and its sum of squares; per block into part[0..nb), [nb..2nb), [2nb..3nb).
+__global__ void __launch_bounds__(256) k_gauss(GridDev G, const double* __restrict__ rho, const double* __restrict__ ex,
+                                               const double* __restrict__ ey, double* part) {
+    __shared__ double s_v[3][256];
+    double q = 0.0, mx = 0.0, ss = 0.0;
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < G.ncell; k += gridDim.x * 256) {
+        const int j = k / G.nx, i = k - j * G.nx;
+        q += rho[k] * G.dx * G.dy;
+        if (G.walls && i == 0) continue;
+        const double exw = ex[i == 0 ? k + G.nx - 1 : k - 1];
+        const double eys = ey[j == 0 ? k + (G.ny - 1) * G.nx : k - G.nx];
+        const double r = (ex[k] - exw) * G.idx + (ey[k] - eys) * G.idy - 4.0 * kPi * rho[k];
+        mx = fmax(mx, fabs(r));
+        ss += r * r;
+    }
+    s_v[0][threadIdx.x] = q;
+    s_v[1][threadIdx.x] = mx;
+    s_v[2][threadIdx.x] = ss;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const double sq = warp_of_block_sum(s_v[0]), s2 = warp_of_block_sum(s_v[2]);
+    double m = 0.0;
+    for (int u = 0; u < 8; u++) m = fmax(m, s_v[1][threadIdx.x + 32 * u]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = sq;
+        part[gridDim.x + blockIdx.x] = m;
+        part[2 * gridDim.x + blockIdx.x] = s2;
+    }
+}
+
+// The blocks' partials (at most 256 of each) in a fixed order.
+__global__ void __launch_bounds__(256) k_gauss_end(int nb, const double* __restrict__ part, double* out) {
+    __shared__ double s_v[3][256];
+    for (int c = 0; c < 3; c++) s_v[c][threadIdx.x] = (int)threadIdx.x < nb ? part[c * nb + threadIdx.x] : 0.0;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const double sq = warp_of_block_sum(s_v[0]), s2 = warp_of_block_sum(s_v[2]);
+    double m = 0.0;
+    for (int u = 0; u < 8; u++) m = fmax(m, s_v[1][threadIdx.x + 32 * u]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) {
+        out[0] = sq;
+        out[1] = m;
+        out[2] = s2;
+    }
+}
+
 // Map device status counters that changed since the last check to a return code.
 int device_errors(pic_sim* s, const DevStatus& hs) {
     int rc = PIC_OK;
@@ -1320,9 +1370,10 @@ int pic_profile(pic_sim* s, int32_t n, double* out, int32_t n_out) {
 
 namespace {
 
-// Device pointer to grid quantity `which` of the selected simulation (J, rho: converted
-// into s->tmp).
-int field_source(pic_sim* s, int32_t which, const double** out_src) {
+// Device pointer to grid quantity `which` of the selected simulation (J, rho: formed in
+// `work`, ncell values, default s->tmp).
+int field_source(pic_sim* s, int32_t which, const double** out_src, double* work = nullptr) {
+    if (!work) work = s->tmp;
     if (which < PIC_EX || which > PIC_DENSITY_E) return fail(s, PIC_EINVAL, "which must be PIC_EX..PIC_DENSITY_E");
     if (which >= PIC_RHSX && which <= PIC_RHSZ && !s->bvec)
         return fail(s, PIC_ESTATE, "the right-hand side is kept in PIC_MIXED32 only");
@@ -1337,16 +1388,16 @@ int field_source(pic_sim* s, int32_t which, const double** out_src) {
             src = s->J64 + c * s->ntot + off;
         } else {
             k_fix_to_f64<<<(unsigned)((nc + 255) / 256), 256, 0, s->stream>>>(
-                nc, s->Jfix + c * s->ntot + off, G.jinv, s->tmp);
-            src = s->tmp;
+                nc, s->Jfix + c * s->ntot + off, G.jinv, work);
+            src = work;
         }
     } else if (which <= PIC_DBZ) {
         src = s->x + (which - PIC_DBX) * s->ntot + off;
     } else if (which <= PIC_RHSZ) {
         src = s->bvec + (which - PIC_RHSX) * s->ntot + off;
     } else {
-        if (int rc = charge_density(s, s->tmp, nullptr, which)) return rc;
-        src = s->tmp;
+        if (int rc = charge_density(s, work, nullptr, which)) return rc;
+        src = work;
     }
     *out_src = src;
     return PIC_OK;
@@ -1359,9 +1410,11 @@ int pic_fields(pic_sim* s, int32_t which, double* out, size_t len) {
     cudaSetDevice(s->device);
     const long long nc = s->hgrids[s->sel].ncell;
     if (!out || len < (size_t)nc) return fail(s, PIC_EINVAL, "out must hold nx*ny values");
+    // what is formed on demand (J, the densities) goes straight into a caller's array on
+    // this device
     const double* src = nullptr;
-    if (int rc = field_source(s, which, &src)) return rc;
-    CK(cudaMemcpyAsync(out, src, nc * sizeof(double), cudaMemcpyDefault, s->stream));
+    if (int rc = field_source(s, which, &src, which >= PIC_JX && on_device(s, out) ? out : nullptr)) return rc;
+    if (src != out) CK(cudaMemcpyAsync(out, src, nc * sizeof(double), cudaMemcpyDefault, s->stream));
     return finish_call(s);
 }
 
@@ -1374,14 +1427,12 @@ int pic_spectrum(pic_sim* s, int32_t which, double* out, size_t len) {
     const double* src = nullptr;
     if (int rc = field_source(s, which, &src)) return rc;
     double* dout = nullptr;
-    CK(dalloc(&dout, nc));
+    CK(temp_alloc((void**)&dout, nc * sizeof(double), s->stream));
     int rc = spectrum_2d(src, G.nx, G.ny, dout, s->stream, s->err);
-    if (rc == PIC_OK) {
-        cudaError_t e = cudaMemcpyAsync(out, dout, nc * sizeof(double), cudaMemcpyDefault, s->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-        if (e != cudaSuccess) rc = fail(s, PIC_ECUDA, std::string("pic_spectrum: ") + cudaGetErrorString(e));
-    }
-    cudaFree(dout);
+    cudaError_t e = cudaSuccess;
+    if (rc == PIC_OK) e = cudaMemcpyAsync(out, dout, nc * sizeof(double), cudaMemcpyDefault, s->stream);
+    temp_free(dout, s->stream);
+    if (e != cudaSuccess) rc = fail(s, PIC_ECUDA, std::string("pic_spectrum: ") + cudaGetErrorString(e));
     if (rc) return rc;
     return finish_call(s);
 }
@@ -1481,43 +1532,26 @@ int pic_conservation(pic_sim* s, double* out, int32_t n_out) {
     cudaSetDevice(s->device);
     if (!out || n_out < 1) return fail(s, PIC_EINVAL, "out is NULL");
     const GridDev& G = s->hgrids[s->sel];
-    double* mom = nullptr;
-    CK(dalloc(&mom, 3));
-    CK(cudaMemsetAsync(mom, 0, 3 * sizeof(double), s->stream));
-    int rc = charge_density(s, s->tmp, mom);
-    const long long nc = G.ncell;
-    std::vector<double> rho(nc), ex(nc), ey(nc);
-    double hm[3] = {0, 0, 0};
-    if (rc == PIC_OK) {
-        cudaError_t e = cudaMemcpyAsync(rho.data(), s->tmp, nc * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ex.data(), s->F + G.cell_off, nc * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ey.data(), s->F + s->ntot + G.cell_off, nc * sizeof(double), cudaMemcpyDeviceToHost,
-                                s->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hm, mom, sizeof hm, cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-        if (e != cudaSuccess) rc = fail(s, PIC_ECUDA, std::string("pic_conservation: ") + cudaGetErrorString(e));
+    // results (momentum, charge, max and sum of squares of the residual), block partials
+    const int nb = (int)std::min<long long>(152, (G.ncell + 255) / 256);
+    double* d = nullptr;
+    CK(temp_alloc((void**)&d, (6 + 3 * (size_t)nb) * sizeof(double), s->stream));
+    cudaError_t e = cudaMemsetAsync(d, 0, 3 * sizeof(double), s->stream);
+    int rc = PIC_OK;
+    double h[6] = {0, 0, 0, 0, 0, 0};
+    if (e == cudaSuccess) rc = charge_density(s, s->tmp, d);
+    if (e == cudaSuccess && rc == PIC_OK) {
+        k_gauss<<<nb, 256, 0, s->stream>>>(G, s->tmp, s->F + G.cell_off, s->F + s->ntot + G.cell_off, d + 6);
+        k_gauss_end<<<1, 256, 0, s->stream>>>(nb, d + 6, d + 3);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, s->stream);
     }
-    cudaFree(mom);
+    temp_free(d, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return fail(s, PIC_ECUDA, std::string("pic_conservation: ") + cudaGetErrorString(e));
     if (rc) return rc;
-    // Gauss's law on the nodes: div E - 4 pi rho (off the wall column with walls, where
-    // the conductor holds the surface charge)
-    double q = 0.0, mx = 0.0, ss = 0.0;
-    long long cnt = 0;
-    for (int j = 0; j < G.ny; j++)
-        for (int i = 0; i < G.nx; i++) {
-            const long long k = (long long)j * G.nx + i;
-            q += rho[k] * G.dx * G.dy;
-            if (G.walls && i == 0) continue;
-            const double exw = ex[(long long)j * G.nx + (i == 0 ? G.nx - 1 : i - 1)];
-            const double eys = ey[(long long)(j == 0 ? G.ny - 1 : j - 1) * G.nx + i];
-            const double r = (ex[k] - exw) * G.idx + (ey[k] - eys) * G.idy - 4.0 * kPi * rho[k];
-            mx = std::max(mx, std::fabs(r));
-            ss += r * r;
-            cnt++;
-        }
-    const double vals[6] = {hm[0], hm[1], hm[2], q, mx, cnt ? std::sqrt(ss / cnt) : 0.0};
+    const long long cnt = G.ncell - (G.walls ? G.ny : 0);
+    const double vals[6] = {h[0], h[1], h[2], h[3], h[4], cnt ? std::sqrt(h[5] / cnt) : 0.0};
     for (int k = 0; k < n_out && k < 6; k++) out[k] = vals[k];
     return PIC_OK;
 }

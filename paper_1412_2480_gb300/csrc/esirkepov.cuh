@@ -138,21 +138,52 @@ __device__ __forceinline__ void esirkepov(int i0, R f0x, int j0, R f0y, int i1, 
 // cell/fraction (i + fx, j + fy): rho(node) += q W_p(x - node) W_p(y - node) on the
 // integer lattice. With walls the part beyond a wall folds back as the mirror image's
 // (even); the unstored wall node x = nx is dropped.
+// The FP64 pipe bounds it (two lanes per cycle and SM): one product per row and one per
+// node, the comparison with 1/2 is the high word's, the order-2 weights go without their
+// factor 1/2 (the caller's q carries the 1/4, exact either way), and the walls' images have
+// a loop of their own (as selects inside one loop they brought every product twice: 44 FP64
+// instructions per warp and particle instead of 28).
+template <int P>
+__device__ __forceinline__ void rho_weights(int i, double f, int& base, double w[P + 1]) {
+    if constexpr (P == 2) {
+        const bool up = __double2hiint(f) >= 0x3FE00000;  // f >= 1/2 (f >= 0)
+        const double d = up ? f - 1.0 : f, hm = 0.5 - d, hp = 0.5 + d;
+        base = up ? i : i - 1;
+        w[0] = hm * hm;
+        w[1] = fma(-2.0 * d, d, 1.5);
+        w[2] = hp * hp;
+    } else {
+        shape_nodes<P, double>(i, f, base, w);
+    }
+}
+
 template <int P>
 __device__ __forceinline__ void deposit_rho(const GridDev& G, int i, double fx, int j, double fy, double q,
                                             double* rho) {
     int bx, by;
     double wx[P + 1], wy[P + 1];
-    shape_nodes<P, double>(i, fx, bx, wx);
-    shape_nodes<P, double>(j, fy, by, wy);
+    rho_weights<P>(i, fx, bx, wx);
+    rho_weights<P>(j, fy, by, wy);
+    if (P == 2) q *= 0.25;
+    if (!G.walls) {
+#pragma unroll
+        for (int b = 0; b <= P; b++) {
+            double* row = rho + (long long)wrapi(by + b, G.ny) * G.nx;
+            const double qy = q * wy[b];
+#pragma unroll
+            for (int a = 0; a <= P; a++) atomicAdd(row + wrapi(bx + a, G.nx), qy * wx[a]);
+        }
+        return;
+    }
 #pragma unroll
     for (int b = 0; b <= P; b++) {
         double* row = rho + (long long)wrapi(by + b, G.ny) * G.nx;
+        const double qy = q * wy[b];
 #pragma unroll
         for (int a = 0; a <= P; a++) {
-            int s = 1, col = wrapi(bx + a, G.nx);
-            if (G.walls) col = wall_col(bx + a, G.nx, false, false, s);
-            if (s) atomicAdd(row + col, s * q * wx[a] * wy[b]);
+            int s;
+            const int col = wall_col(bx + a, G.nx, false, false, s);
+            if (s) atomicAdd(row + col, qy * wx[a]);  // (an even quantity: s is 0 or 1)
         }
     }
 }

@@ -990,27 +990,70 @@ __global__ void k_gather_overflow(long long n_over, int gs, Slots O, long long b
     to_staging(O.p, k, S, d);
 }
 
+// Node density (q[s] per particle, 0: species left out) and w times the total momentum
+// straight from the bins: a block takes part `blockIdx.y` of the particles of one (tile,
+// species), all nine segments (one block row more: the overflow list). The particles are
+// read once, in the bins' order of 32 distinct cells per warp, so the atomics of a warp
+// fall on neighbouring nodes. rho, mom: null where not asked for.
+struct DensityArgs {
+    double q[2], w;
+    double *rho, *mom;
+};
+
 template <int P>
-__global__ void k_rho_staged(long long n, GridDev G, PartArrays S, double q, double* rho) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int c = S.cij[k];
-    deposit_rho<P>(G, c & 0xffff, (double)S.ox[k], c >> 16, (double)S.oy[k], q, rho);
+__device__ __forceinline__ void density_one(const GridDev& G, const unsigned* B, long long k, double q, double* rho,
+                                            double* mom, double m[3]) {
+    const float* F = reinterpret_cast<const float*>(B);
+    if (rho) {
+        const int c = (int)__ldcs(B + aos(k, 0));
+        deposit_rho<P>(G, c & 0xffff, (double)__ldcs(F + aos(k, 1)), c >> 16, (double)__ldcs(F + aos(k, 2)), q, rho);
+    }
+    if (mom)
+#pragma unroll
+        for (int a = 0; a < 3; a++) m[a] += (double)__ldcs(F + aos(k, 3 + a));
 }
 
-__global__ void k_momentum_staged(long long n, PartArrays S, double w, double* out) {
-    __shared__ double red[32];
-    double s[3] = {0.0, 0.0, 0.0};
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        s[0] += S.ux[k];
-        s[1] += S.uy[k];
-        s[2] += S.uz[k];
+template <int P>
+__global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int nbins, const DensityArgs d) {
+    __shared__ double s_m[3][256];
+    const GridDev& G = a.grids[g];
+    const DevStatus* st = a.st;
+    const int par = (int)st->parity;
+    const int tid = threadIdx.x;
+    double m[3] = {0.0, 0.0, 0.0};
+    if ((int)blockIdx.x < nbins) {
+        // (species by halves of the grid: with alternating ones a species left out would
+        // idle every other SM)
+        const int s = (int)blockIdx.x >= G.ntiles ? 1 : 0;
+        const long long bin = 2ll * ((int)blockIdx.x - s * G.ntiles) + s;
+        const double q = s ? d.q[1] : d.q[0];
+        double* rho = q != 0.0 ? d.rho : nullptr;
+        if (!(d.mom || rho)) return;
+        const unsigned* B = par ? a.buf[1] : a.buf[0];
+        const int* cnt = (par ? a.cnt[1] : a.cnt[0]) + ((long long)G.tile_first * 2 + bin) * kSegs;
+        long long base = G.bin_off + bin * bin_stride(G);
+        for (int k = 0; k < kSegs; k++) {
+            const int lim = (int)(k == 0 ? G.cap : G.capo), n = min(cnt[k], lim);
+            for (int v = (int)blockIdx.y * 256 + tid; v < n; v += (int)gridDim.y * 256)
+                density_one<P>(G, B, base + v, q, rho, d.mom, m);
+            base += lim;
+        }
+    } else {
+        const Slots O = par ? a.ovf[1] : a.ovf[0];
+        const long long n = min((long long)st->ovf_count[par], a.ovf_cap);
+        for (long long k = (long long)blockIdx.y * 256 + tid; k < n; k += (long long)gridDim.y * 256) {
+            const int gs = O.gs[k];
+            const double q = gs & 1 ? d.q[1] : d.q[0];
+            if (gs >> 1 == g) density_one<P>(G, O.p, k, q, q != 0.0 ? d.rho : nullptr, d.mom, m);
+        }
     }
-    for (int c = 0; c < 3; c++) {
-        const double t = block_sum(s[c], red);
-        if (threadIdx.x == 0) atomicAdd(out + c, w * t);
-        __syncthreads();
-    }
+    if (!d.mom) return;
+#pragma unroll
+    for (int c = 0; c < 3; c++) s_m[c][tid] = m[c];
+    __syncthreads();
+    if (tid >= 96) return;
+    const double t = warp_of_block_sum(s_m[tid >> 5]);
+    if ((tid & 31) == 0 && t != 0.0) atomicAdd(d.mom + (tid >> 5), d.w * t);
 }
 
 __global__ void k_unstage(long long n, GridDev G, PartArrays S, double* out) {
@@ -1719,29 +1762,19 @@ long long mixed_count(MixedState* m, int g, int s) { return m->n[2 * g + s]; }
 
 int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, double* mom, cudaStream_t st,
                        std::string& err) {
-    DevStatus hs{};
-    if (int rc = read_status(m, hs, st, err)) return rc;
     const GridDev& G = m->G[g];
-    for (int s = 0; s < 2; s++) {
-        PartArrays S{};
-        long long n = 0;
-        if (int rc = gather_species(m, g, (int)hs.parity, s, S, n, st, err)) return rc;
-        if (n && rho && q_s[s] != 0.0) {
-            const double q = q_s[s];
-            switch (G.order) {
-            case 1: k_rho_staged<1><<<grid1(n), 256, 0, st>>>(n, G, S, q, rho); break;
-            case 2: k_rho_staged<2><<<grid1(n), 256, 0, st>>>(n, G, S, q, rho); break;
-            default: k_rho_staged<3><<<grid1(n), 256, 0, st>>>(n, G, S, q, rho); break;
-            }
-        }
-        if (n && mom) k_momentum_staged<<<304, 256, 0, st>>>(n, S, G.w, mom);
-        const cudaError_t e = cudaStreamSynchronize(st);
-        free_parts(S, st);
-        if (e != cudaSuccess) {
-            err = std::string("diagnostics: ") + cudaGetErrorString(e);
-            return PIC_ECUDA;
-        }
+    const DensityArgs d{{q_s[0], q_s[1]}, G.w, rho, mom};
+    const int nbins = 2 * G.ntiles;
+    // about 1024 particles per block (a bin's share of its capacity): with whole bins of 8192
+    // the few blocks of an SM more or less left a third of the device idle
+    const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / 1280)));
+    const MixedArgs a = make_args(m, 0);
+    switch (G.order) {
+    case 1: k_density<1><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
+    case 2: k_density<2><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
+    default: k_density<3><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
     }
+    MCK(cudaGetLastError());
     return PIC_OK;
 }
 long long mixed_rebins(MixedState* m) { return m->rebins; }
