@@ -49,8 +49,9 @@ struct pic_cnn {
     pic::CnnImg* imgs = nullptr;
     int* tile_img = nullptr;
     int geo_nimg = 0, geo_nx = 0, geo_ny = 0;
-    double* d_loss = nullptr;
-    unsigned int* d_err = nullptr;
+    float* part = nullptr;    // weight-gradient slices
+    double* d_loss = nullptr;       // one block of 16 bytes, read back whole: the loss,
+    unsigned int* d_err = nullptr;  // [0] a wait ran out, [1] the waits' poll limit
 };
 
 namespace pic {
@@ -78,7 +79,7 @@ constexpr long long kNParams = 896 + 2 * 9248 + 867;
 static_assert(kNParams == PIC_CNN_NPARAMS, "parameter count");
 
 constexpr int kTile = 128;  // pixels per conv CTA
-constexpr int kChunk = 64;  // pixels per weight-gradient MMA round
+constexpr int kChunk = 64;  // pixels per weight-gradient round
 
 __device__ __forceinline__ int wrapn(int k, int n) { return k < 0 ? k + n : (k >= n ? k - n : k); }
 
@@ -182,136 +183,167 @@ constexpr int conv_smem() {
     return kTile * 9 * CIN * 2 + NOUT * 9 * CIN * 2;
 }
 
-// ---- weight gradient: dW[co][tap][ci] += sum_p dY[p][co] X[nbr(p, tap)][ci] ----------
-// A = rows (tap, ci) x pixels, B = co x pixels; pixels are the reduction dimension, in
-// rounds of 64 pixels; the MT row tiles of 128 accumulate side by side in tensor memory.
+// ---- weight and bias gradients ---------------------------------------------------------
+// dW[co][tap][ci] = sum_p dY[p][co] X[nbr(p, tap)][ci], all four layers in one launch: A =
+// rows (tap, ci) x pixels, B = co x pixels, pixels are the reduction dimension. Both X and
+// dY hold a pixel's channels side by side, which is the MN-major operand layout, so the
+// im2col moves 16-byte vectors (as K-major operands every value was a 2-byte store, and one
+// layer took 64 us on 32 CTAs). One more row of A is constant 1: its sums are the bias
+// gradient. A CTA takes its share of one layer's 64-pixel chunks, the fill of one buffer
+// under the MMAs of the other, and leaves its sums in its own slice of `part`; k_finish adds
+// the slices in a fixed order, so gradients are the same on every run.
+// 8 images of 64 x 64, all layers with biases and Adam: 275 -> 32 us (k_wgrad 25, k_finish 7).
+constexpr int kWThreads = 256;
+constexpr int kWPerLayer = 76;  // CTAs per layer: two per SM over the four layers
+
+template <int CIN, int NOUT>
+struct WShape {
+    static constexpr int kRows = 9 * CIN + 1;  // (tap, ci), then the constant
+    static constexpr int kMT = (kRows + 127) / 128;
+    static constexpr int kABytes = kMT * 128 * kChunk * 2;
+    static constexpr int kBBytes = NOUT * kChunk * 2;
+    static constexpr int kSlice = kRows * NOUT;
+};
+constexpr int kWSmem = 2 * (WShape<32, 32>::kABytes + WShape<32, 32>::kBBytes);
+constexpr int kWSlice = WShape<32, 32>::kSlice;  // the largest layer's; every slice's pitch
+constexpr uint32_t kWCols = 128;                 // tensor-memory columns: three row tiles of 32
+
 struct WgradArgs {
     const CnnImg* imgs;
     const int* tile_img;
-    const bf16* X;    // [P][CIN]
-    const bf16* dY;   // [P][NOUT]
-    float* dW;        // this layer's W[cout][9][cin] gradient
-    int cin, cout;    // real channel counts
+    const bf16* X[4];   // [P][CIN] of each layer
+    const bf16* dY[4];  // [P][NOUT]
+    float* part;        // [4][kWPerLayer][kWSlice]
     long long nchunks;
-    int chunks_per_cta;
+    int ctas;           // CTAs per layer
     unsigned int* err;
 };
 
 template <int CIN, int NOUT>
-__global__ void __launch_bounds__(128) k_wgrad(const WgradArgs a) {
-    constexpr int ROWS = 9 * CIN;
-    constexpr int MT = (ROWS + 127) / 128;
-    constexpr int ABYTES = MT * 128 * kChunk * 2;
+__device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int cta, unsigned char* smem, uint64_t* bar,
+                                            uint32_t tmem) {
+    using S = WShape<CIN, NOUT>;
     constexpr uint32_t SBO = (kChunk / 8) * 128;
-    constexpr uint32_t NCOLS = MT * NOUT <= 32 ? 32 : (MT * NOUT <= 64 ? 64 : 128);
-    extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char* sA = smem;
-    unsigned char* sB = smem + ABYTES;
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t s_tmem;
+    constexpr int BUF = S::kABytes + S::kBBytes;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (warp == 0) tc::tmem_alloc(&s_tmem, NCOLS);
-    if (tid == 0) tc::mbar_init(&bar, 1);
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = s_tmem;
-    const long long c0 = (long long)blockIdx.x * a.chunks_per_cta;
-    const long long c1 = min(a.nchunks, c0 + a.chunks_per_cta);
+    const bf16* X = a.X[layer];
+    const bf16* dY = a.dY[layer];
     const uint32_t lim = __ldg(a.err + 1);  // the waits' poll limit (0: the default bound)
+    // the constant row and the unused ones behind it
+    for (int q = tid; q < 2 * (S::kMT * 16 - 9 * CIN / 8) * kChunk; q += kWThreads) {
+        const int b = q & 1, px = (q >> 1) % kChunk, g = 9 * CIN / 8 + (q >> 1) / kChunk;
+        *reinterpret_cast<uint4*>(smem + b * BUF + tc::mn_offset(8 * g, px, kChunk)) =
+            make_uint4(g == 9 * CIN / 8 ? 0x3F80u : 0u, 0u, 0u, 0u);  // BF16 1.0 in row 9 CIN
+    }
     bool ok = true;
-    for (long long c = c0; c < c1; c++) {
-        const int q = (int)(c - c0);
-        if (q > 0) ok = __syncthreads_and((ok && tc::mbar_wait_lim(&bar, (uint32_t)((q - 1) & 1), lim)) ? 1 : 0) != 0;
-        if (!ok) {  // drain the round in flight before the shared and tensor memory go
-            if (tid == 0) tc::mbar_wait(&bar, (uint32_t)((q - 1) & 1));
-            break;
-        }
+    int n = 0;  // chunks issued
+    for (long long c = cta; c < a.nchunks; c += a.ctas, n++) {
+        const int b = n & 1;
+        unsigned char* sA = smem + b * BUF;
+        unsigned char* sB = sA + S::kABytes;
+        if (n >= 2) ok = __syncthreads_and(tc::mbar_wait_lim(bar + b, (uint32_t)((n / 2 - 1) & 1), lim) ? 1 : 0) != 0;
+        if (!ok) break;
         const long long pix0 = c * kChunk;
         const CnnImg im = a.imgs[a.tile_img[pix0 / kTile]];
-        for (int idx = tid; idx < kChunk * 9; idx += 128) {
-            const int px = idx % kChunk, tap = idx / kChunk;
-            const long long l = pix0 + px - im.off;
-            const int j = (int)(l / im.nx), i = (int)(l - (long long)j * im.nx);
+        const int l0 = (int)(pix0 - im.off);
+        constexpr int VX = CIN / 8, VY = NOUT / 8;
+#pragma unroll
+        for (int q0 = 0; q0 < kChunk * 9 * VX; q0 += kWThreads) {
+            const int q = q0 + tid;  // vectors of a pixel side by side, then pixels, then taps
+            if (kChunk * 9 * VX % kWThreads != 0 && q >= kChunk * 9 * VX) break;
+            const int v = q % VX, px = q / VX % kChunk, tap = q / (VX * kChunk);
+            const int l = l0 + px, j = l / im.nx, i = l - j * im.nx;
             const int ni = wrapn(i + tap % 3 - 1, im.nx), nj = wrapn(j + tap / 3 - 1, im.ny);
-            const uint4* src = reinterpret_cast<const uint4*>(a.X + (im.off + (long long)nj * im.nx + ni) * CIN);
-#pragma unroll
-            for (int k8 = 0; k8 < CIN / 8; k8++) {
-                const uint4 v = __ldg(src + k8);
-                const uint16_t* e = reinterpret_cast<const uint16_t*>(&v);
-#pragma unroll
-                for (int t = 0; t < 8; t++)
-                    *reinterpret_cast<uint16_t*>(sA + tc::canon_offset(tap * CIN + k8 * 8 + t, px, kChunk)) = e[t];
-            }
+            *reinterpret_cast<uint4*>(sA + tc::mn_offset(tap * CIN + 8 * v, px, kChunk)) =
+                __ldg(reinterpret_cast<const uint4*>(X + (im.off + (long long)nj * im.nx + ni) * CIN) + v);
         }
-        for (int idx = tid; idx < kChunk * (NOUT / 8); idx += 128) {
-            const int px = idx / (NOUT / 8), c8 = idx % (NOUT / 8);
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.dY + (pix0 + px) * NOUT) + c8);
-            const uint16_t* e = reinterpret_cast<const uint16_t*>(&v);
-#pragma unroll
-            for (int t = 0; t < 8; t++)
-                *reinterpret_cast<uint16_t*>(sB + tc::canon_offset(c8 * 8 + t, px, kChunk)) = e[t];
+        for (int q = tid; q < kChunk * VY; q += kWThreads) {
+            const int v = q % VY, px = q / VY;
+            *reinterpret_cast<uint4*>(sB + tc::mn_offset(8 * v, px, kChunk)) =
+                __ldg(reinterpret_cast<const uint4*>(dY + (pix0 + px) * NOUT) + v);
         }
         tc::fence_smem_to_async();
         __syncthreads();
         if (tid == 0) {
             tc::fence_after_sync();
-            const uint32_t idesc = tc::make_idesc(128, NOUT);
+            const uint32_t idesc = tc::make_idesc_mn(128, NOUT);
             const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB);
 #pragma unroll 1
-            for (int m = 0; m < MT; m++)
-#pragma unroll 1
+            for (int m = 0; m < S::kMT; m++)
+#pragma unroll
                 for (int s = 0; s < kChunk / 16; s++)
                     tc::mma_bf16(tmem + (uint32_t)(m * NOUT),
                                  tc::make_desc(a0 + (uint32_t)m * 128u * kChunk * 2u + s * 256, tc::kLbo, SBO),
-                                 tc::make_desc(b0 + s * 256, tc::kLbo, SBO), idesc, (q > 0 || s > 0) ? 1u : 0u);
-            tc::mma_commit(&bar);
+                                 tc::make_desc(b0 + s * 256, tc::kLbo, SBO), idesc, (n > 0 || s > 0) ? 1u : 0u);
+            tc::mma_commit(bar + b);
         }
     }
-    const int nq = (int)(c1 - c0);
-    if (ok && nq > 0) {
-        ok = __syncthreads_and(tc::mbar_wait_lim(&bar, (uint32_t)((nq - 1) & 1), lim) ? 1 : 0) != 0;
-        if (!ok && tid == 0) tc::mbar_wait(&bar, (uint32_t)((nq - 1) & 1));  // drain
+    // the last commit of each buffer
+    if (ok) {
+        bool w = true;
+        for (int b = 0; b < 2 && b < n; b++)
+            w = tc::mbar_wait_lim(bar + b, (uint32_t)(((n - 1 - b) / 2) & 1), lim) && w;
+        ok = __syncthreads_and(w ? 1 : 0) != 0;
+    }
+    if (!ok) {  // drain what is in flight before the shared and tensor memory go
+        if (tid == 0) {
+            for (int b = 0; b < 2 && b < n; b++) tc::mbar_wait(bar + b, (uint32_t)(((n - 1 - b) / 2) & 1));
+            atomicExch(a.err, 1u);
+        }
+        return;
     }
     tc::fence_after_sync();
-    if (ok && nq > 0) {
+    if (warp >= 4) return;
+    float* out = a.part + ((size_t)layer * kWPerLayer + cta) * kWSlice;
 #pragma unroll 1
-        for (int m = 0; m < MT; m++) {
-            float acc[NOUT];
+    for (int m = 0; m < S::kMT; m++) {
+        float acc[NOUT];
 #pragma unroll
-            for (int cc = 0; cc < NOUT; cc += 16)
-                tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(m * NOUT + cc), acc + cc);
-            const int row = m * 128 + warp * 32 + lane;
-            if (row < ROWS) {
-                const int tap = row / CIN, ci = row % CIN;
-                if (ci < a.cin) {
+        for (int cc = 0; cc < NOUT; cc += 16)
+            tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(m * NOUT + cc), acc + cc);
+        const int row = m * 128 + warp * 32 + lane;
+        if (row < S::kRows)
 #pragma unroll
-                    for (int co = 0; co < NOUT; co++)
-                        if (co < a.cout) atomicAdd(a.dW + ((long long)co * 9 + tap) * a.cin + ci, acc[co]);
-                }
-            }
-        }
-    } else if (!ok && tid == 0) {
-        atomicExch(a.err, 1u);
+            for (int co = 0; co < NOUT; co += 4)
+                *reinterpret_cast<float4*>(out + (size_t)row * NOUT + co) =
+                    make_float4(acc[co], acc[co + 1], acc[co + 2], acc[co + 3]);
+    }
+}
+
+__global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ uint32_t s_tmem;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    if (warp == 0) tc::tmem_alloc(&s_tmem, kWCols);
+    if (tid == 0) {
+        tc::mbar_init(bar, 1);
+        tc::mbar_init(bar + 1, 1);
+    }
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
+    const int layer = blockIdx.x / a.ctas, cta = blockIdx.x - layer * a.ctas;
+    switch (layer) {
+    case 0: wgrad_layer<16, 32>(a, 0, cta, smem, bar, tmem); break;
+    case 3: wgrad_layer<32, 16>(a, 3, cta, smem, bar, tmem); break;
+    default: wgrad_layer<32, 32>(a, layer, cta, smem, bar, tmem); break;
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_free(tmem, NCOLS);
-}
-
-template <int CIN, int NOUT>
-constexpr int wgrad_smem() {
-    return ((9 * CIN + 127) / 128) * 128 * kChunk * 2 + NOUT * kChunk * 2;
+    if (warp == 0) tc::tmem_free(tmem, kWCols);
 }
 
 // ---- small kernels -------------------------------------------------------------------
 // Operand-layout BF16 weights from the FP32 parameters: forward (rows = output
 // channels, columns = (tap, input channel)) and input gradient (rows = input channels,
 // columns = (tap', output channel) with the tap mirrored).
-__global__ void k_pack(const float* __restrict__ prm, uint16_t* wf0, uint16_t* wf1, uint16_t* wf2, uint16_t* wf3,
-                       uint16_t* wd1, uint16_t* wd2, uint16_t* wd3) {
-    uint16_t* wf[4] = {wf0, wf1, wf2, wf3};
-    uint16_t* wd[4] = {nullptr, wd1, wd2, wd3};
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+struct PackArgs {
+    const float* prm;
+    uint16_t *wf[4], *wd[4];
+};
+__device__ __forceinline__ void pack_weight(const PackArgs& a, int t) {
+    const float* prm = a.prm;
     int base = 0;
     for (int L = 0; L < 4; L++) {
         const Layer y = kLd[L];
@@ -320,7 +352,7 @@ __global__ void k_pack(const float* __restrict__ prm, uint16_t* wf0, uint16_t* w
             const int e = t - base, n = e / Kf, k = e % Kf, tap = k / y.cin_pad, ci = k % y.cin_pad;
             const float v = (n < y.cout && ci < y.cin) ? prm[y.w_off + ((long long)n * 9 + tap) * y.cin + ci] : 0.f;
             const bf16 h = __float2bfloat16_rn(v);
-            wf[L][tc::canon_offset(n, k, Kf) / 2] = *reinterpret_cast<const uint16_t*>(&h);
+            a.wf[L][tc::canon_offset(n, k, Kf) / 2] = *reinterpret_cast<const uint16_t*>(&h);
         }
         base += nf;
         if (L == 0) continue;
@@ -329,7 +361,7 @@ __global__ void k_pack(const float* __restrict__ prm, uint16_t* wf0, uint16_t* w
             const int e = t - base, n = e / Kd, k = e % Kd, tp = k / y.cout_pad, co = k % y.cout_pad;
             const float v = (co < y.cout) ? prm[y.w_off + ((long long)co * 9 + (8 - tp)) * y.cin + n] : 0.f;
             const bf16 h = __float2bfloat16_rn(v);
-            wd[L][tc::canon_offset(n, k, Kd) / 2] = *reinterpret_cast<const uint16_t*>(&h);
+            a.wd[L][tc::canon_offset(n, k, Kd) / 2] = *reinterpret_cast<const uint16_t*>(&h);
         }
         base += nd;
     }
@@ -344,9 +376,17 @@ int pack_total() {
     return n;
 }
 
-// Caller planes [img][3][ny][nx] (FP32) -> BF16 [P][16].
-__global__ void k_planes_in(long long P, long long npi, const float* __restrict__ in, bf16* __restrict__ X0) {
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// The start of a call: the weights into operand layout (the first npack blocks), the
+// caller's planes [img][3][ny][nx] (FP32) -> BF16 [P][16] (the others); the loss zeroed.
+__global__ void k_begin(const PackArgs pack, int npack, int total, long long P, long long npi,
+                        const float* __restrict__ in, bf16* __restrict__ X0, double* loss) {
+    if ((int)blockIdx.x < npack) {
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        if (t == 0) *loss = 0.0;
+        if (t < total) pack_weight(pack, t);
+        return;
+    }
+    const long long p = (long long)(blockIdx.x - npack) * blockDim.x + threadIdx.x;
     if (p >= P) return;
     const long long img = p / npi, l = p - img * npi;
     __align__(16) bf16 v[16];
@@ -391,30 +431,40 @@ __global__ void k_loss(long long P, long long npi, const float* __restrict__ out
     if (threadIdx.x == 0) atomicAdd(loss, s / (double)(3 * P));
 }
 
-// db[co] += sum_p dY[p][co], co < cout.
-template <int NOUT>
-__global__ void k_bias_grad(long long P, const bf16* __restrict__ dY, int cout, float* db) {
-    __shared__ float red[32];
-    for (int co = 0; co < cout; co++) {
-        float s = 0.f;
-        for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x)
-            s += __bfloat162float(dY[p * NOUT + co]);
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) atomicAdd(db + co, s);
-        __syncthreads();
-    }
-}
+// The gradient of every parameter: its layer's slices added in order. With w, Adam's step
+// on the parameters follows in the same thread (unless a wait of the call ran out).
+struct AdamArgs {
+    float *w, *m1, *m2;
+    float lr, c1, c2;
+};
 
-__global__ void k_adam(long long n, float* w, const float* g, float* m1, float* m2, float lr, float c1, float c2) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+__global__ void k_finish(const float* __restrict__ part, int ctas, float* __restrict__ grads, const AdamArgs u,
+                         const unsigned int* err) {
+    // one thread per (row, output channel) of a layer's slice, output channels side by side
+    const int layer = blockIdx.y;
+    const Layer y = kLd[layer];
+    const int rows = 9 * y.cin_pad + 1, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= rows * y.cout_pad) return;
+    const int row = t / y.cout_pad, co = t - row * y.cout_pad, tap = row / y.cin_pad, ci = row - tap * y.cin_pad;
+    if (co >= y.cout || (tap < 9 && ci >= y.cin)) return;  // (row 9 cin_pad, tap 9: the bias)
+    const float* p = part + (size_t)layer * kWPerLayer * kWSlice + t;
+    float g = 0.f;
+    for (int c = 0; c < ctas; c += 4) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = c + k < ctas ? p[(size_t)(c + k) * kWSlice] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; k++) g += v[k];
+    }
+    const long long k = tap < 9 ? y.w_off + ((long long)co * 9 + tap) * y.cin + ci : y.b_off + co;
+    grads[k] = g;
+    if (!u.w || *err) return;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float gi = g[k];
-    const float a = b1 * m1[k] + (1.f - b1) * gi;
-    const float b = b2 * m2[k] + (1.f - b2) * gi * gi;
-    m1[k] = a;
-    m2[k] = b;
-    w[k] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+    const float a = b1 * u.m1[k] + (1.f - b1) * g;
+    const float b = b2 * u.m2[k] + (1.f - b2) * g * g;
+    u.m1[k] = a;
+    u.m2[k] = b;
+    u.w[k] -= u.lr * (a / u.c1) / (sqrtf(b / u.c2) + eps);
 }
 
 // The learned guess of the solver: x0 = K * b + bias rms(b), K the network collapsed
@@ -572,12 +622,7 @@ cudaError_t set_smem_once() {
         if (r == cudaSuccess)
             r = cudaFuncSetAttribute(k_conv<32, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      conv_smem<32, 16, true>());
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_wgrad<16, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, wgrad_smem<16, 32>());
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_wgrad<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, wgrad_smem<32, 32>());
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_wgrad<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, wgrad_smem<32, 16>());
+        if (r == cudaSuccess) r = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
         if (r == cudaSuccess)
             r = cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         return r;
@@ -590,24 +635,6 @@ void conv(long long ntiles, const CnnImg* imgs, const int* tile_img, const uint1
           const float* bias, int cout, void* Y, unsigned int* err, cudaStream_t st) {
     ConvArgs a{imgs, tile_img, reinterpret_cast<const bf16*>(X), W, bias, cout, Y, err};
     k_conv<CIN, NOUT, OUTF32><<<(unsigned)ntiles, kTile, conv_smem<CIN, NOUT, OUTF32>(), st>>>(a);
-}
-
-template <int CIN, int NOUT>
-void wgrad(long long P, const CnnImg* imgs, const int* tile_img, const uint16_t* X, const uint16_t* dY, float* dW,
-           int cin, int cout, unsigned int* err, cudaStream_t st) {
-    WgradArgs a{};
-    a.imgs = imgs;
-    a.tile_img = tile_img;
-    a.X = reinterpret_cast<const bf16*>(X);
-    a.dY = reinterpret_cast<const bf16*>(dY);
-    a.dW = dW;
-    a.cin = cin;
-    a.cout = cout;
-    a.nchunks = P / kChunk;
-    a.chunks_per_cta = 16;
-    a.err = err;
-    const long long ncta = (a.nchunks + a.chunks_per_cta - 1) / a.chunks_per_cta;
-    k_wgrad<CIN, NOUT><<<(unsigned)ncta, 128, wgrad_smem<CIN, NOUT>(), st>>>(a);
 }
 
 // The forward pass X0 -> out through buffers Xa, Xb (X1..X3 kept when keep != null).
@@ -795,55 +822,66 @@ int prepare(pic_cnn* c, int nimg, int nx, int ny) {
     return PIC_OK;
 }
 
-int pack(pic_cnn* c) {
-    k_pack<<<blocks(pack_total()), 256, 0, c->stream>>>(c->params, c->wf[0], c->wf[1], c->wf[2], c->wf[3], c->wd[1],
-                                                         c->wd[2], c->wd[3]);
+// Weights into operand layout and, with in, its P pixels into X0; the loss zeroed.
+int begin(pic_cnn* c, const float* in, long long P, long long npi) {
+    PackArgs a{c->params, {c->wf[0], c->wf[1], c->wf[2], c->wf[3]}, {nullptr, c->wd[1], c->wd[2], c->wd[3]}};
+    const unsigned np = blocks(pack_total());
+    k_begin<<<np + (in ? blocks(P) : 0), 256, 0, c->stream>>>(a, (int)np, pack_total(), in ? P : 0, npi, in,
+                                                              reinterpret_cast<bf16*>(c->X[0]), c->d_loss);
     CCK(cudaGetLastError());
     return PIC_OK;
 }
 
-int check_err(pic_cnn* c) {
-    unsigned int h = 0;
-    CCK(cudaMemcpyAsync(&h, c->d_err, sizeof h, cudaMemcpyDeviceToHost, c->stream));
+// Waits for the call's work; its loss, and whether a wait in it ran out.
+int finish(pic_cnn* c, double* loss) {
+    struct {
+        double loss;
+        unsigned int err[2];
+    } h{};
+    static_assert(sizeof h == 16, "one copy");
+    CCK(cudaMemcpyAsync(&h, c->d_loss, sizeof h, cudaMemcpyDeviceToHost, c->stream));
     CCK(cudaStreamSynchronize(c->stream));
-    if (h) {
+    if (h.err[0]) {
         CCK(cudaMemsetAsync(c->d_err, 0, sizeof(unsigned int), c->stream));  // reported once
         CCK(cudaStreamSynchronize(c->stream));
         return cfail(c, PIC_ETIMEOUT, "a tensor-core completion wait timed out");
     }
+    if (loss) *loss = h.loss;
     return PIC_OK;
 }
 
-// forward (kept activations) + loss + backward into c->grads (zeroed first)
-int gradient(pic_cnn* c, int nimg, int nx, int ny, const float* in, const float* tgt, double* loss) {
+// Enqueues forward (kept activations), loss and backward into c->grads, with `adam` the
+// update of the parameters too.
+int gradient(pic_cnn* c, int nimg, int nx, int ny, const float* in, const float* tgt, const AdamArgs& adam) {
     if (int rc = prepare(c, nimg, nx, ny)) return rc;
+    if (!c->part) CCK(dalloc(&c->part, (size_t)4 * kWPerLayer * kWSlice));
     const long long npi = (long long)nx * ny, P = npi * nimg, nt = P / kTile;
     cudaStream_t st = c->stream;
     CCK(cudaMemcpyAsync(c->planes, in, P * 3 * sizeof(float), cudaMemcpyDefault, st));
-    CCK(cudaMemcpyAsync(c->planes + P * 3, tgt, P * 3 * sizeof(float), cudaMemcpyDefault, st));
-    if (int rc = pack(c)) return rc;
-    k_planes_in<<<blocks(P), 256, 0, st>>>(P, npi, c->planes, reinterpret_cast<bf16*>(c->X[0]));
+    if (int rc = begin(c, c->planes, P, npi)) return rc;
     forward(c->wf, nullptr, c->params, P, c->imgs, c->tile_img, c->X[0], c->X[1], c->X[2], c->X[3], c->out, c->d_err, st);
-    CCK(cudaMemsetAsync(c->d_loss, 0, sizeof(double), st));
+    // (the target's copy after the forward launches, which run meanwhile)
+    CCK(cudaMemcpyAsync(c->planes + P * 3, tgt, P * 3 * sizeof(float), cudaMemcpyDefault, st));
     k_loss<<<blocks(P), 256, 0, st>>>(P, npi, c->out, c->planes + P * 3, reinterpret_cast<bf16*>(c->dY[3]), c->d_loss);
     // input gradients: dY3 = bf16(dY4 * W4^T), dY2, dY1
     conv<16, 32, false>(nt, c->imgs, c->tile_img, c->dY[3], c->wd[3], nullptr, 0, c->dY[2], c->d_err, st);
     conv<32, 32, false>(nt, c->imgs, c->tile_img, c->dY[2], c->wd[2], nullptr, 0, c->dY[1], c->d_err, st);
     conv<32, 32, false>(nt, c->imgs, c->tile_img, c->dY[1], c->wd[1], nullptr, 0, c->dY[0], c->d_err, st);
-    // weight and bias gradients
-    CCK(cudaMemsetAsync(c->grads, 0, kNParams * sizeof(float), st));
-    wgrad<16, 32>(P, c->imgs, c->tile_img, c->X[0], c->dY[0], c->grads + kL[0].w_off, 3, 32, c->d_err, st);
-    wgrad<32, 32>(P, c->imgs, c->tile_img, c->X[1], c->dY[1], c->grads + kL[1].w_off, 32, 32, c->d_err, st);
-    wgrad<32, 32>(P, c->imgs, c->tile_img, c->X[2], c->dY[2], c->grads + kL[2].w_off, 32, 32, c->d_err, st);
-    wgrad<32, 16>(P, c->imgs, c->tile_img, c->X[3], c->dY[3], c->grads + kL[3].w_off, 32, 3, c->d_err, st);
-    const unsigned bb = (unsigned)std::min<long long>(blocks(P), 304);
-    k_bias_grad<32><<<bb, 256, 0, st>>>(P, reinterpret_cast<bf16*>(c->dY[0]), 32, c->grads + kL[0].b_off);
-    k_bias_grad<32><<<bb, 256, 0, st>>>(P, reinterpret_cast<bf16*>(c->dY[1]), 32, c->grads + kL[1].b_off);
-    k_bias_grad<32><<<bb, 256, 0, st>>>(P, reinterpret_cast<bf16*>(c->dY[2]), 32, c->grads + kL[2].b_off);
-    k_bias_grad<16><<<bb, 256, 0, st>>>(P, reinterpret_cast<bf16*>(c->dY[3]), 3, c->grads + kL[3].b_off);
+    WgradArgs w{};
+    w.imgs = c->imgs;
+    w.tile_img = c->tile_img;
+    for (int L = 0; L < 4; L++) {
+        w.X[L] = reinterpret_cast<const bf16*>(c->X[L]);
+        w.dY[L] = reinterpret_cast<const bf16*>(c->dY[L]);
+    }
+    w.part = c->part;
+    w.nchunks = P / kChunk;
+    w.ctas = (int)std::min<long long>(w.nchunks, kWPerLayer);
+    w.err = c->d_err;
+    k_wgrad<<<4 * w.ctas, kWThreads, kWSmem, st>>>(w);
+    k_finish<<<dim3(blocks(kWSlice), 4), 256, 0, st>>>(c->part, w.ctas, c->grads, adam, c->d_err);
     CCK(cudaGetLastError());
-    if (loss) CCK(cudaMemcpyAsync(loss, c->d_loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-    return check_err(c);
+    return PIC_OK;
 }
 
 }  // namespace
@@ -865,14 +903,14 @@ int pic_cnn_create(pic_cnn** out) {
         e = dalloc(&c->wf[L], (size_t)kL[L].cout_pad * 9 * kL[L].cin_pad);
         if (e == cudaSuccess && L) e = dalloc(&c->wd[L], (size_t)kL[L].cin * 9 * kL[L].cout_pad);
     }
-    if (e == cudaSuccess) e = dalloc(&c->d_loss, 1);
-    if (e == cudaSuccess) e = dalloc(&c->d_err, 2);  // [0] a wait ran out, [1] the waits' poll limit
+    if (e == cudaSuccess) e = dalloc(&c->d_loss, 2);
+    if (e == cudaSuccess) c->d_err = reinterpret_cast<unsigned int*>(c->d_loss + 1);
     if (e == cudaSuccess) e = cudaMemset(c->params, 0, kNParams * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(c->m1, 0, kNParams * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(c->m2, 0, kNParams * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, 2 * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(c->d_loss, 0, 2 * sizeof(double));
     if (e == cudaSuccess) e = set_smem_once();
-    if (e == cudaSuccess && pack(c) != PIC_OK) e = cudaErrorUnknown;
+    if (e == cudaSuccess && begin(c, nullptr, 0, 1) != PIC_OK) e = cudaErrorUnknown;
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         g_cnn_err = std::string("pic_cnn_create: ") + cudaGetErrorString(e);
@@ -889,7 +927,7 @@ void pic_cnn_free(pic_cnn* c) {
     cudaSetDevice(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
     free_call_buffers(c);
-    void* ps[] = {c->params, c->grads, c->m1, c->m2, c->d_loss, c->d_err};
+    void* ps[] = {c->params, c->grads, c->m1, c->m2, c->part, c->d_loss};
     for (void* p : ps)
         if (p) cudaFree(p);
     for (int L = 0; L < 4; L++) {
@@ -910,7 +948,7 @@ int pic_cnn_set_params(pic_cnn* c, const float* p, int64_t n) {
     CCK(cudaMemsetAsync(c->m1, 0, kNParams * sizeof(float), c->stream));
     CCK(cudaMemsetAsync(c->m2, 0, kNParams * sizeof(float), c->stream));
     c->adam_t = 0;
-    if (int rc = pack(c)) return rc;
+    if (int rc = begin(c, nullptr, 0, 1)) return rc;
     CCK(cudaStreamSynchronize(c->stream));
     return PIC_OK;
 }
@@ -932,13 +970,12 @@ int pic_cnn_forward(pic_cnn* c, int32_t nimg, int32_t nx, int32_t ny, const floa
     const long long npi = (long long)nx * ny, P = npi * nimg;
     cudaStream_t st = c->stream;
     CCK(cudaMemcpyAsync(c->planes, in, P * 3 * sizeof(float), cudaMemcpyDefault, st));
-    if (int rc = pack(c)) return rc;
-    k_planes_in<<<blocks(P), 256, 0, st>>>(P, npi, c->planes, reinterpret_cast<bf16*>(c->X[0]));
+    if (int rc = begin(c, c->planes, P, npi)) return rc;
     forward(c->wf, nullptr, c->params, P, c->imgs, c->tile_img, c->X[0], c->X[1], c->X[2], c->X[3], c->out, c->d_err, st);
     k_planes_out<<<blocks(P), 256, 0, st>>>(P, npi, c->out, c->planes + P * 3);
     CCK(cudaGetLastError());
     CCK(cudaMemcpyAsync(out, c->planes + P * 3, P * 3 * sizeof(float), cudaMemcpyDefault, st));
-    return check_err(c);
+    return finish(c, nullptr);
 }
 
 int pic_cnn_gradient(pic_cnn* c, int32_t nimg, int32_t nx, int32_t ny, const float* in, const float* target,
@@ -946,7 +983,8 @@ int pic_cnn_gradient(pic_cnn* c, int32_t nimg, int32_t nx, int32_t ny, const flo
     if (!c) return PIC_EINVAL;
     cudaSetDevice(c->device);
     if (!in || !target || !grad) return cfail(c, PIC_EINVAL, "NULL array");
-    if (int rc = gradient(c, nimg, nx, ny, in, target, loss)) return rc;
+    if (int rc = gradient(c, nimg, nx, ny, in, target, AdamArgs{})) return rc;
+    if (int rc = finish(c, loss)) return rc;
     CCK(cudaMemcpyAsync(grad, c->grads, kNParams * sizeof(float), cudaMemcpyDefault, c->stream));
     CCK(cudaStreamSynchronize(c->stream));
     return PIC_OK;
@@ -958,12 +996,11 @@ int pic_cnn_train_step(pic_cnn* c, int32_t nimg, int32_t nx, int32_t ny, const f
     cudaSetDevice(c->device);
     if (!in || !target) return cfail(c, PIC_EINVAL, "NULL array");
     if (!(lr > 0.f) || lr > 1.f) return cfail(c, PIC_EINVAL, "lr must lie in (0, 1]");
-    if (int rc = gradient(c, nimg, nx, ny, in, target, loss)) return rc;
+    const float t = (float)(c->adam_t + 1);
+    const AdamArgs u{c->params, c->m1, c->m2, lr, 1.f - std::pow(0.9f, t), 1.f - std::pow(0.999f, t)};
+    if (int rc = gradient(c, nimg, nx, ny, in, target, u)) return rc;
+    if (int rc = finish(c, loss)) return rc;
     c->adam_t++;
-    const float c1 = 1.f - std::pow(0.9f, (float)c->adam_t), c2 = 1.f - std::pow(0.999f, (float)c->adam_t);
-    k_adam<<<blocks(kNParams), 256, 0, c->stream>>>(kNParams, c->params, c->grads, c->m1, c->m2, lr, c1, c2);
-    CCK(cudaGetLastError());
-    CCK(cudaStreamSynchronize(c->stream));
     return PIC_OK;
 }
 

@@ -23,6 +23,15 @@ __host__ __device__ __forceinline__ uint32_t canon_offset(int r, int k, int K) {
     return (uint32_t)((r >> 3) * (K >> 3) * 128 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
+// The same matrix with its rows contiguous ("MN-major, no swizzle"): core matrices of 8
+// rows x 8 columns whose columns are 16 bytes of 8 rows each. With kLbo = 128 bytes between
+// core matrices along K and (K / 8) * 128 between 8-row groups, element (r, k) sits at
+// (r / 8) * sbo + 16 k + (r % 8) * 2, so 8 rows of one column are one 16-byte store. One MMA
+// still moves 256 bytes along K.
+__host__ __device__ __forceinline__ uint32_t mn_offset(int r, int k, int K) {
+    return (uint32_t)((r >> 3) * (K >> 3) * 128 + k * 16 + (r & 7) * 2);
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -44,6 +53,9 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+
+// The same with both operands MN-major.
+__host__ __device__ constexpr uint32_t make_idesc_mn(int M, int N) { return make_idesc(M, N) | (1u << 15) | (1u << 16); }
 
 // Whole warp: allocate ncols (power of two >= 32) tensor-memory columns; the address is
 // written to *dst (shared memory).
