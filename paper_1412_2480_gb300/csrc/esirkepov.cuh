@@ -59,8 +59,8 @@ __device__ __forceinline__ R window_weight(const R w[P + 1], bool sh, int k) {
 //   Jx(i+1/2) = Jx(i-1/2) - fx Wx, Jy(j+1/2) = Jy(j-1/2) - fy Wy, Jz += fz Wz,
 // with fx = q dx/(dt dx dy), fy = q dy/(dt dx dy), fz = q vz/(dx dy). The Jx running sum
 // over the last window column is zero (charge conservation), so only P+1 columns of Jx
-// (and P+1 rows of Jy) are written. `add(comp, ix, iy, value)` receives window-origin
-// node indices (unwrapped).
+// (and P+1 rows of Jy) are written. `add(comp, ix, iy, value, on)` receives window-origin
+// node indices (unwrapped); a value with `on` false is not added.
 //
 // When the old and new shapes start on the same row (the move does not shift the y
 // base), the window's last row has S0y = S1y = 0: every Wx and Wz there is zero, and the
@@ -75,7 +75,7 @@ __device__ __forceinline__ R window_weight(const R w[P + 1], bool sh, int k) {
 template <int P, int WY, typename R, typename Add>
 __device__ __forceinline__ void esirkepov_window(int ox, int oy, const R S0x[P + 2], const R DSx[P + 2],
                                                  const R S0y[P + 2], const R DSy[P + 2], R fx, R fy, R fz,
-                                                 bool ysame, Add add) {
+                                                 bool ysame, Add& add) {
     // row b of the window is an exact zero for this lane
     const auto row0 = [&](int b) { return WY == P + 2 && b == P + 1 && ysame; };
 #pragma unroll
@@ -85,7 +85,7 @@ __device__ __forceinline__ void esirkepov_window(int ox, int oy, const R S0x[P +
 #pragma unroll
         for (int a = 0; a <= P; a++) {
             run = xfma(-DSx[a], ry, run);
-            if (!row0(b)) add(0, ox + a, oy + b, run);
+            add(0, ox + a, oy + b, run, !row0(b));
         }
     }
 #pragma unroll
@@ -95,7 +95,7 @@ __device__ __forceinline__ void esirkepov_window(int ox, int oy, const R S0x[P +
 #pragma unroll
         for (int b = 0; b < WY - 1; b++) {
             run = xfma(-DSy[b], rx, run);
-            if (b < P || !ysame) add(1, ox + a, oy + b, run);
+            add(1, ox + a, oy + b, run, b < P || !ysame);
         }
     }
 #pragma unroll
@@ -104,13 +104,14 @@ __device__ __forceinline__ void esirkepov_window(int ox, int oy, const R S0x[P +
         const R cy1 = xmul(fz, xfma(R(1.0 / 3.0), DSy[b], xmul(R(0.5), S0y[b])));
 #pragma unroll
         for (int a = 0; a < P + 2; a++)
-            if (!row0(b)) add(2, ox + a, oy + b, xfma(S0x[a], cy0, xmul(DSx[a], cy1)));
+            add(2, ox + a, oy + b, xfma(S0x[a], cy0, xmul(DSx[a], cy1)), !row0(b));
     }
+    if constexpr (sizeof(R) == 4) add.last();
 }
 
 template <int P, typename R, typename Add>
 __device__ __forceinline__ void esirkepov(int i0, R f0x, int j0, R f0y, int i1, R f1x, int j1,
-                                          R f1y, R fx, R fy, R fz, Add add) {
+                                          R f1y, R fx, R fy, R fz, Add& add) {
     int b0x, b1x, b0y, b1y;
     R s0x[P + 1], s1x[P + 1], s0y[P + 1], s1y[P + 1];
     shape_nodes<P, R>(i0, f0x, b0x, s0x);

@@ -107,20 +107,21 @@ k_push_fp64(const GridDev* __restrict__ grids, const SegDev* __restrict__ segs,
             if (G.deposit) {
                 const int i1 = (int)floor(X1), j1 = (int)floor(Y1);
                 double* Jb = J + G.cell_off;
+                auto add = [&](int comp, int ix, int iy, double v, bool on) {
+                    if (!on) return;
+                    double* row = Jb + comp * ntot + (long long)wrapi(iy, ny) * nx;
+                    if (!walls) {
+                        atomicAdd(row + wrapi(ix, nx), v);
+                        return;
+                    }
+                    // a reflected particle continues as its mirror image: Jx folds odd, Jy and
+                    // Jz even
+                    int s;
+                    const int cx = wall_col(ix, nx, comp == 0, comp == 0, s);
+                    if (s != 0) atomicAdd(row + cx, s < 0 ? -v : v);
+                };
                 esirkepov<P, double>(i, fxp, j, fyp, i1, X1 - i1, j1, Y1 - j1, G.p64_fx[S.species],
-                                     G.p64_fy[S.species], G.p64_fz[S.species] * (u[2] * ig),
-                                     [&](int comp, int ix, int iy, double v) {
-                                         double* row = Jb + comp * ntot + (long long)wrapi(iy, ny) * nx;
-                                         if (!walls) {
-                                             atomicAdd(row + wrapi(ix, nx), v);
-                                             return;
-                                         }
-                                         // a reflected particle continues as its mirror image:
-                                         // Jx folds odd, Jy and Jz even
-                                         int s;
-                                         const int cx = wall_col(ix, nx, comp == 0, comp == 0, s);
-                                         if (s != 0) atomicAdd(row + cx, s < 0 ? -v : v);
-                                     });
+                                     G.p64_fy[S.species], G.p64_fz[S.species] * (u[2] * ig), add);
             }
             if (walls) {  // specular reflection at the walls
                 if (X1 < 0.0) {
