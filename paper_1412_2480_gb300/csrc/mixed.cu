@@ -1047,59 +1047,189 @@ __global__ void k_gather_overflow(long long n_over, int gs, Slots O, long long b
 
 // Node density (q[s] per particle, 0: species left out) and w times the total momentum
 // straight from the bins: a block takes part `blockIdx.y` of the particles of one (tile,
-// species), all nine segments (one block row more: the overflow list). The particles are
-// read once, in the bins' order of 32 distinct cells per warp, so the atomics of a warp
-// fall on neighbouring nodes. rho, mom: null where not asked for.
+// species), all nine segments (one block row more: the overflow list). rho, mom: null where
+// not asked for.
+//
+// In FP64 throughout the kernel was bound by that pipe (two lanes per cycle and SM, 28
+// operations per particle at order 2: 376 us for 8.4e6 particles). Here weights and their
+// products are 64-bit whole numbers, exact to 2^-56 of a full weight, and so are the sums in
+// the tile's window in shared memory; FP64 is left to the window's nodes when the block is
+// done, and to the offsets below 2^-17 that have smaller bits. A window's node holds up to
+// 256 full weights (113 at order 3); what wraps goes to the output at once. 1024 x 256 with 16
+// per cell, order 2 (8.4e6 particles, 101 MB): 376 -> 95 us, bound by the bank conflicts of
+// the two atomics per node (3.3 wavefronts each on random nodes) and the 64-bit products.
+// Against exact sums the error is no larger than FP64's at any density from one particle per
+// cell (order 2, 16 per cell: 6e-17 against 3.2e-16, relative to the density's norm).
 struct DensityArgs {
     double q[2], w;
     double *rho, *mom;
 };
 
 template <int P>
-__device__ __forceinline__ void density_one(const GridDev& G, const unsigned* B, long long k, double q, double* rho,
-                                            double* mom, double m[3]) {
-    const float* F = reinterpret_cast<const float*>(B);
-    if (rho) {
-        const int c = (int)__ldcs(B + aos(k, 0));
-        deposit_rho<P>(G, c & 0xffff, (double)__ldcs(F + aos(k, 1)), c >> 16, (double)__ldcs(F + aos(k, 2)), q, rho);
+__device__ __noinline__ void density_global(const GridDev& G, int c, float fx, float fy, double q, double* rho) {
+    deposit_rho<P>(G, c & 0xffff, (double)fx, c >> 16, (double)fy, q, rho);
+}
+
+// rho += v at the node (ix, iy), which may lie beyond the grid's edges by a window's margin
+__device__ __forceinline__ void density_node(const GridDev& G, int ix, int iy, double v, double* rho) {
+    int sign = 1, col;
+    if (G.walls) col = wall_col(ix, G.nx, false, false, sign);
+    else col = wrap_window(ix, G.nx);
+    if (sign) atomicAdd(rho + (long long)wrap_window(iy, G.ny) * G.nx + col, v);
+}
+
+struct DensityWin {
+    unsigned *lo, *hi;  // words of the sums, wx per row
+    int wx, X0, Y0;     // the window's row length and first node
+    double unit;
+    double* rho;
+};
+
+// the sums of window nodes k0 + (bit / 4) wx + bit % 4 passed 2^64 units
+__device__ __noinline__ void density_wrapped(const GridDev& G, int k0, unsigned bits, int X0, int Y0, double unit,
+                                             double* rho) {
+    for (; bits; bits &= bits - 1) {
+        const int n = __ffs(bits) - 1, k = k0 + (n >> 2) * G.wx + (n & 3);
+        density_node(G, X0 + k % G.wx, Y0 + k / G.wx, unit * 18446744073709551616.0, rho);
     }
-    if (mom)
+}
+
+// 64-bit sums of N neighbouring nodes, each from two 32-bit atomics: the one that sees a word
+// wrap carries. All low words, then all high ones: one wait for each, not for each node.
+// Returns which sums wrapped.
+template <int N>
+__device__ __forceinline__ unsigned density_add(const DensityWin& W, int k, const unsigned long long v[N]) {
+    unsigned l[N], h[N], wrapped = 0;
 #pragma unroll
-        for (int a = 0; a < 3; a++) m[a] += (double)__ldcs(F + aos(k, 3 + a));
+    for (int a = 0; a < N; a++) l[a] = atomicAdd(W.lo + k + a, (unsigned)v[a]);
+#pragma unroll
+    for (int a = 0; a < N; a++) {
+        const unsigned vh = (unsigned)(v[a] >> 32) + (l[a] + (unsigned)v[a] < l[a] ? 1u : 0u);
+        l[a] = vh;
+        h[a] = atomicAdd(W.hi + k + a, vh);
+    }
+#pragma unroll
+    for (int a = 0; a < N; a++) wrapped |= h[a] + l[a] < h[a] ? 1u << a : 0u;
+    return wrapped;
+}
+
+// The weights of each axis add up to one, so the products of one column and one row (the
+// middle ones: the largest weight, at order 1 the lower node's) follow from the others by
+// subtraction: 4 products instead of 9 at order 2, and a particle's charge is exact. A
+// product a few units from zero may come out below it: cut there, but for the middle one's
+// own, which is at least 2^8 units.
+template <int P>
+__device__ __forceinline__ void density_window(const GridDev& G, const DensityWin& W, int i, unsigned long long fx,
+                                               int j, unsigned long long fy) {
+    constexpr int C = P == 1 ? 0 : 1;
+    constexpr int one = P == 3 ? 3 : 0;  // the weights' sum is 2^60, at order 3 6 x 2^58
+    int bx, by;
+    unsigned long long X[P + 1], Y[P + 1];
+    rho_weights_fixed<P>(i, fx, bx, X);
+    rho_weights_fixed<P>(j, fy, by, Y);
+    const int k0 = by * W.wx + bx;
+    const auto whole = [&](unsigned long long w) { return one ? (w >> 5) * 3 : w >> 4; };  // w times the sum
+    const auto cut = [](unsigned long long v) { return (long long)v < 0 ? 0ull : v; };
+    unsigned long long mid[P + 1];  // the middle row
+    unsigned wrapped = 0;
+#pragma unroll
+    for (int a = 0; a <= P; a++) mid[a] = whole(X[a]);
+#pragma unroll
+    for (int b = 0; b <= P; b++) {
+        if (b == C) continue;
+        unsigned long long v[P + 1];
+        v[C] = whole(Y[b]);
+#pragma unroll
+        for (int a = 0; a <= P; a++) {
+            if (a == C) continue;
+            v[a] = mul_hi(X[a], Y[b]);
+            v[C] -= v[a];
+            mid[a] -= v[a];
+        }
+        v[C] = cut(v[C]);
+        mid[C] -= v[C];
+        wrapped |= density_add<P + 1>(W, k0 + b * W.wx, v) << 4 * b;
+    }
+#pragma unroll
+    for (int a = 0; a <= P; a++)
+        if (a != C) mid[a] = cut(mid[a]);
+    wrapped |= density_add<P + 1>(W, k0 + C * W.wx, mid) << 4 * C;
+    if (wrapped) density_wrapped(G, k0, wrapped, W.X0, W.Y0, W.unit, W.rho);
 }
 
 template <int P>
 __global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int nbins, const DensityArgs d) {
+    extern __shared__ unsigned dens_win[];  // [2][wx * wy]: low and high words
     __shared__ double s_m[3][256];
     const GridDev& G = a.grids[g];
     const DevStatus* st = a.st;
     const int par = (int)st->parity;
     const int tid = threadIdx.x;
     double m[3] = {0.0, 0.0, 0.0};
+    const auto momentum = [&](const float* F, long long k) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) m[c] += (double)__ldcs(F + aos(k, 3 + c));
+    };
     if ((int)blockIdx.x < nbins) {
         // (species by halves of the grid: with alternating ones a species left out would
         // idle every other SM)
-        const int s = (int)blockIdx.x >= G.ntiles ? 1 : 0;
-        const long long bin = 2ll * ((int)blockIdx.x - s * G.ntiles) + s;
+        const int s = (int)blockIdx.x >= G.ntiles ? 1 : 0, t = (int)blockIdx.x - s * G.ntiles;
+        const long long bin = 2ll * t + s;
         const double q = s ? d.q[1] : d.q[0];
         double* rho = q != 0.0 ? d.rho : nullptr;
         if (!(d.mom || rho)) return;
         const unsigned* B = par ? a.buf[1] : a.buf[0];
+        const float* F = reinterpret_cast<const float*>(B);
         const int* cnt = (par ? a.cnt[1] : a.cnt[0]) + ((long long)G.tile_first * 2 + bin) * kSegs;
+        const int X0 = t % G.ntx * G.tx, Y0 = t / G.ntx * G.ty, NW = G.wx * G.wy;
+        const int nx = G.nx, ny = G.ny, tx = G.tx, ty = G.ty;
+        const DensityWin W{dens_win, dens_win + NW, G.wx, X0 - 2, Y0 - 2, q / kRhoUnits<P>, rho};
+        if (rho)
+            for (int k = tid; k < 2 * NW; k += 256) dens_win[k] = 0u;
+        __syncthreads();
         long long base = G.bin_off + bin * bin_stride(G);
         for (int k = 0; k < kSegs; k++) {
             const int lim = (int)(k == 0 ? G.cap : G.capo), n = min(cnt[k], lim);
-            for (int v = (int)blockIdx.y * 256 + tid; v < n; v += (int)gridDim.y * 256)
-                density_one<P>(G, B, base + v, q, rho, d.mom, m);
+            for (int v = (int)blockIdx.y * 256 + tid; v < n; v += (int)gridDim.y * 256) {
+                if (rho) {
+                    const int c = (int)__ldcs(B + aos(base + v, 0));
+                    const float fx = __ldcs(F + aos(base + v, 1)), fy = __ldcs(F + aos(base + v, 2));
+                    // cell within the window (its origin is X0 - 2, Y0 - 2): the tile's own
+                    // and, in the outboxes, the next ones around it, across the periodic edge
+                    int i = (c & 0xffff) - X0 + 2, j = (c >> 16) - Y0 + 2;
+                    if (i < 1) i += nx;
+                    else if (i > tx + 2) i -= nx;
+                    if (j < 1) j += ny;
+                    else if (j > ty + 2) j -= ny;
+                    unsigned long long Fx, Fy;
+                    const bool fine = offset_fixed(fx, Fx) && offset_fixed(fy, Fy);
+                    if (fine && i >= 1 && i <= tx + 2 && j >= 1 && j <= ty + 2)
+                        density_window<P>(G, W, i, Fx, j, Fy);
+                    else
+                        density_global<P>(G, c, fx, fy, q, rho);
+                }
+                if (d.mom) momentum(F, base + v);
+            }
             base += lim;
+        }
+        if (rho) {
+            __syncthreads();
+            for (int k = tid; k < NW; k += 256) {
+                const unsigned long long v = (unsigned long long)W.hi[k] << 32 | W.lo[k];
+                if (v) density_node(G, W.X0 + k % G.wx, W.Y0 + k / G.wx, W.unit * (double)v, rho);
+            }
         }
     } else {
         const Slots O = par ? a.ovf[1] : a.ovf[0];
+        const float* F = reinterpret_cast<const float*>(O.p);
         const long long n = min((long long)st->ovf_count[par], a.ovf_cap);
         for (long long k = (long long)blockIdx.y * 256 + tid; k < n; k += (long long)gridDim.y * 256) {
             const int gs = O.gs[k];
+            if (gs >> 1 != g) continue;
             const double q = gs & 1 ? d.q[1] : d.q[0];
-            if (gs >> 1 == g) density_one<P>(G, O.p, k, q, q != 0.0 ? d.rho : nullptr, d.mom, m);
+            if (d.rho && q != 0.0)
+                density_global<P>(G, (int)O.p[aos(k, 0)], F[aos(k, 1)], F[aos(k, 2)], q, d.rho);
+            if (d.mom) momentum(F, k);
         }
     }
     if (!d.mom) return;
@@ -1820,14 +1950,18 @@ int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, d
     const GridDev& G = m->G[g];
     const DensityArgs d{{q_s[0], q_s[1]}, G.w, rho, mom};
     const int nbins = 2 * G.ntiles;
-    // about 1024 particles per block (a bin's share of its capacity): with whole bins of 8192
-    // the few blocks of an SM more or less left a third of the device idle
-    const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / 1280)));
+    // Parts of a bin: 4096 particles each (5120 of its capacity) keep the window's cost, its
+    // zeroing and its nodes' FP64, below a tenth of the block's time; half as many where that
+    // leaves fewer than the eight blocks that an SM holds (512 x 256, 8 per cell: 30 -> 22 us;
+    // 1024 x 256, 16 per cell: 95 us against 101 with the short parts).
+    const long long chunk = nbins * std::max(1ll, G.cap / 5120) < 8 * 152 ? 2560 : 5120;
+    const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / chunk)));
+    const size_t sm = d.rho ? (size_t)2 * G.wx * G.wy * sizeof(unsigned) : 0;
     const MixedArgs a = make_args(m, 0);
     switch (G.order) {
-    case 1: k_density<1><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
-    case 2: k_density<2><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
-    default: k_density<3><<<nb, 256, 0, st>>>(a, g, nbins, d); break;
+    case 1: k_density<1><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
+    case 2: k_density<2><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
+    default: k_density<3><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
     }
     MCK(cudaGetLastError());
     return PIC_OK;
