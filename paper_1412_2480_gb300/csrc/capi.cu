@@ -53,6 +53,7 @@ struct pic_sim {
     CgState* cg = nullptr;
     unsigned int* done = nullptr;
     DevStatus* st = nullptr;
+    DevStatus* host_st = nullptr;    // [2], pinned: the status before and after a chunk of steps
     double* tmp = nullptr;  // ntot scratch for conversions (pic_fields of J in MIXED32)
     // FP64 particles, one set of arrays per species (grid units)
     double* pa[2][5] = {{nullptr}};
@@ -906,6 +907,7 @@ int init_handle(const pic_params* prm, int n, pic_sim** out) {
     A(dalloc(&s->cg, s->ngrids));
     A(dalloc(&s->done, s->ngrids));
     A(dalloc(&s->st, 1));
+    A(cudaMallocHost((void**)&s->host_st, 2 * sizeof(DevStatus)));
     A(dalloc(&s->tmp, s->ntot));
     A(dalloc(&s->dgrids, s->ngrids));
     A(dalloc(&s->dblk_grid, s->nblk));
@@ -1180,13 +1182,15 @@ int pic_load_particles(pic_sim* s, int32_t sp, const double* x, const double* y,
     if (n < 0) return fail(s, PIC_EINVAL, "n must be >= 0");
     if (n > 0 && (!x || !y || !ux || !uy || !uz)) return fail(s, PIC_EINVAL, "NULL particle array");
     if (n > (int64_t)1 << 40) return fail(s, PIC_EINVAL, "n too large");
-    drop_graph(s);
     if (s->prm.precision == PIC_MIXED32) {
+        // (its graph holds the bins' addresses, not their counts: it stays unless the bins
+        // were reallocated, which check_graph_generation sees)
         int rc = mixed_load(s->mixed, s->sel, sp, x, y, ux, uy, uz, n, s->stream, s->err);
         if (rc == PIC_OK) rc = finish_call(s);
         return rc;
     }
     // FP64: arrays for n particles (plus what the injector can add)
+    drop_graph(s);
     s->np[sp] = 0;
     if (int rc = fp64_arrays(s, sp, n + inj_capacity(s->hgrids[0]), 0)) return rc;
     const double* src[5] = {x, y, ux, uy, uz};
@@ -1233,17 +1237,14 @@ namespace {
 // host re-sorts them into larger bins after a chunk.
 constexpr int kStepChunk = 32;
 
+// One wait per chunk: the status before and after it comes through pinned memory, in
+// stream order with the steps.
 int step_chunk(pic_sim* s, int32_t n) {
     // a new chunk starts clean: errors stop the rest of the chunk that raised them, and
     // the call returns
-    DevStatus hs{};
-    CK(cudaMemcpyAsync(&hs, s->st, sizeof hs, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaStreamSynchronize(s->stream));
-    const unsigned long long steps0 = hs.steps_done;
-    const unsigned long long li0 = hs.loop_iters[0], lr0 = hs.loop_iters[1];
-    hs.stop = 0;
-    hs.stop_next = 0;
-    CK(cudaMemcpyAsync(s->st, &hs, sizeof hs, cudaMemcpyHostToDevice, s->stream));
+    DevStatus *before = s->host_st, *after = s->host_st + 1;
+    CK(cudaMemcpyAsync(before, s->st, sizeof *before, cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemsetAsync(&s->st->stop, 0, sizeof s->st->stop + sizeof s->st->stop_next, s->stream));
     if (s->prm.precision == PIC_MIXED32) {
         int rc = mixed_before_steps(s->mixed, s->stream, s->err);
         if (rc) return rc;
@@ -1261,13 +1262,15 @@ int step_chunk(pic_sim* s, int32_t n) {
             if (int rc = run_step_direct(s)) return rc;
         }
     }
-    CK(cudaMemcpyAsync(&hs, s->st, sizeof hs, cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(after, s->st, sizeof *after, cudaMemcpyDeviceToHost, s->stream));
     if (int rc = finish_call(s)) return rc;
-    s->steps += (long long)(hs.steps_done - steps0);
-    s->kernels += n * per_step + loop_kernels(s, hs.loop_iters[0] - li0, hs.loop_iters[1] - lr0);
+    const DevStatus hs = *after;
+    s->steps += (long long)(hs.steps_done - before->steps_done);
+    s->kernels += n * per_step + loop_kernels(s, hs.loop_iters[0] - before->loop_iters[0],
+                                             hs.loop_iters[1] - before->loop_iters[1]);
     if (int rc0 = fp64_counts(s)) return rc0;
     int rc = device_errors(s, hs);
-    if (rc == PIC_OK && s->prm.precision == PIC_MIXED32) rc = mixed_after_steps(s->mixed, s->stream, s->err);
+    if (rc == PIC_OK && s->prm.precision == PIC_MIXED32) rc = mixed_after_steps(s->mixed, hs, s->stream, s->err);
     return rc;
 }
 
@@ -1346,7 +1349,7 @@ int profile_chunk(pic_sim* s, int32_t n, double* acc) {
     if (int rc0 = fp64_counts(s)) return rc0;
     acc[4] += (double)(c1.total_iters - c0.total_iters);
     int rc = device_errors(s, hs);
-    if (rc == PIC_OK && s->prm.precision == PIC_MIXED32) rc = mixed_after_steps(s->mixed, s->stream, s->err);
+    if (rc == PIC_OK && s->prm.precision == PIC_MIXED32) rc = mixed_after_steps(s->mixed, hs, s->stream, s->err);
     return rc;
 }
 
@@ -1699,6 +1702,7 @@ void pic_free(pic_sim* s) {
                     s->part, s->cg_part, s->cg, s->done, s->st, s->tmp, s->dsegs, s->dblk_seg[0], s->dblk_seg[1],
                     s->bvec, s->r32, s->p32, s->q32, s->e32, s->r32b, s->z32};
     for (void* p : ptrs) dfree(p);
+    if (s->host_st) cudaFreeHost(s->host_st);
     for (int sp = 0; sp < 2; sp++)
         for (int a = 0; a < 5; a++) dfree(s->pa[sp][a]);
     if (s->body_stream) cudaStreamDestroy(s->body_stream);

@@ -1918,9 +1918,7 @@ int mixed_step_kernels(const MixedState* m) {
     return k + (m->inject_grids ? 1 : 0);
 }
 
-int mixed_after_steps(MixedState* m, cudaStream_t st, std::string& err) {
-    DevStatus hs{};
-    if (int rc = read_status(m, hs, st, err)) return rc;
+int mixed_after_steps(MixedState* m, const DevStatus& hs, cudaStream_t st, std::string& err) {
     if (m->inject_grids) {  // the injector's pairs join the live counts
         std::vector<unsigned long long> add((size_t)2 * m->ngrids);
         MCK(cudaMemcpyAsync(add.data(), m->injected, add.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));

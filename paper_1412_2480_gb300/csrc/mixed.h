@@ -34,7 +34,8 @@ int mixed_load(MixedState* m, int g, int sp, const double* x, const double* y, c
 void mixed_enqueue(MixedState* m, cudaStream_t s, int part);
 // Host bookkeeping around a pic_step call (re-bin when bins overflowed).
 int mixed_before_steps(MixedState* m, cudaStream_t s, std::string& err);
-int mixed_after_steps(MixedState* m, cudaStream_t s, std::string& err);
+// hs: the device status as it is after the steps
+int mixed_after_steps(MixedState* m, const DevStatus& hs, cudaStream_t s, std::string& err);
 
 // Kernels mixed_enqueue launches per step (all parts together).
 int mixed_step_kernels(const MixedState* m);

@@ -94,6 +94,7 @@ struct DevStatus {
     unsigned int cg_noconv;          // PCG hit maxit
     unsigned int stop;               // nonzero: this and later steps of the call are skipped
     unsigned int stop_next;          // set during a step; becomes `stop` at the next step
+                                     // (the host clears the two words with one memset)
     unsigned long long steps_done;   // steps completed (the failing step included)
     unsigned int grids_done;         // counter of the last-grid-finished pattern
     unsigned int n_active;           // simulations whose PCG is still iterating
