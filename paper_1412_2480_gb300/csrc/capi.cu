@@ -84,6 +84,8 @@ struct pic_sim {
     CnnGuess guess;
     // MIXED32 solve as one cooperative kernel
     bool use_coop = false;
+    int cells_blocks = 0;             // > 0: the cooperative kernel on cells (any nx) instead
+    unsigned int* cells_bar = nullptr;
     CoopSolve coop;
     // bookkeeping
     long long steps = 0;
@@ -300,7 +302,7 @@ FieldArgs field_args(pic_sim* s, int use_cond, cudaGraphConditionalHandle cond) 
     a.e32 = s->e32;
     a.r32b = s->r32b;
     a.z32 = s->z32;
-    a.bar = s->use_coop ? s->coop.bar : nullptr;
+    a.bar = s->use_coop ? s->coop.bar : s->cells_bar;
     return a;
 }
 
@@ -467,6 +469,17 @@ int capture(pic_sim* s, int mask, cudaGraph_t* gout, cudaGraphExec_t* xout) {
             launch_nodal(field_args(s, 0, 0), st);
             continue;
         }
+        if (s->cells_blocks) {  // the same with the starting residual in FP64
+            launch_rhs(field_args(s, 0, 0), st);
+            if (s->learned) {
+                launch_learned_guess(s->guess, s->dgrids, s->cg, s->ntot, s->bvec, nullptr, s->x, nullptr, st);
+                launch_guess_residual(field_args(s, 0, 0), st);
+            }
+            e = launch_mp_cells(field_args(s, 0, 0), s->cells_blocks, st);
+            if (e == cudaSuccess) launch_field_update(field_args(s, 0, 0), st);
+            launch_nodal(field_args(s, 0, 0), st);
+            continue;
+        }
         if (s->use_coop) {
             // rhs -> (learned guess) -> one cooperative kernel for the whole PCG -> update
             launch_rhs(field_args(s, 0, 0), st);
@@ -564,7 +577,7 @@ long long step_kernels(pic_sim* s, bool graph) {
         k += s->hgrids[0].inject ? 1 : 0;
     }
     if (s->learned) k += 2;  // k_guess, k_guess_residual
-    if (s->use_coop || (s->prm.precision == PIC_FP64 && !(s->prm.flags & PIC_EXPLICIT))) k += 1;
+    if (s->use_coop || s->cells_blocks || (s->prm.precision == PIC_FP64 && !(s->prm.flags & PIC_EXPLICIT))) k += 1;
     if (s->any_nodal) k += 1;  // k_nodal
     return k;
 }
@@ -572,7 +585,7 @@ long long step_kernels(pic_sim* s, bool graph) {
 // Kernels the PCG loop launched for the given loop-counter increments (none with the
 // cooperative solve: its iterations run inside one launch).
 long long loop_kernels(const pic_sim* s, unsigned long long d_iters, unsigned long long d_refine) {
-    if (s->use_coop || s->prm.precision == PIC_FP64) return 0;
+    if (s->use_coop || s->cells_blocks || s->prm.precision == PIC_FP64) return 0;
     return 2 * (long long)d_iters + 3 * (long long)d_refine;
 }
 
@@ -600,8 +613,10 @@ int run_step_direct(pic_sim* s) {
             launch_guess_residual(a, st);
         }
     }
-    if (s->use_coop || s->prm.precision == PIC_FP64) {
-        CK(s->use_coop ? launch_mp_coop(s->coop, a, st) : launch_cg(a, s->hgrids[0].ncell, s->device, st));
+    if (s->use_coop || s->cells_blocks || s->prm.precision == PIC_FP64) {
+        CK(s->use_coop ? launch_mp_coop(s->coop, a, st)
+                       : (s->cells_blocks ? launch_mp_cells(a, s->cells_blocks, st)
+                                          : launch_cg(a, s->hgrids[0].ncell, s->device, st)));
         launch_field_update(a, st);
         launch_nodal(a, st);
         enqueue_part(s, kPartEnd, st);
@@ -952,6 +967,10 @@ int init_handle(const pic_params* prm, int n, pic_sim** out) {
                                    s->err);
         if (rc == PIC_ECUDA) return bail(rc);
         s->use_coop = rc == PIC_OK;
+        if (!s->use_coop && !s->quads) {
+            A(mp_cells_blocks(s->ngrids, s->nblk, s->device, &s->cells_blocks));
+            if (s->cells_blocks) A(dalloc(&s->cells_bar, 1));
+        }
     }
     if (prm[0].precision == PIC_MIXED32) {
         int rc = mixed_create(&s->mixed, prm, s->ngrids, s->hgrids.data(), s->dgrids, s->ntot, s->F32,
@@ -1700,7 +1719,7 @@ void pic_free(pic_sim* s) {
     coop_free(&s->coop);
     void* ptrs[] = {s->dgrids, s->dblk_grid, s->F, s->J64, s->Jfix, s->F32, s->Fn, s->x, s->r, s->p, s->q,
                     s->part, s->cg_part, s->cg, s->done, s->st, s->tmp, s->dsegs, s->dblk_seg[0], s->dblk_seg[1],
-                    s->bvec, s->r32, s->p32, s->q32, s->e32, s->r32b, s->z32};
+                    s->bvec, s->r32, s->p32, s->q32, s->e32, s->r32b, s->z32, s->cells_bar};
     for (void* p : ptrs) dfree(p);
     if (s->host_st) cudaFreeHost(s->host_st);
     for (int sp = 0; sp < 2; sp++)

@@ -73,6 +73,11 @@ void launch_nodal(const FieldArgs& a, cudaStream_t s);
 // FP32 copy of the FP64 fields (after pic_set_fields / init), node-averaged where asked.
 void launch_fields_to_f32(const FieldArgs& a, cudaStream_t s);
 
+// The MIXED32 solve of launch_mp_* as one cooperative kernel, for grids whose nx is no
+// multiple of 4: the blocks it takes (0: it cannot be used), and its launch.
+cudaError_t mp_cells_blocks(int ngrids, int nblk, int dev, int* blocks);
+cudaError_t launch_mp_cells(const FieldArgs& a, int blocks, cudaStream_t s);
+
 // The MIXED32 solve as one cooperative persistent kernel (solve_coop.cu), used when the
 // device supports cooperative launches and a handle holds at most kCoopMaxGrids
 // simulations; otherwise the WHILE-node solve above runs.
@@ -87,7 +92,6 @@ struct CoopSolve {
     unsigned int* bar = nullptr;  // grid barrier: arrivals
     int nchunks = 0, nblocks = 0, ngrids = 0, ntiles = 0;
     int cheb = 0, cg_any = 0;     // some simulation takes the Chebyshev inner solve, the CG
-    int vec = 0;                  // every nx is a multiple of 4: quads of cells
     int tile_y = 0;               // height of the Chebyshev tiles
     int rsplit = 1;               // items per chunk of the pair residual
 };

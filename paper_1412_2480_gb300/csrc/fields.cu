@@ -53,25 +53,38 @@ __device__ __forceinline__ Cell cell_at(const GridDev& G, int g, int l) {
 // integer-x lattice (Ey, Ez, Bx, and the currents Jy, Jz as the field solve sees them) is
 // odd under reflection at a wall and vanishes on the wall nodes; one on a half-integer
 // lattice (Ex, By, Bz, Jx) is even. Without walls these are the periodic neighbours.
-template <typename T>
-__device__ __forceinline__ T east_odd(const T* V, const Cell& c) { return c.ew ? T(0) : V[c.ke]; }
-template <typename T>
-__device__ __forceinline__ T west_odd(const T* V, const Cell& c) { return c.ww ? -V[c.k + 1] : V[c.kw]; }
-template <typename T>
-__device__ __forceinline__ T east_even(const T* V, const Cell& c) { return c.ew ? V[c.k] : V[c.ke]; }
-template <typename T>
-__device__ __forceinline__ T west_even(const T* V, const Cell& c) { return c.ww ? V[c.k] : V[c.kw]; }
+// (V: a pointer, or an L2View of it)
+#define ELEM(V) decltype((V)[0] + (V)[0])
+template <typename A>
+__device__ __forceinline__ auto east_odd(A V, const Cell& c) -> ELEM(V) { return c.ew ? ELEM(V)(0) : V[c.ke]; }
+template <typename A>
+__device__ __forceinline__ auto west_odd(A V, const Cell& c) -> ELEM(V) { return c.ww ? -V[c.k + 1] : V[c.kw]; }
+template <typename A>
+__device__ __forceinline__ auto east_even(A V, const Cell& c) -> ELEM(V) { return c.ew ? V[c.k] : V[c.ke]; }
+template <typename A>
+__device__ __forceinline__ auto west_even(A V, const Cell& c) -> ELEM(V) { return c.ww ? V[c.k] : V[c.kw]; }
 // Sum of the two x-neighbours of component a of a B-lattice vector (a = 0: Bx, odd).
-template <typename T>
-__device__ __forceinline__ T nbx(const T* V, const Cell& c, int a) {
+template <typename A>
+__device__ __forceinline__ auto nbx(A V, const Cell& c, int a) -> ELEM(V) {
     return a == 0 ? east_odd(V, c) + west_odd(V, c) : east_even(V, c) + west_even(V, c);
 }
+#undef ELEM
+
+// An array read from L2: other blocks of the same kernel write it.
+template <typename T>
+struct L2View {
+    const T* p;
+    __device__ __forceinline__ T operator[](long long k) const { return __ldcg(p + k); }
+    __device__ __forceinline__ L2View operator+(long long o) const { return {p + o}; }
+};
 
 // Grid-stride loop over the cells of simulation g. A simulation gets a bounded number
 // of blocks (a few per SM), so the per-simulation completion counter of the reductions
 // sees few same-address atomics per kernel.
-#define FOR_CELLS(G, g, c)                                                                  \
-    for (int l_ = (blockIdx.x - (G).blk_first) * blockDim.x + threadIdx.x; l_ < (G).ncell;  \
+#define FOR_CELLS(G, g, c) FOR_CELLS_OF(G, g, c, blockIdx.x)
+// the same as block vb
+#define FOR_CELLS_OF(G, g, c, vb)                                                           \
+    for (int l_ = ((vb) - (G).blk_first) * blockDim.x + threadIdx.x; l_ < (G).ncell;        \
          l_ += (G).nblk * blockDim.x)                                                       \
         if (const Cell c = cell_at((G), (g), l_); true)
 
@@ -91,21 +104,25 @@ __device__ __forceinline__ double dld(const T* p, long long k1, long long k2, do
     else return (p[k1] - p[k2]) * s;
 }
 
+// Sum of a simulation's nblk partials by one warp, the four chains of a lane in parallel.
+__device__ __forceinline__ double partials_sum(const double* p, int nblk) {
+    const int lane = threadIdx.x & 31;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = lane; b < nblk; b += 128)
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (b + 32 * u < nblk) acc[u] += __ldcg(p + b + 32 * u);
+    return warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+}
+
 // Simulation-wide sums of its blocks' partials, in every thread of the finishing block:
-// warp a sums value a, the four chains of a lane in parallel.
+// warp a sums value a.
 template <int NV>
 __device__ __forceinline__ void finish_sums(const GridDev& G, const double* part, int nblk_total, double tot[NV]) {
     __shared__ double s_tot[NV];
     if (threadIdx.x < 32 * NV) {
-        const int lane = threadIdx.x & 31;
-        const double* p = part + (threadIdx.x >> 5) * nblk_total + G.blk_first;
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int b = lane; b < G.nblk; b += 128)
-#pragma unroll
-            for (int u = 0; u < 4; u++)
-                if (b + 32 * u < G.nblk) acc[u] += __ldcg(p + b + 32 * u);
-        const double s = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-        if (lane == 0) s_tot[threadIdx.x >> 5] = s;
+        const double s = partials_sum(part + (threadIdx.x >> 5) * nblk_total + G.blk_first, G.nblk);
+        if ((threadIdx.x & 31) == 0) s_tot[threadIdx.x >> 5] = s;
     }
     __syncthreads();
 #pragma unroll
@@ -1006,12 +1023,143 @@ constexpr int kMaxInnerIters = 64;
 
 // Inner preconditioned CG (MIXED32): z = M r with M = pc0 I + pcx (E + W) + pcy (N + S)
 // (GridDev), the same 5-point shape and wall images as A.
-template <typename T>
-__device__ __forceinline__ T precond_at(const GridDev& G, const T* V, const Cell& c, int a) {
+template <typename A>
+__device__ __forceinline__ auto precond_at(const GridDev& G, A V, const Cell& c, int a) -> decltype(V[0] + V[0]) {
+    using T = decltype(V[0] + V[0]);
     return T(G.pc0) * V[c.k] + T(G.pcx) * nbx(V, c, a) + T(G.pcy) * (V[c.kn] + V[c.ks]);
 }
 
+// The five passes of an iteration and a refinement over the cells of (virtual) block vb, one
+// text for the kernels of the WHILE node and for the cooperative kernel (k_mp_cells), so
+// that both give the same numbers. A cell's loads of all components go before its stores.
+
 // r32 = r / rms(r) (buffer 0), e = 0, z = M r32; (r, r) and (r, z).
+template <typename A>
+__device__ __forceinline__ void mp_begin(const GridDev& G, int g, int vb, long long ntot, double scale, A r, float* r32,
+                                         float* z32, float* e32, double v[2]) {
+    float acc = 0.f, acc2 = 0.f;
+    FOR_CELLS_OF(G, g, c, vb) {
+        float f[3], z[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            f[a] = (float)(r[a * ntot + c.k] * scale);
+            z[a] = (float)(precond_at(G, r + a * ntot, c, a) * scale);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const long long o = a * ntot + c.k;
+            r32[o] = f[a];
+            z32[o] = z[a];
+            e32[o] = 0.f;
+            acc = fmaf(f[a], f[a], acc);
+            acc2 = fmaf(f[a], z[a], acc2);
+        }
+    }
+    v[0] = (double)acc;
+    v[1] = (double)acc2;
+}
+
+// p = z + beta p, q = A z + beta q (= A p); (p, q).
+template <typename A>
+__device__ __forceinline__ void mp_direction(const GridDev& G, int g, int vb, long long ntot, float beta, A z32,
+                                             float* p32, float* q32, double v[1]) {
+    const float c0 = (float)G.c0, cx = (float)G.cx, cy = (float)G.cy;
+    float acc = 0.f;  // a thread's few products in FP32, summed across threads in FP64
+    FOR_CELLS_OF(G, g, c, vb) {
+        float pn[3], qn[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const long long o = a * ntot;
+            const A Z = z32 + o;
+            const float zc = Z[c.k];
+            const float Az = c0 * zc - cx * nbx(Z, c, a) - cy * (Z[c.kn] + Z[c.ks]);
+            if (beta == 0.f) {
+                pn[a] = zc;
+                qn[a] = Az;
+            } else {
+                pn[a] = fmaf(beta, p32[o + c.k], zc);
+                qn[a] = fmaf(beta, q32[o + c.k], Az);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const long long o = a * ntot + c.k;
+            p32[o] = pn[a];
+            q32[o] = qn[a];
+            acc = fmaf(pn[a], qn[a], acc);
+        }
+    }
+    v[0] = (double)acc;
+}
+
+// r' = r - alpha q into the other residual buffer, e += alpha p, z = M r' (formed from r
+// and q at the neighbours, which this pass does not change); (r', r') and (r', z).
+template <typename A>
+__device__ __forceinline__ void mp_update(const GridDev& G, int g, int vb, long long ntot, float alpha, A Rc, float* Rn,
+                                          A q32, const float* p32, float* z32, float* e32, double v[2]) {
+    const float pc0 = (float)G.pc0, pcx = (float)G.pcx, pcy = (float)G.pcy;
+    float acc = 0.f, acc2 = 0.f;
+    FOR_CELLS_OF(G, g, c, vb) {
+        float wc[3], z[3], e[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const long long o = a * ntot;
+            const A R = Rc + o, Q = q32 + o;
+            const auto w = [&](long long k) { return fmaf(-alpha, Q[k], R[k]); };
+            wc[a] = w(c.k);
+            float wx;  // sum of the two x-neighbours, images at the walls as in nbx
+            if (a == 0) wx = (c.ew ? 0.f : w(c.ke)) + (c.ww ? -w(c.k + 1) : w(c.kw));
+            else wx = (c.ew ? wc[a] : w(c.ke)) + (c.ww ? wc[a] : w(c.kw));
+            z[a] = fmaf(pc0, wc[a], fmaf(pcx, wx, pcy * (w(c.kn) + w(c.ks))));
+            e[a] = fmaf(alpha, p32[o + c.k], e32[o + c.k]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const long long o = a * ntot + c.k;
+            Rn[o] = wc[a];
+            z32[o] = z[a];
+            e32[o] = e[a];
+            acc = fmaf(wc[a], wc[a], acc);
+            acc2 = fmaf(wc[a], z[a], acc2);
+        }
+    }
+    v[0] = (double)acc;
+    v[1] = (double)acc2;
+}
+
+// x += e (FP64).
+__device__ __forceinline__ void mp_x(const GridDev& G, int g, int vb, long long ntot, double inv, double* x,
+                                     const float* e32) {
+    FOR_CELLS_OF(G, g, c, vb) {
+        double t[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) t[a] = x[a * ntot + c.k] + (double)e32[a * ntot + c.k] * inv;
+#pragma unroll
+        for (int a = 0; a < 3; a++) x[a * ntot + c.k] = t[a];
+    }
+}
+
+// r = b - A x (FP64); (r, r).
+template <typename A>
+__device__ __forceinline__ void mp_r(const GridDev& G, int g, int vb, long long ntot, const double* b, A x, double* r,
+                                     double v[1]) {
+    v[0] = 0.0;
+    FOR_CELLS_OF(G, g, c, vb) {
+        double rn[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const A X = x + a * ntot;
+            const double Ax = G.c0 * X[c.k] - G.cx * nbx(X, c, a) - G.cy * (X[c.kn] + X[c.ks]);
+            rn[a] = b[a * ntot + c.k] - Ax;
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            r[a * ntot + c.k] = rn[a];
+            v[0] += rn[a] * rn[a];
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kFieldThreads)
 k_mp_begin(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids,
            int nblk_total, long long ntot, const double* __restrict__ r, float* __restrict__ r32,
@@ -1022,21 +1170,8 @@ k_mp_begin(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
     if (!cg[g].active) return;
     const GridDev& G = grids[g];
     const double scale = sqrt(3.0 * G.ncell / cg[g].rr);  // r32 of unit RMS
-    float acc = 0.f, acc2 = 0.f;
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot + c.k;
-            const float f = (float)(r[o] * scale);
-            const float z = (float)(precond_at(G, r + a * ntot, c, a) * scale);
-            r32[o] = f;
-            z32[o] = z;
-            e32[o] = 0.f;
-            acc = fmaf(f, f, acc);
-            acc2 = fmaf(f, z, acc2);
-        }
-    }
-    double v[2] = {(double)acc, (double)acc2};
+    double v[2];
+    mp_begin(G, g, blockIdx.x, ntot, scale, r, r32, z32, e32, v);
     double tot[2];
     if (!reduce_and_finish<2>(G, g, v, part, nblk_total, done, tot)) return;
     if (threadIdx.x == 0) {
@@ -1054,7 +1189,7 @@ k_mp_begin(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
     finish_all_grids<true>(ngrids, (int)n_part, cg, st, cond_in, use_cond);
 }
 
-// p = z + beta p, q = A z + beta q (= A p); alpha = (r, z) / (p, q).
+// alpha = (r, z) / (p, q)
 __global__ void __launch_bounds__(kFieldThreads)
 k_mp_direction(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids,
                int nblk_total, long long ntot, const float* __restrict__ z32, float* __restrict__ p32,
@@ -1063,36 +1198,14 @@ k_mp_direction(const GridDev* __restrict__ grids, const int* __restrict__ blk_gr
     if (!cg[g].in_active) return;
     const GridDev& G = grids[g];
     const float beta = (float)cg[g].beta_in;
-    const float c0 = (float)G.c0, cx = (float)G.cx, cy = (float)G.cy;
-    float acc = 0.f;  // a thread's few products in FP32, summed across threads in FP64
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot;
-            const float* Z = z32 + o;
-            const float zc = Z[c.k];
-            const float Az = c0 * zc - cx * nbx(Z, c, a) - cy * (Z[c.kn] + Z[c.ks]);
-            float pn, qn;
-            if (beta == 0.f) {
-                pn = zc;
-                qn = Az;
-            } else {
-                pn = fmaf(beta, p32[o + c.k], zc);
-                qn = fmaf(beta, q32[o + c.k], Az);
-            }
-            p32[o + c.k] = pn;
-            q32[o + c.k] = qn;
-            acc = fmaf(pn, qn, acc);
-        }
-    }
-    double v[1] = {(double)acc};
+    double v[1];
+    mp_direction(G, g, blockIdx.x, ntot, beta, z32, p32, q32, v);
     double tot[1];
     if (!reduce_and_finish<1>(G, g, v, part, nblk_total, done, tot)) return;
     if (threadIdx.x == 0) cg[g].alpha_in = cg[g].rz_in / tot[0];
 }
 
-// r' = r - alpha q into the other residual buffer, e += alpha p, z = M r' (formed from r
-// and q at the neighbours, which this kernel does not change); beta = (r', z) / (r, z).
+// beta = (r', z) / (r, z)
 __global__ void __launch_bounds__(kFieldThreads)
 k_mp_update(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids,
             int nblk_total, long long ntot, float* __restrict__ e32, float* __restrict__ r32a,
@@ -1104,31 +1217,9 @@ k_mp_update(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid,
     if (!cg[g].in_active) return;
     const GridDev& G = grids[g];
     const float alpha = (float)cg[g].alpha_in;
-    const float pc0 = (float)G.pc0, pcx = (float)G.pcx, pcy = (float)G.pcy;
     const bool odd = cg[g].in_iters & 1;  // buffer b holds r after an odd number of updates
-    const float* Rc = odd ? r32b : r32a;
-    float* Rn = odd ? r32a : r32b;
-    float acc = 0.f, acc2 = 0.f;
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot;
-            const float* R = Rc + o;
-            const float* Q = q32 + o;
-            const auto w = [&](long long k) { return fmaf(-alpha, Q[k], R[k]); };
-            const float wc = w(c.k);
-            float wx;  // sum of the two x-neighbours, images at the walls as in nbx
-            if (a == 0) wx = (c.ew ? 0.f : w(c.ke)) + (c.ww ? -w(c.k + 1) : w(c.kw));
-            else wx = (c.ew ? wc : w(c.ke)) + (c.ww ? wc : w(c.kw));
-            const float z = fmaf(pc0, wc, fmaf(pcx, wx, pcy * (w(c.kn) + w(c.ks))));
-            Rn[o + c.k] = wc;
-            z32[o + c.k] = z;
-            e32[o + c.k] = fmaf(alpha, p32[o + c.k], e32[o + c.k]);
-            acc = fmaf(wc, wc, acc);
-            acc2 = fmaf(wc, z, acc2);
-        }
-    }
-    double v[2] = {(double)acc, (double)acc2};
+    double v[2];
+    mp_update(G, g, blockIdx.x, ntot, alpha, (const float*)(odd ? r32b : r32a), odd ? r32a : r32b, q32, p32, z32, e32, v);
     double tot[2];
     if (!reduce_and_finish<2>(G, g, v, part, nblk_total, done, tot)) return;
     if (threadIdx.x == 0) {
@@ -1152,11 +1243,7 @@ k_mp_x(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, long
     const int g = blk_grid[blockIdx.x];
     if (!cg[g].active) return;
     const GridDev& G = grids[g];
-    const double inv = 1.0 / cg[g].in_scale;
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) x[a * ntot + c.k] += (double)e32[a * ntot + c.k] * inv;
-    }
+    mp_x(G, g, blockIdx.x, ntot, 1.0 / cg[g].in_scale, x, e32);
 }
 
 // r = b - A x (FP64) and the outer convergence test.
@@ -1169,18 +1256,8 @@ k_mp_r(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int 
     const unsigned n_part = st->n_active;
     if (!cg[g].active) return;
     const GridDev& G = grids[g];
-    double v[1] = {0.0};
-    FOR_CELLS(G, g, c) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const long long o = a * ntot;
-            const double* X = x + o;
-            const double Ax = G.c0 * X[c.k] - G.cx * nbx(X, c, a) - G.cy * (X[c.kn] + X[c.ks]);
-            const double rn = b[o + c.k] - Ax;
-            r[o + c.k] = rn;
-            v[0] += rn * rn;
-        }
-    }
+    double v[1];
+    mp_r(G, g, blockIdx.x, ntot, b, x, r, v);
     double tot[1];
     if (!reduce_and_finish<1>(G, g, v, part, nblk_total, done, tot)) return;
     if (threadIdx.x == 0) {
@@ -1198,6 +1275,157 @@ k_mp_r(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int 
         }
     }
     finish_all_grids(ngrids, (int)n_part, cg, st, cond, use_cond, 1);
+}
+
+// The whole solve of the kernels above as one cooperative kernel, for grids whose nx is no
+// multiple of 4 (the quads of solve_coop.cu's inner solves need one). Blocks take the
+// kernels' blocks in turn, with the same cells per thread, sums of a block and order of the
+// partials: the result has the WHILE node's bits, which matters where FP32 particles
+// amplify the solver's last places over several steps. A grid barrier and one pass over the
+// partials, by every block alike, stand in for the kernel boundary, the last block's sums and
+// the loop condition. Field part of a step, WHILE node and
+// here: 98 x 98 332 and 179 us, 1413 x 247 594 and 451, 2831 x 460 1272 and 1032. Bound by
+// the latency of a phase (a barrier, the partials, one to nine cells in turn per thread).
+// The Chebyshev tiles of solve_coop.cu on single cells were faster (1413 x 247: 250 us) but
+// converge to another point within the tolerance: fields and currents drifted from the WHILE
+// node's by up to 9e-9 in seven steps.
+struct MpSim {
+    double rr, bb, rr_in0, rz, alpha, beta, tol, scale;
+    int active, in_active, iters, in_iters, outer;
+};
+enum MpPhase { kMpBegin, kMpDirection, kMpUpdate, kMpX, kMpR };
+constexpr int kMpMaxGrids = 64;
+
+__global__ void __launch_bounds__(kFieldThreads, 4)
+k_mp_cells(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int ngrids, int nblk, long long ntot,
+           const double* __restrict__ b, double* x, double* r, float* r32a, float* r32b, float* z32, float* p32,
+           float* q32, float* e32, CgState* cg, double* part, unsigned int* bar, DevStatus* st) {
+    __shared__ MpSim sim[kMpMaxGrids];
+    __shared__ double s_v[2][kFieldThreads];
+    if (st->stop) return;  // the same for every block: stop changes only between launches
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned int limit = st->spin_limit ? st->spin_limit : (1u << 22);
+    unsigned int epoch = 0;
+    int set = 0;  // of two sets of partials: a block can be one phase ahead of another
+    for (int g = tid; g < ngrids; g += kFieldThreads) {
+        MpSim s{};
+        s.rr = cg[g].rr;
+        s.bb = cg[g].bb;
+        s.active = cg[g].active;
+        sim[g] = s;
+    }
+    __syncthreads();
+    const auto takes = [&](MpPhase ph, const MpSim& s) {
+        return s.active && (s.in_active || (ph != kMpDirection && ph != kMpUpdate));
+    };
+    const auto any = [&](bool inner) {
+        int n = 0;
+        for (int g = 0; g < ngrids; g++) n += sim[g].active && (!inner || sim[g].in_active);
+        return n > 0;
+    };
+    // one pass, its barrier and, but for x, its sums; false: a barrier ran out
+    const auto phase = [&](const MpPhase ph) {
+        const int nv = ph == kMpBegin || ph == kMpUpdate ? 2 : 1;
+        double* P = part + (size_t)set * 2 * nblk;
+        for (int vb = blockIdx.x; vb < nblk; vb += gridDim.x) {
+            const int g = __ldg(blk_grid + vb);
+            const MpSim& s = sim[g];
+            if (!takes(ph, s)) continue;  // uniform over the block
+            const GridDev& G = grids[g];
+            double v[2] = {0.0, 0.0};
+            if (ph == kMpBegin) mp_begin(G, g, vb, ntot, s.scale, L2View<double>{r}, r32a, z32, e32, v);
+            if (ph == kMpDirection) mp_direction(G, g, vb, ntot, (float)s.beta, L2View<float>{z32}, p32, q32, v);
+            if (ph == kMpUpdate)
+                mp_update(G, g, vb, ntot, (float)s.alpha, L2View<float>{s.in_iters & 1 ? r32b : r32a},
+                          s.in_iters & 1 ? r32a : r32b, L2View<float>{q32}, p32, z32, e32, v);
+            if (ph == kMpX) {
+                mp_x(G, g, vb, ntot, 1.0 / s.scale, x, e32);
+                continue;
+            }
+            if (ph == kMpR) mp_r(G, g, vb, ntot, b, L2View<double>{x}, r, v);
+            s_v[0][tid] = v[0];
+            s_v[1][tid] = v[1];
+            __syncthreads();
+            if (tid < 32 * nv) {
+                const double t = warp_of_block_sum(s_v[warp]);
+                if (lane == 0) P[warp * nblk + vb] = t;
+            }
+            __syncthreads();
+        }
+        if (!grid_barrier(bar, gridDim.x, ++epoch, &st->sync_timeout, limit)) return false;
+        if (ph == kMpX) return true;
+        for (int g = warp; g < ngrids; g += kFieldThreads / 32) {
+            MpSim& s = sim[g];
+            if (!takes(ph, s)) continue;
+            const GridDev& G = grids[g];
+            const double t = partials_sum(P + G.blk_first, G.nblk);
+            const double t2 = nv == 2 ? partials_sum(P + nblk + G.blk_first, G.nblk) : 0.0;
+            __syncwarp();
+            if (lane != 0) continue;
+            if (ph == kMpBegin) {
+                s.rr_in0 = t;
+                s.rz = t2;
+                s.beta = 0.0;
+                s.in_iters = 0;
+                s.tol = fmax(2e-6, 0.5 * G.rtol * sqrt(s.bb / fmax(s.rr, 1e-300)));
+                s.in_active = (t > 0.0 && t2 > 0.0) ? 1 : 0;
+            } else if (ph == kMpDirection) {
+                s.alpha = s.rz / t;
+            } else if (ph == kMpUpdate) {
+                s.beta = t2 / s.rz;
+                s.rz = t2;
+                s.in_iters += 1;
+                s.iters += 1;
+                if (sqrt(t / s.rr_in0) <= s.tol || s.in_iters >= kMaxInnerIters || s.iters >= G.maxit || !(t2 > 0.0))
+                    s.in_active = 0;
+            } else {
+                s.rr = t;
+                s.outer += 1;
+                if (sqrt(t / s.bb) <= G.rtol) {
+                    s.active = 0;
+                } else if (s.iters >= G.maxit || s.outer >= G.maxit) {
+                    s.active = 0;
+                    if (blockIdx.x == 0) {
+                        atomicAdd(&st->cg_noconv, 1u);
+                        st->stop_next = 1u;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        set ^= 1;
+        return true;
+    };
+    bool ok = true;
+    const bool first = blockIdx.x == 0 && tid == 0;
+    while (ok && any(false)) {
+        __syncthreads();
+        for (int g = tid; g < ngrids; g += kFieldThreads)
+            if (sim[g].active) sim[g].scale = sqrt(3.0 * grids[g].ncell / sim[g].rr);  // r32 of unit RMS
+        __syncthreads();
+        ok = phase(kMpBegin);
+        while (ok && any(true)) {
+            ok = phase(kMpDirection) && phase(kMpUpdate);
+            if (first) st->loop_iters[0] += 1ull;
+        }
+        ok = ok && phase(kMpX) && phase(kMpR);
+        if (first) st->loop_iters[1] += 1ull;
+    }
+    if (!ok) {
+        if (tid == 0) st->stop_next = 1u;
+        return;
+    }
+    if (blockIdx.x == 0)
+        for (int g = tid; g < ngrids; g += kFieldThreads) {
+            CgState& c = cg[g];
+            const MpSim& s = sim[g];
+            c.rr = s.rr;
+            if (s.outer) c.rel = sqrt(s.rr / s.bb);
+            c.active = 0;
+            c.iters = s.iters;
+            c.outer = s.outer;
+            c.total_outer += s.outer;
+        }
 }
 
 // After a learned initial guess x0 (every simulation): r = b - A x0 (FP64) and the
@@ -1322,6 +1550,31 @@ void launch_mp_refine(const FieldArgs& a, cudaStream_t s) {
     k_mp_r<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ngrids, a.nblk, a.ntot, a.b,
                                             a.x, a.r, a.cg, a.part, a.done, a.st, a.cond,
                                             a.use_cond);
+}
+
+cudaError_t mp_cells_blocks(int ngrids, int nblk, int dev, int* blocks) {
+    *blocks = 0;
+    int nsm = 0, occ = 0, coop = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mp_cells, kFieldThreads, 0);
+    if (e == cudaSuccess && coop && ngrids <= kMpMaxGrids) *blocks = std::min(nblk, occ * nsm);
+    return e;
+}
+
+cudaError_t launch_mp_cells(const FieldArgs& a, int blocks, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kFieldThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    // (the right-hand side's kernel zeroed the barrier's counter)
+    return cudaLaunchKernelEx(&cfg, k_mp_cells, a.grids, a.blk_grid, a.ngrids, a.nblk, a.ntot, (const double*)a.b, a.x,
+                              a.r, a.r32, a.r32b, a.z32, a.p32, a.q32, a.e32, a.cg, a.part, a.bar, a.st);
 }
 
 void launch_explicit_fields(const FieldArgs& a, cudaStream_t s) {

@@ -296,4 +296,33 @@ __device__ __forceinline__ double warp_of_block_sum(const double* v) {
     return warp_sum(((v[0] + v[32]) + (v[64] + v[96])) + ((v[128] + v[160]) + (v[192] + v[224])));
 }
 
+// Grid-wide barrier of a cooperative launch (all CTAs resident): arrivals on one counter
+// that only grows; the epoch-th barrier is passed when it reaches epoch * nblocks. Bounded:
+// false if the other CTAs did not arrive within `limit` polls; the CTA then leaves the
+// kernel, and so do the others at their next barrier (none waits for ever). 1.3 us on 152
+// CTAs (measured); a counter that is reset, with a generation word and a sleep between
+// polls, took about twice that, a two-level tree of counters more.
+static __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned int epoch, unsigned int* timeout,
+                             unsigned int limit) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        unsigned int seen;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        for (unsigned int it = 0;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+            if (seen >= epoch * nblocks) break;
+            if (++it > limit) {
+                atomicExch(timeout, 1u);
+                ok = 0;
+                break;
+            }
+        }
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
 }  // namespace pic

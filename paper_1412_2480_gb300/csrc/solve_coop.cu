@@ -124,35 +124,6 @@ struct GState {
     DW C0, CX, CY;
 };
 
-// Grid-wide barrier of a cooperative launch (all CTAs resident): arrivals on one counter
-// that only grows; the epoch-th barrier is passed when it reaches epoch * nblocks. Bounded:
-// false if the other CTAs did not arrive within `limit` polls; the CTA then leaves the
-// kernel, and so do the others at their next barrier (none waits for ever). 1.3 us on 152
-// CTAs (measured); a counter that is reset, with a generation word and a sleep between
-// polls, took about twice that, a two-level tree of counters more.
-__device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned int epoch, unsigned int* timeout,
-                             unsigned int limit) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        unsigned int seen;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        for (unsigned int it = 0;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-            if (seen >= epoch * nblocks) break;
-            if (++it > limit) {
-                atomicExch(timeout, 1u);
-                ok = 0;
-                break;
-            }
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 // Sum of a simulation's n partials: value k goes to slot k mod 256, the slots are added in
 // a fixed tree. By a whole block (one slot per thread, the result in warp 0) or by one warp
 // (eight slots per lane), with the same bits.
@@ -589,91 +560,21 @@ __device__ __forceinline__ void residual_quads(const CoopArgs& a, const ChunkC& 
     }
 }
 
-// Any nx: one cell per thread and step, kCellsAhead in flight. Neighbouring cells of a
-// warp's row come from the same lines, so the scalar loads cost issue slots and not traffic.
-constexpr int kCellsAhead = 2;  // (four spill)
-template <int NC>
-__device__ __forceinline__ void residual_cells(const CoopArgs& a, const ChunkC& q, int c0, float (&acc)[NC]) {
-#pragma unroll 1
-    for (int q0 = 0; q0 < kPerThread; q0 += kCellsAhead) {
-        int k[kCellsAhead], kw[kCellsAhead], ke[kCellsAhead], kn[kCellsAhead], ks[kCellsAhead], ii[kCellsAhead];
-#pragma unroll
-        for (int u = 0; u < kCellsAhead; u++) {
-            // (a cell beyond the grid repeats its last one, and counts for nothing)
-            const int l = q.l0 + (q0 + u) * kCoopThreads + (int)threadIdx.x, lc = min(l, q.ncell - 1);
-            const int j = lc / q.nx, i = lc - j * q.nx, row = j * q.nx;
-            ii[u] = i;
-            k[u] = lc;
-            kw[u] = row + (i == 0 ? q.nx - 1 : i - 1);
-            ke[u] = row + (i + 1 == q.nx ? 0 : i + 1);
-            kn[u] = (j + 1 == q.ny ? 0 : j + 1) * q.nx + i;
-            ks[u] = (j == 0 ? q.ny - 1 : j - 1) * q.nx + i;
-        }
-#pragma unroll
-        for (int cc = 0; cc < NC; cc++) {
-            const int c = c0 + cc;
-            const long long o = c * q.ntot + q.off;
-            const float* XH = a.p32 + o;
-            const float* XL = a.q32 + o;
-            DW xc[kCellsAhead], xw[kCellsAhead], xe[kCellsAhead], xn[kCellsAhead], xs[kCellsAhead];
-            double bv[kCellsAhead];
-#pragma unroll
-            for (int u = 0; u < kCellsAhead; u++) {
-                xc[u] = DW{__ldcg(XH + k[u]), __ldcg(XL + k[u])};
-                xw[u] = DW{__ldcg(XH + kw[u]), __ldcg(XL + kw[u])};
-                xe[u] = DW{__ldcg(XH + ke[u]), __ldcg(XL + ke[u])};
-                xn[u] = DW{__ldcg(XH + kn[u]), __ldcg(XL + kn[u])};
-                xs[u] = DW{__ldcg(XH + ks[u]), __ldcg(XL + ks[u])};
-                bv[u] = __ldcg(a.b + o + k[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < kCellsAhead; u++) {
-                if (q.walls) {
-                    if (ii[u] == 0) xw[u] = c == 0 ? dw_neg(xe[u]) : xc[u];
-                    if (ii[u] + 1 == q.nx) xe[u] = c == 0 ? DW{0.f, 0.f} : xc[u];
-                }
-                const DW r = pair_residual(q, xc[u], xw[u], xe[u], xn[u], xs[u], bv[u]);
-                if (q.l0 + (q0 + u) * kCoopThreads + (int)threadIdx.x < q.ncell) {
-                    a.r32[0][o + k[u]] = r.h;
-                    acc[cc] = fmaf(r.h, r.h, acc[cc]);
-                }
-            }
-        }
-    }
-}
-
 // Components c0 .. c0 + NC - 1 of a chunk's pair residual and their partial sums.
-template <bool VEC, int NC>
+template <int NC>
 __device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, int g, int ch, int c0, double* part) {
     const ChunkC q = chunk_consts(a, s, g, ch, 0);
     float acc[NC];
 #pragma unroll
     for (int cc = 0; cc < NC; cc++) acc[cc] = 0.f;
-    if constexpr (VEC) {
-        if (q.l0 + kChunkCells <= q.ncell) {
-            residual_quads<NC, kQuads>(a, q, c0, 0, acc);
-        } else {
-#pragma unroll 1
-            for (int qq = 0; qq < kQuads; qq++)
-                if (q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x) < q.ncell) residual_quads<NC, 1>(a, q, c0, qq, acc);
-        }
+    if (q.l0 + kChunkCells <= q.ncell) {
+        residual_quads<NC, kQuads>(a, q, c0, 0, acc);
     } else {
-        residual_cells<NC>(a, q, c0, acc);
+#pragma unroll 1
+        for (int qq = 0; qq < kQuads; qq++)
+            if (q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x) < q.ncell) residual_quads<NC, 1>(a, q, c0, qq, acc);
     }
     block_sums_dw<NC>(acc, part + c0);
-}
-
-// x = h + l (FP64) on a chunk of any nx.
-__device__ __forceinline__ void join_cells(const CoopArgs& a, const ChunkC& q) {
-#pragma unroll
-    for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int u = 0; u < kPerThread; u++) {
-            const int l = q.l0 + u * kCoopThreads + (int)threadIdx.x;
-            if (l >= q.ncell) continue;
-            const long long o = c * q.ntot + q.off + l;
-            a.x[o] = dw_join({__ldcg(a.p32 + o), __ldcg(a.q32 + o)});
-        }
 }
 
 template <int PH>
@@ -707,11 +608,6 @@ __device__ __forceinline__ void chunk_phase(const CoopArgs& a, const ChunkC& q, 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-template <int BYTES>  // 4 or 8, aligned likewise
-__device__ __forceinline__ void cp_async_small(void* smem, const void* gmem) {
-    const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -750,8 +646,7 @@ __device__ __forceinline__ void cheb_step(const float* __restrict__ src, float* 
     }
 }
 
-// VEC: nx and the simulations' offsets are multiples of 4 cells.
-template <bool VEC, int kChebTileY>
+template <int kChebTileY>
 __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, int g, int t, int c, float* ew) {
     constexpr int kChebRows = ChebTile<kChebTileY>::kRows, kChebCells = ChebTile<kChebTileY>::kCells;
     constexpr int kChebTileCells = ChebTile<kChebTileY>::kInterior;
@@ -785,24 +680,11 @@ __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, in
     float* eb = ew + kChebCells;
     // the interior's x, staged asynchronously during the steps: pairs (h rows, then l
     // rows) or, in the solve's first refinement, FP64 values; rows of kChebTileX, in 16-byte
-    // chunks with VEC (nx, the offsets and X0 are multiples of 4 cells then, so chunks stay
-    // aligned), one value at a time without
+    // chunks (nx, the offsets and X0 are multiples of 4 cells, so chunks stay aligned)
     float* xst = ew + 2 * kChebCells;
     const int nrow = Y1 - Y0, ncol = X1 - X0;
     const long long ob = c * a.ntot + off + (long long)Y0 * nx + X0;
-    if constexpr (!VEC) {
-        for (int q = tid; q < kChebTileCells; q += kCoopThreads) {
-            const int y = q / kChebTileX, xx = q - y * kChebTileX;
-            if (y >= nrow || xx >= ncol) continue;
-            const long long k = ob + (long long)y * nx + xx;
-            if (s.dw) {
-                cp_async_small<4>(xst + q, a.p32 + k);
-                cp_async_small<4>(xst + kChebTileCells + q, a.q32 + k);
-            } else {
-                cp_async_small<8>(reinterpret_cast<double*>(xst) + q, a.x + k);
-            }
-        }
-    } else if (s.dw) {
+    if (s.dw) {
         for (int q = tid; q < 2 * kChebTileY * (kChebTileX / 4); q += kCoopThreads) {
             const int arr = q / (kChebTileY * (kChebTileX / 4)), rem = q - arr * (kChebTileY * (kChebTileX / 4));
             const int y = rem / (kChebTileX / 4), x4 = 4 * (rem - y * (kChebTileX / 4));
@@ -881,9 +763,8 @@ __device__ __forceinline__ void cheb_tile(const CoopArgs& a, const GState& s, in
 // CG inner solve: 4 CTAs per SM (64 registers), 608 resident CTAs, so a 2048 x 512
 // grid (512 chunks) gives every CTA at most one chunk per phase. With Chebyshev tiles
 // (CHEB): 2 CTAs per SM, so that a thread holds its column strip in registers.
-// CHEB, CG: some simulation takes the Chebyshev solve, the CG; VEC: every simulation's nx is a multiple of
-// 4 (the CG needs it); TY: tile height.
-template <bool CHEB, bool CG, bool VEC, int TY>
+// CHEB, CG: some simulation takes the Chebyshev solve, the CG; TY: tile height.
+template <bool CHEB, bool CG, int TY>
 __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __grid_constant__ CoopArgs a) {
     __shared__ GState gs[kCoopMaxGrids];
     __shared__ double red[32], s_slot[kCoopThreads];
@@ -952,8 +833,8 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __
             const int ch = it / a.rsplit;
             const int g = __ldg(a.chunk_grid + ch);
             if (!(gs[g].active && gs[g].dw)) continue;  // uniform over the CTA
-            if (a.rsplit == 3) pair_chunk<VEC, 1>(a, gs[g], g, ch, it - 3 * ch, part + 3 * (size_t)ch);
-            else pair_chunk<VEC, 3>(a, gs[g], g, ch, 0, part + 3 * (size_t)ch);
+            if (a.rsplit == 3) pair_chunk<1>(a, gs[g], g, ch, it - 3 * ch, part + 3 * (size_t)ch);
+            else pair_chunk<3>(a, gs[g], g, ch, 0, part + 3 * (size_t)ch);
         }
     };
     // One pass over this CTA's chunks of the simulations taking part in `ph`, with
@@ -968,8 +849,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __
             float acc1 = 0.f, acc2 = 0.f;
             double accd = 0.0;
             if constexpr (!CG) {  // (no other phase is reached without CG)
-                if constexpr (VEC) chunk_phase<kJoin>(a, q, acc1, acc2, accd);
-                else join_cells(a, q);
+                chunk_phase<kJoin>(a, q, acc1, acc2, accd);
                 continue;
             } else {
                 switch (ph) {
@@ -1121,7 +1001,7 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __
                 const int t = it / 3, c = it - 3 * (it / 3);
                 const int g = __ldg(a.tile_grid + t);
                 if (!(gs[g].active && gs[g].cheb)) continue;  // uniform over the CTA
-                if constexpr (CHEB) cheb_tile<VEC, TY>(a, gs[g], g, t, c, ew);
+                if constexpr (CHEB) cheb_tile<TY>(a, gs[g], g, t, c, ew);
             }
             for (int g = tid; g < a.ngrids; g += blockDim.x)
                 if (gs[g].active && gs[g].cheb) {
@@ -1217,11 +1097,11 @@ size_t window_floats(int ty) {
 
 using CoopKernel = void (*)(const CoopArgs);
 CoopKernel coop_kernel(const CoopSolve& cs) {
-    if (cs.cg_any) return cs.cheb ? k_mp_coop<true, true, true, 64> : k_mp_coop<false, true, true, 64>;
+    if (cs.cg_any) return cs.cheb ? k_mp_coop<true, true, 64> : k_mp_coop<false, true, 64>;
     switch (cs.tile_y) {
-    case 16: return cs.vec ? k_mp_coop<true, false, true, 16> : k_mp_coop<true, false, false, 16>;
-    case 32: return cs.vec ? k_mp_coop<true, false, true, 32> : k_mp_coop<true, false, false, 32>;
-    default: return cs.vec ? k_mp_coop<true, false, true, 64> : k_mp_coop<true, false, false, 64>;
+    case 16: return k_mp_coop<true, false, 16>;
+    case 32: return k_mp_coop<true, false, 32>;
+    default: return k_mp_coop<true, false, 64>;
     }
 }
 
@@ -1247,10 +1127,10 @@ size_t coop_smem(const CoopSolve& cs) {
 int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std::string& err) {
     coop_free(cs);
     if (ngrids > kCoopMaxGrids) return PIC_EINVAL;  // the caller keeps the WHILE-node solve
+    for (int g = 0; g < ngrids; g++)
+        if (hg[g].nx % 4) return PIC_EINVAL;  // quads of 4 cells along x
     std::vector<double> tk((size_t)ngrids * (kChebMaxIt + 1), 0.0);
-    cs->vec = 1;
     for (int g = 0; g < ngrids; g++) {
-        if (hg[g].nx % 4) cs->vec = 0;  // no quads of 4 cells along x
         double* T = tk.data() + (size_t)g * (kChebMaxIt + 1);
         if (cg_inner || !cheb_ok(hg[g])) {
             cs->cg_any = 1;
@@ -1260,10 +1140,6 @@ int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std
         T[0] = 1.0;
         const double ash = std::acosh((double)(float)cheb_sigma(hg[g]));
         for (int k = 1; k <= kChebMaxIt; k++) T[k] = std::cosh(k * ash);
-    }
-    if (!cs->vec && cs->cg_any) {  // the CG's passes run on quads
-        *cs = CoopSolve{};
-        return PIC_EINVAL;
     }
     std::vector<int2> gc(ngrids);
     std::vector<int> cg;
