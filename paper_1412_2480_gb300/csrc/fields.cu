@@ -1648,7 +1648,11 @@ cudaError_t launch_cg(const FieldArgs& a, int ncell, int dev, cudaStream_t s) {
 }
 
 void launch_field_update(const FieldArgs& a, cudaStream_t s) {
-    if (a.Jfix && a.quads)
+    // quads of cells only where they leave every thread one; below that a cell per thread
+    // has four times the threads to hide the same latency (64 x 64: the field
+    // part of a step 66 -> 62 us, 128 x 128 66 -> 61; 2048 x 512 with quads 371, without 379)
+    const bool quads = a.quads && a.ntot / 4 >= (long long)a.nblk * kFieldThreads;
+    if (a.Jfix && quads)
         k_update_E_dw4<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.F, a.Jfix, a.x, a.cg,
                                                         a.st);
     else if (a.Jfix)
@@ -1657,7 +1661,7 @@ void launch_field_update(const FieldArgs& a, cudaStream_t s) {
     else
         k_update_E<double><<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.F,
                                                             a.J64, a.x, a.cg, a.st);
-    if (a.Jfix && a.quads)
+    if (a.Jfix && quads)
         k_update_B4<<<a.nblk, kFieldThreads, 0, s>>>(a.grids, a.blk_grid, a.ntot, a.F, a.x, a.cg, a.st,
                                                      a.F32);
     else
