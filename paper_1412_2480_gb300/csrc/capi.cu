@@ -53,7 +53,7 @@ struct pic_sim {
     CgState* cg = nullptr;
     unsigned int* done = nullptr;
     DevStatus* st = nullptr;
-    DevStatus* host_st = nullptr;    // [2], pinned: the status before and after a chunk of steps
+    DevStatus seen{};                // the counters of steps and loop iterations as last read
     double* tmp = nullptr;  // ntot scratch for conversions (pic_fields of J in MIXED32)
     // FP64 particles, one set of arrays per species (grid units)
     double* pa[2][5] = {{nullptr}};
@@ -922,7 +922,6 @@ int init_handle(const pic_params* prm, int n, pic_sim** out) {
     A(dalloc(&s->cg, s->ngrids));
     A(dalloc(&s->done, s->ngrids));
     A(dalloc(&s->st, 1));
-    A(cudaMallocHost((void**)&s->host_st, 2 * sizeof(DevStatus)));
     A(dalloc(&s->tmp, s->ntot));
     A(dalloc(&s->dgrids, s->ngrids));
     A(dalloc(&s->dblk_grid, s->nblk));
@@ -1256,13 +1255,11 @@ namespace {
 // host re-sorts them into larger bins after a chunk.
 constexpr int kStepChunk = 32;
 
-// One wait per chunk: the status before and after it comes through pinned memory, in
-// stream order with the steps.
+// One wait per chunk, the status being read after it alone: the counters before it are
+// those of the last read (s->seen; pic_profile and pic_restore keep it too).
 int step_chunk(pic_sim* s, int32_t n) {
     // a new chunk starts clean: errors stop the rest of the chunk that raised them, and
     // the call returns
-    DevStatus *before = s->host_st, *after = s->host_st + 1;
-    CK(cudaMemcpyAsync(before, s->st, sizeof *before, cudaMemcpyDeviceToHost, s->stream));
     CK(cudaMemsetAsync(&s->st->stop, 0, sizeof s->st->stop + sizeof s->st->stop_next, s->stream));
     if (s->prm.precision == PIC_MIXED32) {
         int rc = mixed_before_steps(s->mixed, s->stream, s->err);
@@ -1281,12 +1278,13 @@ int step_chunk(pic_sim* s, int32_t n) {
             if (int rc = run_step_direct(s)) return rc;
         }
     }
-    CK(cudaMemcpyAsync(after, s->st, sizeof *after, cudaMemcpyDeviceToHost, s->stream));
+    DevStatus hs{};
+    CK(cudaMemcpyAsync(&hs, s->st, sizeof hs, cudaMemcpyDeviceToHost, s->stream));
     if (int rc = finish_call(s)) return rc;
-    const DevStatus hs = *after;
-    s->steps += (long long)(hs.steps_done - before->steps_done);
-    s->kernels += n * per_step + loop_kernels(s, hs.loop_iters[0] - before->loop_iters[0],
-                                             hs.loop_iters[1] - before->loop_iters[1]);
+    s->steps += (long long)(hs.steps_done - s->seen.steps_done);
+    s->kernels += n * per_step + loop_kernels(s, hs.loop_iters[0] - s->seen.loop_iters[0],
+                                             hs.loop_iters[1] - s->seen.loop_iters[1]);
+    s->seen = hs;
     if (int rc0 = fp64_counts(s)) return rc0;
     int rc = device_errors(s, hs);
     if (rc == PIC_OK && s->prm.precision == PIC_MIXED32) rc = mixed_after_steps(s->mixed, hs, s->stream, s->err);
@@ -1365,6 +1363,7 @@ int profile_chunk(pic_sim* s, int32_t n, double* acc) {
     CK(cudaStreamSynchronize(s->stream));
     s->steps += (long long)(hs.steps_done - steps0);
     s->kernels += n * step_kernels(s, false) + loop_kernels(s, hs.loop_iters[0] - li0, hs.loop_iters[1] - lr0);
+    s->seen = hs;
     if (int rc0 = fp64_counts(s)) return rc0;
     acc[4] += (double)(c1.total_iters - c0.total_iters);
     int rc = device_errors(s, hs);
@@ -1699,6 +1698,7 @@ int pic_restore(pic_sim* s, const char* path) {
     CK(cudaMemcpyAsync(&hs, s->st, sizeof hs, cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     hs.steps_done = (unsigned long long)steps[1];
+    s->seen = hs;
     CK(cudaMemcpyAsync(s->st, &hs, sizeof hs, cudaMemcpyHostToDevice, s->stream));
     s->steps = steps[0];
     launch_fields_to_f32(field_args(s, 0, 0), s->stream);
@@ -1721,7 +1721,6 @@ void pic_free(pic_sim* s) {
                     s->part, s->cg_part, s->cg, s->done, s->st, s->tmp, s->dsegs, s->dblk_seg[0], s->dblk_seg[1],
                     s->bvec, s->r32, s->p32, s->q32, s->e32, s->r32b, s->z32, s->cells_bar};
     for (void* p : ptrs) dfree(p);
-    if (s->host_st) cudaFreeHost(s->host_st);
     for (int sp = 0; sp < 2; sp++)
         for (int a = 0; a < 5; a++) dfree(s->pa[sp][a]);
     if (s->body_stream) cudaStreamDestroy(s->body_stream);
