@@ -97,7 +97,8 @@ extern "C" {
                               every theta in [1/2, 1] and CFL in (0, 1], so 13 steps always
                               reduce the error by 4e3 at least. A simulation asking for
                               cg_rtol < 1e-13 keeps the CG (the pairs resolve about 1e-14 of
-                              ||b||). The same FP64-class test ||r|| <= rtol ||b|| ends the
+                              ||b||), and so does a handle with a grid whose nx is no
+                              multiple of 4 (the graph-driven loop's passes in one kernel). The same FP64-class test ||r|| <= rtol ||b|| ends the
                               solve either way. NO_GRAPH, NO_COOP, EXPLICIT and CG_INNER are
                               per handle: every simulation of a batch gives the same. */
 

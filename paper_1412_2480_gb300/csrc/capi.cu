@@ -3,10 +3,11 @@
 //
 // One step (Sec. 2, Sec. 3 of Ikeya & Matsumoto 2015):
 //   step_begin -> J = 0 -> particle half (gather E^n,B^n; push; move; deposit J^{n+1/2})
-//   -> rhs of Eq. (7) -> WHILE(any simulation active) { PCG iteration } -> E,B update
-//   (Eqs. (5)-(6)) -> step_end.
-// The step is captured once into a CUDA graph whose PCG loop is a WHILE conditional
-// node driven from the device, so pic_step(n) launches n graphs and synchronises once.
+//   -> rhs of Eq. (7) -> the PCG as one cooperative kernel -> E,B update (Eqs. (5)-(6))
+//   -> step_end.
+// The step is captured once into a CUDA graph, so pic_step(n) launches n graphs and
+// synchronises once. (MIXED32 with PIC_NO_COOP: the PCG loop is a WHILE conditional node
+// driven from the device.)
 #include <cuda_runtime.h>
 
 #include <algorithm>

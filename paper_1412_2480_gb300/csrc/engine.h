@@ -80,7 +80,7 @@ cudaError_t launch_mp_cells(const FieldArgs& a, int blocks, cudaStream_t s);
 
 // The MIXED32 solve as one cooperative persistent kernel (solve_coop.cu), used when the
 // device supports cooperative launches and a handle holds at most kCoopMaxGrids
-// simulations; otherwise the WHILE-node solve above runs.
+// simulations, every nx a multiple of 4; otherwise launch_mp_cells or the WHILE node runs.
 constexpr int kCoopMaxGrids = 64;
 struct CoopSolve {
     int2* gchunk = nullptr;       // per simulation: first chunk, chunk count
@@ -95,7 +95,7 @@ struct CoopSolve {
     int tile_y = 0;               // height of the Chebyshev tiles
     int rsplit = 1;               // items per chunk of the pair residual
 };
-// PIC_OK, PIC_EINVAL (not applicable: keep the WHILE-node solve) or PIC_ECUDA. cg_inner:
+// PIC_OK, PIC_EINVAL (not applicable: another form of the solve) or PIC_ECUDA. cg_inner:
 // the inner solve is always the CG (PIC_CG_INNER).
 int coop_create(CoopSolve* cs, const GridDev* hgrids, int ngrids, bool cg_inner, std::string& err);
 // Dynamic shared memory of the cooperative solve's launch.

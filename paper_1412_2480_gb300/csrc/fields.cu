@@ -1284,13 +1284,17 @@ k_mp_r(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, int 
 // amplify the solver's last places over several steps. A grid barrier and one pass over the
 // partials, by every block alike, stand in for the kernel boundary, the last block's sums and
 // the loop condition. Field part of a step, WHILE node and
-// here: 98 x 98 332 and 179 us, 1413 x 247 594 and 451, 2831 x 460 1272 and 1032. Bound by
-// the latency of a phase (a barrier, the partials, one to nine cells in turn per thread).
+// here: 98 x 98 332 and 170 us, 1413 x 247 594 and 423, 2831 x 460 1272 and 980. Bound by
+// the latency of a phase (a barrier, the partials, one to nine cells in turn per thread) and,
+// on large grids, in a refinement's passes by the FP64 pipe. One thread's divisions and roots
+// stood between the phases: the inner test is on the squares, a refinement's scale and its
+// inverse are formed once (98 x 98 179 us before that, 2831 x 460 1032).
 // The Chebyshev tiles of solve_coop.cu on single cells were faster (1413 x 247: 250 us) but
 // converge to another point within the tolerance: fields and currents drifted from the WHILE
 // node's by up to 9e-9 in seven steps.
 struct MpSim {
-    double rr, bb, rr_in0, rz, alpha, beta, tol, scale;
+    double rr, bb, rr_in0, rz, tol, lim, scale, inv;  // lim = tol^2 rr_in0
+    float alphaf, betaf;
     int active, in_active, iters, in_iters, outer;
 };
 enum MpPhase { kMpBegin, kMpDirection, kMpUpdate, kMpX, kMpR };
@@ -1301,7 +1305,7 @@ k_mp_cells(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
            const double* __restrict__ b, double* x, double* r, float* r32a, float* r32b, float* z32, float* p32,
            float* q32, float* e32, CgState* cg, double* part, unsigned int* bar, DevStatus* st) {
     __shared__ MpSim sim[kMpMaxGrids];
-    __shared__ double s_v[2][kFieldThreads];
+    __shared__ double s_v[2][kFieldThreads], s_tot[kMpMaxGrids][2];
     if (st->stop) return;  // the same for every block: stop changes only between launches
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const unsigned int limit = st->spin_limit ? st->spin_limit : (1u << 22);
@@ -1334,12 +1338,12 @@ k_mp_cells(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
             const GridDev& G = grids[g];
             double v[2] = {0.0, 0.0};
             if (ph == kMpBegin) mp_begin(G, g, vb, ntot, s.scale, L2View<double>{r}, r32a, z32, e32, v);
-            if (ph == kMpDirection) mp_direction(G, g, vb, ntot, (float)s.beta, L2View<float>{z32}, p32, q32, v);
+            if (ph == kMpDirection) mp_direction(G, g, vb, ntot, s.betaf, L2View<float>{z32}, p32, q32, v);
             if (ph == kMpUpdate)
-                mp_update(G, g, vb, ntot, (float)s.alpha, L2View<float>{s.in_iters & 1 ? r32b : r32a},
+                mp_update(G, g, vb, ntot, s.alphaf, L2View<float>{s.in_iters & 1 ? r32b : r32a},
                           s.in_iters & 1 ? r32a : r32b, L2View<float>{q32}, p32, z32, e32, v);
             if (ph == kMpX) {
-                mp_x(G, g, vb, ntot, 1.0 / s.scale, x, e32);
+                mp_x(G, g, vb, ntot, s.inv, x, e32);
                 continue;
             }
             if (ph == kMpR) mp_r(G, g, vb, ntot, b, L2View<double>{x}, r, v);
@@ -1354,29 +1358,38 @@ k_mp_cells(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
         }
         if (!grid_barrier(bar, gridDim.x, ++epoch, &st->sync_timeout, limit)) return false;
         if (ph == kMpX) return true;
-        for (int g = warp; g < ngrids; g += kFieldThreads / 32) {
+        // a warp per simulation and sum, then a thread per simulation
+        for (int it = warp; it < ngrids * nv; it += kFieldThreads / 32) {
+            const int g = nv == 2 ? it >> 1 : it, v = nv == 2 ? it & 1 : 0;
+            if (!takes(ph, sim[g])) continue;
+            const double t = partials_sum(P + v * nblk + grids[g].blk_first, grids[g].nblk);
+            if (lane == 0) s_tot[g][v] = t;
+        }
+        __syncthreads();
+        for (int g = tid; g < ngrids; g += kFieldThreads) {
             MpSim& s = sim[g];
             if (!takes(ph, s)) continue;
             const GridDev& G = grids[g];
-            const double t = partials_sum(P + G.blk_first, G.nblk);
-            const double t2 = nv == 2 ? partials_sum(P + nblk + G.blk_first, G.nblk) : 0.0;
-            __syncwarp();
-            if (lane != 0) continue;
+            const double t = s_tot[g][0], t2 = s_tot[g][1];
             if (ph == kMpBegin) {
                 s.rr_in0 = t;
                 s.rz = t2;
-                s.beta = 0.0;
+                s.betaf = 0.f;
                 s.in_iters = 0;
                 s.tol = fmax(2e-6, 0.5 * G.rtol * sqrt(s.bb / fmax(s.rr, 1e-300)));
+                s.lim = s.tol * s.tol * t;
                 s.in_active = (t > 0.0 && t2 > 0.0) ? 1 : 0;
             } else if (ph == kMpDirection) {
-                s.alpha = s.rz / t;
+                s.alphaf = (float)(s.rz / t);
             } else if (ph == kMpUpdate) {
-                s.beta = t2 / s.rz;
+                s.betaf = (float)(t2 / s.rz);
                 s.rz = t2;
                 s.in_iters += 1;
                 s.iters += 1;
-                if (sqrt(t / s.rr_in0) <= s.tol || s.in_iters >= kMaxInnerIters || s.iters >= G.maxit || !(t2 > 0.0))
+                // sqrt(t / rr_in0) <= tol, on the squares unless they are within rounding
+                bool done = t <= s.lim * (1.0 + 1e-12);
+                if (done && t >= s.lim * (1.0 - 1e-12)) done = sqrt(t / s.rr_in0) <= s.tol;
+                if (done || s.in_iters >= kMaxInnerIters || s.iters >= G.maxit || !(t2 > 0.0))
                     s.in_active = 0;
             } else {
                 s.rr = t;
@@ -1401,7 +1414,10 @@ k_mp_cells(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, 
     while (ok && any(false)) {
         __syncthreads();
         for (int g = tid; g < ngrids; g += kFieldThreads)
-            if (sim[g].active) sim[g].scale = sqrt(3.0 * grids[g].ncell / sim[g].rr);  // r32 of unit RMS
+            if (sim[g].active) {
+                sim[g].scale = sqrt(3.0 * grids[g].ncell / sim[g].rr);  // r32 of unit RMS
+                sim[g].inv = 1.0 / sim[g].scale;
+            }
         __syncthreads();
         ok = phase(kMpBegin);
         while (ok && any(true)) {

@@ -30,7 +30,8 @@
 // arithmetic (dword.cuh), so no FP64 instruction is spent inside a refinement; x is
 // joined back to FP64 at the end. A refinement costs two grid barriers (tiles,
 // residual) instead of two per inner iteration. PIC_CG_INNER, or a simulation's
-// cg_rtol below 1e-13, keeps the CG.
+// cg_rtol below 1e-13, keeps the CG. Every nx is a multiple of 4 here; the other grids'
+// solve is k_mp_cells (fields.cu).
 //
 // Work is cut into fixed chunks of 2048 cells of one simulation; a chunk's partial sums
 // are formed in a fixed order and written to its own slot, and every CTA forms each
