@@ -1069,8 +1069,8 @@ __global__ void k_gather_overflow(long long n_over, int gs, Slots O, long long b
 // the tile's window in shared memory; FP64 is left to the window's nodes when the block is
 // done, and to the offsets below 2^-17 that have smaller bits. A window's node holds up to
 // 256 full weights (113 at order 3); what wraps goes to the output at once. 1024 x 256 with 16
-// per cell, order 2 (8.4e6 particles, 101 MB): 376 -> 95 us, bound by the bank conflicts of
-// the two atomics per node (3.3 wavefronts each on random nodes) and the 64-bit products.
+// per cell, order 2 (8.4e6 particles, 101 MB): 376 -> 92 us, bound by instruction issue (69%
+// active: 64-bit products, carries) and the two atomics per node (3.0 wavefronts each).
 // Against exact sums the error is no larger than FP64's at any density from one particle per
 // cell (order 2, 16 per cell: 6e-17 against 3.2e-16, relative to the density's norm).
 struct DensityArgs {
@@ -1107,22 +1107,33 @@ __device__ __noinline__ void density_wrapped(const GridDev& G, int k0, unsigned 
     }
 }
 
+// hi + 1 if l + v passes 2^32, else hi
+__device__ __forceinline__ unsigned carry_into(unsigned l, unsigned v, unsigned hi) {
+    unsigned r;
+    asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %3, 0;\n}\n" : "=r"(r) : "r"(l), "r"(v), "r"(hi));
+    return r;
+}
+
 // 64-bit sums of N neighbouring nodes, each from two 32-bit atomics: the one that sees a word
 // wrap carries. All low words, then all high ones: one wait for each, not for each node.
-// Returns which sums wrapped.
+// Returns which sums wrapped: none while the high words found are below 2^32 - 2^24 - 1, as
+// a contribution's is at most 2^24, and only then is each looked at.
 template <int N>
 __device__ __forceinline__ unsigned density_add(const DensityWin& W, int k, const unsigned long long v[N]) {
-    unsigned l[N], h[N], wrapped = 0;
+    unsigned l[N], h[N], most = 0, wrapped = 0;
 #pragma unroll
     for (int a = 0; a < N; a++) l[a] = atomicAdd(W.lo + k + a, (unsigned)v[a]);
 #pragma unroll
     for (int a = 0; a < N; a++) {
-        const unsigned vh = (unsigned)(v[a] >> 32) + (l[a] + (unsigned)v[a] < l[a] ? 1u : 0u);
-        l[a] = vh;
-        h[a] = atomicAdd(W.hi + k + a, vh);
+        l[a] = carry_into(l[a], (unsigned)v[a], (unsigned)(v[a] >> 32));
+        h[a] = atomicAdd(W.hi + k + a, l[a]);
     }
 #pragma unroll
-    for (int a = 0; a < N; a++) wrapped |= h[a] + l[a] < h[a] ? 1u << a : 0u;
+    for (int a = 0; a < N; a++) most = max(most, h[a]);
+    if (most >= 0xfeffffffu) {
+#pragma unroll
+        for (int a = 0; a < N; a++) wrapped |= h[a] + l[a] < h[a] ? 1u << a : 0u;
+    }
     return wrapped;
 }
 
@@ -1964,7 +1975,7 @@ int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, d
     // Parts of a bin: 4096 particles each (5120 of its capacity) keep the window's cost, its
     // zeroing and its nodes' FP64, below a tenth of the block's time; half as many where that
     // leaves fewer than the eight blocks that an SM holds (512 x 256, 8 per cell: 30 -> 22 us;
-    // 1024 x 256, 16 per cell: 95 us against 101 with the short parts).
+    // 1024 x 256, 16 per cell: 92 us against 98 with the short parts).
     const long long chunk = nbins * std::max(1ll, G.cap / 5120) < 8 * 152 ? 2560 : 5120;
     const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / chunk)));
     const size_t sm = d.rho ? (size_t)2 * G.wx * G.wy * sizeof(unsigned) : 0;
