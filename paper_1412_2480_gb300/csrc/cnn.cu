@@ -188,18 +188,26 @@ constexpr int conv_smem() {
 // rows (tap, ci) x pixels, B = co x pixels, pixels are the reduction dimension. Both X and
 // dY hold a pixel's channels side by side, which is the MN-major operand layout, so the
 // im2col moves 16-byte vectors (as K-major operands every value was a 2-byte store, and one
-// layer took 64 us on 32 CTAs). One more row of A is constant 1: its sums are the bias
-// gradient. A CTA takes its share of one layer's 64-pixel chunks, the fill of one buffer
-// under the MMAs of the other, and leaves its sums in its own slice of `part`; k_finish adds
-// the slices in a fixed order, so gradients are the same on every run.
-// 8 images of 64 x 64, all layers with biases and Adam: 275 -> 32 us (k_wgrad 25, k_finish 7).
+// layer took 64 us on 32 CTAs). A CTA takes its share of one layer's 64-pixel chunks, the
+// fill of one buffer under the MMAs of the other, and leaves its sums in its own slice of
+// `part`; k_finish adds the slices in a fixed order, so gradients are the same on every run.
+//
+// The tensor cores cut each addition to their FP32 accumulator short, always to the same
+// side, so the error of a sum grows with its length: 5e-7 of the sum of magnitudes after 7
+// chunks, 5e-6 after 54, 3e-5 after 216 (16 images of 256 x 256). So no more than kWFlush
+// chunks are added up in tensor memory; the sums then join the slice in FP32, rounded to
+// nearest: errors up to 8e-7 at every batch size, for 2 to 6% of a training step (16 images
+// of 256 x 256: k_wgrad 657 -> 764 us; with 8 chunks 5e-7 and twice that, with 16 1.2e-6). The
+// bias gradient, a plain sum of dY, is formed in FP32 from the vectors as they are staged.
+// 8 images of 64 x 64, the whole training step: 421 us with atomics, 141 here.
 constexpr int kWThreads = 256;
+constexpr int kWFlush = 12;
 constexpr int kWPerLayer = 76;  // CTAs per layer: two per SM over the four layers
 
 template <int CIN, int NOUT>
 struct WShape {
-    static constexpr int kRows = 9 * CIN + 1;  // (tap, ci), then the constant
-    static constexpr int kMT = (kRows + 127) / 128;
+    static constexpr int kRows = 9 * CIN + 1;  // of a slice: (tap, ci), then the bias
+    static constexpr int kMT = (9 * CIN + 127) / 128;
     static constexpr int kABytes = kMT * 128 * kChunk * 2;
     static constexpr int kBBytes = NOUT * kChunk * 2;
     static constexpr int kSlice = kRows * NOUT;
@@ -221,7 +229,7 @@ struct WgradArgs {
 
 template <int CIN, int NOUT>
 __device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int cta, unsigned char* smem, uint64_t* bar,
-                                            uint32_t tmem) {
+                                            uint32_t tmem, float (*s_bias)[32]) {
     using S = WShape<CIN, NOUT>;
     constexpr uint32_t SBO = (kChunk / 8) * 128;
     constexpr int BUF = S::kABytes + S::kBBytes;
@@ -229,24 +237,72 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int c
     const bf16* X = a.X[layer];
     const bf16* dY = a.dY[layer];
     const uint32_t lim = __ldg(a.err + 1);  // the waits' poll limit (0: the default bound)
-    // the constant row and the unused ones behind it
+    float* out = a.part + ((size_t)layer * kWPerLayer + cta) * kWSlice;
+    // the unused rows of A
     for (int q = tid; q < 2 * (S::kMT * 16 - 9 * CIN / 8) * kChunk; q += kWThreads) {
         const int b = q & 1, px = (q >> 1) % kChunk, g = 9 * CIN / 8 + (q >> 1) / kChunk;
-        *reinterpret_cast<uint4*>(smem + b * BUF + tc::mn_offset(8 * g, px, kChunk)) =
-            make_uint4(g == 9 * CIN / 8 ? 0x3F80u : 0u, 0u, 0u, 0u);  // BF16 1.0 in row 9 CIN
+        *reinterpret_cast<uint4*>(smem + b * BUF + tc::mn_offset(8 * g, px, kChunk)) = make_uint4(0u, 0u, 0u, 0u);
     }
     bool ok = true;
     int n = 0;  // chunks issued
+    // the last commit of each buffer
+    const auto wait_all = [&]() {
+        bool w = true;
+        for (int b = 0; b < 2 && b < n; b++)
+            w = tc::mbar_wait_lim(bar + b, (uint32_t)(((n - 1 - b) / 2) & 1), lim) && w;
+        return __syncthreads_and(w ? 1 : 0) != 0;
+    };
+    // the sums in tensor memory become the slice's, or join them (warps 0-3 take the row
+    // tiles 0 and 2, warps 4-7 tile 1; a warp reads the 32 lanes of its place among four)
+    const auto flush = [&](bool first) {
+        const int quad = warp & 3;
+#pragma unroll 1
+        for (int m = warp >> 2; m < S::kMT; m += 2) {
+            float acc[NOUT];
+#pragma unroll
+            for (int cc = 0; cc < NOUT; cc += 16)
+                tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(m * NOUT + cc), acc + cc);
+            const int row = m * 128 + quad * 32 + lane;
+            if (row < 9 * CIN) {
+                float4* o = reinterpret_cast<float4*>(out + (size_t)row * NOUT);
+                float4 old[NOUT / 4];
+#pragma unroll
+                for (int k = 0; k < NOUT / 4; k++) old[k] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : o[k];
+#pragma unroll
+                for (int k = 0; k < NOUT / 4; k++)
+                    o[k] = make_float4(old[k].x + acc[4 * k], old[k].y + acc[4 * k + 1], old[k].z + acc[4 * k + 2],
+                                       old[k].w + acc[4 * k + 3]);
+            }
+            __syncwarp();  // the next load from tensor memory is the whole warp's
+        }
+    };
+    // dY's sums over this thread's pixel of every chunk, eight channels: since the last
+    // flush, and before it
+    float bias[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, bias0[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    constexpr int VX = CIN / 8, VY = NOUT / 8;
+    static_assert(kChunk * VY <= kWThreads, "one vector of dY per thread");
     for (long long c = cta; c < a.nchunks; c += a.ctas, n++) {
         const int b = n & 1;
         unsigned char* sA = smem + b * BUF;
         unsigned char* sB = sA + S::kABytes;
-        if (n >= 2) ok = __syncthreads_and(tc::mbar_wait_lim(bar + b, (uint32_t)((n / 2 - 1) & 1), lim) ? 1 : 0) != 0;
+        if (n > 0 && n % kWFlush == 0) ok = wait_all();
+        else if (n >= 2) ok = __syncthreads_and(tc::mbar_wait_lim(bar + b, (uint32_t)((n / 2 - 1) & 1), lim) ? 1 : 0) != 0;
         if (!ok) break;
+        if (n > 0 && n % kWFlush == 0) {
+            tc::fence_after_sync();
+            flush(n == kWFlush);
+            tc::fence_before_sync();  // the next MMAs overwrite what was read
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                bias0[k] += bias[k];
+                bias[k] = 0.f;
+            }
+        }
         const long long pix0 = c * kChunk;
         const CnnImg im = a.imgs[a.tile_img[pix0 / kTile]];
         const int l0 = (int)(pix0 - im.off);
-        constexpr int VX = CIN / 8, VY = NOUT / 8;
+        uint4 y = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < kChunk * VY) y = __ldg(reinterpret_cast<const uint4*>(dY + (pix0 + tid / VY) * NOUT) + tid % VY);
 #pragma unroll
         for (int q0 = 0; q0 < kChunk * 9 * VX; q0 += kWThreads) {
             const int q = q0 + tid;  // vectors of a pixel side by side, then pixels, then taps
@@ -257,11 +313,7 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int c
             *reinterpret_cast<uint4*>(sA + tc::mn_offset(tap * CIN + 8 * v, px, kChunk)) =
                 __ldg(reinterpret_cast<const uint4*>(X + (im.off + (long long)nj * im.nx + ni) * CIN) + v);
         }
-        for (int q = tid; q < kChunk * VY; q += kWThreads) {
-            const int v = q % VY, px = q / VY;
-            *reinterpret_cast<uint4*>(sB + tc::mn_offset(8 * v, px, kChunk)) =
-                __ldg(reinterpret_cast<const uint4*>(dY + (pix0 + px) * NOUT) + v);
-        }
+        if (tid < kChunk * VY) *reinterpret_cast<uint4*>(sB + tc::mn_offset(8 * (tid % VY), tid / VY, kChunk)) = y;
         tc::fence_smem_to_async();
         __syncthreads();
         if (tid == 0) {
@@ -274,17 +326,17 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int c
                 for (int s = 0; s < kChunk / 16; s++)
                     tc::mma_bf16(tmem + (uint32_t)(m * NOUT),
                                  tc::make_desc(a0 + (uint32_t)m * 128u * kChunk * 2u + s * 256, tc::kLbo, SBO),
-                                 tc::make_desc(b0 + s * 256, tc::kLbo, SBO), idesc, (n > 0 || s > 0) ? 1u : 0u);
+                                 tc::make_desc(b0 + s * 256, tc::kLbo, SBO), idesc, (n % kWFlush > 0 || s > 0) ? 1u : 0u);
             tc::mma_commit(bar + b);
         }
+        const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {  // (a BF16 number is the upper half of an FP32 one)
+            bias[2 * k] += __uint_as_float(w[k] << 16);
+            bias[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
+        }
     }
-    // the last commit of each buffer
-    if (ok) {
-        bool w = true;
-        for (int b = 0; b < 2 && b < n; b++)
-            w = tc::mbar_wait_lim(bar + b, (uint32_t)(((n - 1 - b) / 2) & 1), lim) && w;
-        ok = __syncthreads_and(w ? 1 : 0) != 0;
-    }
+    if (ok) ok = wait_all();
     if (!ok) {  // drain what is in flight before the shared and tensor memory go
         if (tid == 0) {
             for (int b = 0; b < 2 && b < n; b++) tc::mbar_wait(bar + b, (uint32_t)(((n - 1 - b) / 2) & 1));
@@ -293,20 +345,21 @@ __device__ __forceinline__ void wgrad_layer(const WgradArgs& a, int layer, int c
         return;
     }
     tc::fence_after_sync();
-    if (warp >= 4) return;
-    float* out = a.part + ((size_t)layer * kWPerLayer + cta) * kWSlice;
-#pragma unroll 1
-    for (int m = 0; m < S::kMT; m++) {
-        float acc[NOUT];
+    flush(n <= kWFlush);
+    // the bias: lanes that hold the same channels, then the warps
 #pragma unroll
-        for (int cc = 0; cc < NOUT; cc += 16)
-            tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(m * NOUT + cc), acc + cc);
-        const int row = m * 128 + warp * 32 + lane;
-        if (row < S::kRows)
+    for (int k = 0; k < 8; k++) {
+        float t = bias0[k] + bias[k];
 #pragma unroll
-            for (int co = 0; co < NOUT; co += 4)
-                *reinterpret_cast<float4*>(out + (size_t)row * NOUT + co) =
-                    make_float4(acc[co], acc[co + 1], acc[co + 2], acc[co + 3]);
+        for (int o = VY; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane < VY) s_bias[warp][8 * lane + k] = t;
+    }
+    __syncthreads();
+    if (tid < NOUT) {  // (warps without a vector hold zeros)
+        float t[4];
+#pragma unroll
+        for (int w = 0; w < 4; w++) t[w] = s_bias[w][tid] + s_bias[w + 4][tid];
+        out[(size_t)9 * CIN * NOUT + tid] = (t[0] + t[1]) + (t[2] + t[3]);
     }
 }
 
@@ -314,6 +367,7 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t s_tmem;
+    __shared__ float s_bias[kWThreads / 32][32];
     const int tid = threadIdx.x, warp = tid >> 5;
     if (warp == 0) tc::tmem_alloc(&s_tmem, kWCols);
     if (tid == 0) {
@@ -325,9 +379,9 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a) {
     const uint32_t tmem = s_tmem;
     const int layer = blockIdx.x / a.ctas, cta = blockIdx.x - layer * a.ctas;
     switch (layer) {
-    case 0: wgrad_layer<16, 32>(a, 0, cta, smem, bar, tmem); break;
-    case 3: wgrad_layer<32, 16>(a, 3, cta, smem, bar, tmem); break;
-    default: wgrad_layer<32, 32>(a, layer, cta, smem, bar, tmem); break;
+    case 0: wgrad_layer<16, 32>(a, 0, cta, smem, bar, tmem, s_bias); break;
+    case 3: wgrad_layer<32, 16>(a, 3, cta, smem, bar, tmem, s_bias); break;
+    default: wgrad_layer<32, 32>(a, layer, cta, smem, bar, tmem, s_bias); break;
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -448,14 +502,15 @@ __global__ void k_finish(const float* __restrict__ part, int ctas, float* __rest
     const int row = t / y.cout_pad, co = t - row * y.cout_pad, tap = row / y.cin_pad, ci = row - tap * y.cin_pad;
     if (co >= y.cout || (tap < 9 && ci >= y.cin)) return;  // (row 9 cin_pad, tap 9: the bias)
     const float* p = part + (size_t)layer * kWPerLayer * kWSlice + t;
-    float g = 0.f;
-    for (int c = 0; c < ctas; c += 4) {
-        float v[4];
+    float s[4] = {0.f, 0.f, 0.f, 0.f};  // four chains: shorter ones round less
+    for (int c = 0; c < ctas; c += 16) {
+        float v[16];
 #pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = c + k < ctas ? p[(size_t)(c + k) * kWSlice] : 0.f;
+        for (int k = 0; k < 16; k++) v[k] = c + k < ctas ? p[(size_t)(c + k) * kWSlice] : 0.f;
 #pragma unroll
-        for (int k = 0; k < 4; k++) g += v[k];
+        for (int k = 0; k < 16; k++) s[k & 3] += v[k];
     }
+    const float g = (s[0] + s[1]) + (s[2] + s[3]);
     const long long k = tap < 9 ? y.w_off + ((long long)co * 9 + tap) * y.cin + ci : y.b_off + co;
     grads[k] = g;
     if (!u.w || *err) return;
