@@ -8,6 +8,7 @@
 // The step is captured once into a CUDA graph, so pic_step(n) launches n graphs and
 // synchronises once. (MIXED32 with PIC_NO_COOP: the PCG loop is a WHILE conditional node
 // driven from the device.)
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -725,13 +726,30 @@ int charge_density(pic_sim* s, double* rho, double* mom = nullptr, int which = P
     return PIC_OK;
 }
 
-// Whether p is memory of the handle's device that its kernels can write.
-bool on_device(const pic_sim* s, const void* p) {
-    cudaPointerAttributes at{};
-    const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
-                    at.device == s->device;
-    cudaGetLastError();
-    return ok;
+// Whether kernels may write n values at p: memory of the handle's device, aligned for FP64,
+// and all of it inside one allocation. Anything else goes through a copy, which takes any
+// address and checks the range itself; a kernel's store would fault.
+bool on_device(const pic_sim* s, const double* p, long long n) {
+    using GetAttributes = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const GetAttributes get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q);
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<GetAttributes>(f) : nullptr;
+    }();
+    unsigned int type = 0, managed = 0;
+    int dev = -1;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* to[5] = {&type, &managed, &dev, &base, &size};
+    const CUdeviceptr a = reinterpret_cast<CUdeviceptr>(p);
+    // (an address CUDA does not know leaves zeros)
+    return a % sizeof(double) == 0 && get && get(5, what, to, a) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
+           !managed && dev == s->device && base && a >= base && a - base <= size &&
+           (size_t)n <= (size - (size_t)(a - base)) / sizeof(double);
 }
 
 int check_species(pic_sim* s, int sp) {
@@ -1435,7 +1453,7 @@ int pic_fields(pic_sim* s, int32_t which, double* out, size_t len) {
     // what is formed on demand (J, the densities) goes straight into a caller's array on
     // this device
     const double* src = nullptr;
-    if (int rc = field_source(s, which, &src, which >= PIC_JX && on_device(s, out) ? out : nullptr)) return rc;
+    if (int rc = field_source(s, which, &src, which >= PIC_JX && on_device(s, out, nc) ? out : nullptr)) return rc;
     if (src != out) CK(cudaMemcpyAsync(out, src, nc * sizeof(double), cudaMemcpyDefault, s->stream));
     return finish_call(s);
 }
@@ -1532,7 +1550,7 @@ int pic_particles(pic_sim* s, int32_t sp, double* out, int64_t n) {
     // through a temporary of the library's pool
     double* t = nullptr;
     cudaError_t e = cudaSuccess;
-    const bool direct = on_device(s, out);
+    const bool direct = on_device(s, out, 5 * (long long)n);
     if (!direct) e = temp_alloc((void**)&t, 2 * (size_t)n * sizeof(double), s->stream);
     double* pos = direct ? out : t;
     if (e == cudaSuccess) {
