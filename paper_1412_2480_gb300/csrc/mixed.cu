@@ -117,6 +117,7 @@ struct MixedState {
     long long* inj_first = nullptr;  // device [inject_grids + 1]: first thread of each
     long long rebins = 0;
     long long gen = 0;  // allocation generation of the bin buffers
+    bool lost = true;   // no bins, or none that the descriptors and counts fit: nothing may run on them
 };
 
 namespace {
@@ -1479,10 +1480,18 @@ int sort_into_bins(MixedState* m, int g, int par, int s, PartArrays S, long long
     return rc;
 }
 
+// Refuses work on bins that could not be allocated anew: their particles are gone.
+int check_bins(const MixedState* m, std::string& err) {
+    if (!m->lost) return PIC_OK;
+    err = "the particles were lost when their bins could not be allocated; free the handle";
+    return PIC_ESTATE;
+}
+
 // All live particles of species s of simulation g (every bin segment of buffer `par` +
 // its overflow-list entries) into a new staging set.
 int gather_species(MixedState* m, int g, int par, int s, PartArrays& S, long long& n, cudaStream_t st,
                    std::string& err) {
+    if (int rc = check_bins(m, err)) return rc;
     const GridDev& G = m->G[g];
     const long long nb_seg = (long long)G.ntiles * kSegs;
     std::vector<int> cnt(2 * nb_seg);
@@ -1565,7 +1574,11 @@ int plan_items(MixedState* m, std::string& err) {
     }
     if (m->items) cudaFree(m->items);
     m->items = nullptr;
-    MCK(dalloc(&m->items, items.size()));
+    if (dalloc(&m->items, items.size()) != cudaSuccess) {
+        cudaGetLastError();
+        err = "work item allocation failed (" + std::to_string(items.size()) + " items)";
+        return PIC_ENOMEM;
+    }
     MCK(cudaMemcpy(m->items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice));
     return PIC_OK;
 }
@@ -1574,6 +1587,7 @@ int plan_items(MixedState* m, std::string& err) {
 // capacity capo[g] (contents are not preserved; all counts are zeroed).
 int alloc_bins(MixedState* m, const std::vector<long long>& cap, const std::vector<long long>& capo,
                cudaStream_t st, std::string& err) {
+    m->lost = true;  // until the caller has filled them
     for (int p = 0; p < 2; p++) {
         if (m->buf[p]) cudaFree(m->buf[p]);
         m->buf[p] = nullptr;
@@ -1638,6 +1652,7 @@ int place_all(MixedState* m, int par, Staged& A, std::vector<long long> cap, std
     MCK(cudaMemsetAsync(m->injected, 0, 2 * m->ngrids * sizeof(unsigned long long), st));
     MCK(cudaStreamSynchronize(st));
     for (int q = 0; q < 2 * m->ngrids; q++) m->n[q] = A.n[q];
+    m->lost = false;
     return PIC_OK;
 }
 
@@ -1819,6 +1834,7 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         mixed_destroy(m);
         return rc;
     }
+    m->lost = false;
     *out = m;
     return PIC_OK;
 }
@@ -1838,6 +1854,7 @@ void mixed_destroy(MixedState* m) {
 
 int mixed_load(MixedState* m, int g, int s, const double* x, const double* y, const double* ux,
                const double* uy, const double* uz, long long n, cudaStream_t st, std::string& err) {
+    if (int rc = check_bins(m, err)) return rc;
     DevStatus hs{};
     if (int rc = read_status(m, hs, st, err)) return rc;
     // fold any overflow-list particles back into bins first so the list holds none of s
@@ -1921,7 +1938,7 @@ void mixed_enqueue(MixedState* m, cudaStream_t st, int part) {
     }
 }
 
-int mixed_before_steps(MixedState*, cudaStream_t, std::string&) { return PIC_OK; }
+int mixed_before_steps(MixedState* m, cudaStream_t, std::string& err) { return check_bins(m, err); }
 
 int mixed_step_kernels(const MixedState* m) {
     int k = 3;  // k_mixed_begin, k_push_overflow, k_mixed_end
@@ -1969,6 +1986,7 @@ long long mixed_count(MixedState* m, int g, int s) { return m->n[2 * g + s]; }
 
 int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, double* mom, cudaStream_t st,
                        std::string& err) {
+    if (int rc = check_bins(m, err)) return rc;
     const GridDev& G = m->G[g];
     const DensityArgs d{{q_s[0], q_s[1]}, G.w, rho, mom};
     const int nbins = 2 * G.ntiles;
