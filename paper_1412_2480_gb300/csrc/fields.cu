@@ -455,7 +455,7 @@ k_zero_x(const GridDev* __restrict__ grids, const int* __restrict__ blk_grid, lo
 
 // Sum of v over all threads of the grid, the same bits in every block, and a grid-wide
 // barrier: writes before it are visible to loads (of L2) after it. Every block leaves its
-// partial sum, adds one to a counter that only grows, and when the counter says that all
+// partial sum, adds one to a counter (which may wrap: arrivals.h), and when it says that all
 // have, one warp of each block adds the partials in a fixed order. It leaves the sum S and
 // the quotient S / scale (inv: scale / S) in out[0..1] (shared memory): a division repeated
 // by every thread costs as much here as the rest of an iteration. The partials alternate
@@ -480,7 +480,7 @@ __device__ bool grid_sum(double v, double scale, bool inv, double out[2], double
             unsigned int seen;
             for (unsigned int it = 0;;) {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-                if (seen >= epoch * gridDim.x) break;
+                if (all_arrived(seen, epoch, gridDim.x)) break;
                 if (++it > limit) {
                     ok = 0;
                     atomicExch(timeout, 1u);

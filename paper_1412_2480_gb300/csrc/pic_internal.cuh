@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "arrivals.h"
+
 namespace pic {
 
 constexpr double kPi = 3.14159265358979323846;
@@ -297,7 +299,7 @@ __device__ __forceinline__ double warp_of_block_sum(const double* v) {
 }
 
 // Grid-wide barrier of a cooperative launch (all CTAs resident): arrivals on one counter
-// that only grows; the epoch-th barrier is passed when it reaches epoch * nblocks. Bounded:
+// (arrivals.h); the epoch-th barrier is passed when it reaches epoch * nblocks. Bounded:
 // false if the other CTAs did not arrive within `limit` polls; the CTA then leaves the
 // kernel, and so do the others at their next barrier (none waits for ever). 1.3 us on 152
 // CTAs (measured); a counter that is reset, with a generation word and a sleep between
@@ -312,7 +314,7 @@ static __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned 
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         for (unsigned int it = 0;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-            if (seen >= epoch * nblocks) break;
+            if (all_arrived(seen, epoch, nblocks)) break;
             if (++it > limit) {
                 atomicExch(timeout, 1u);
                 ok = 0;
