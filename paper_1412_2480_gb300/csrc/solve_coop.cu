@@ -161,21 +161,22 @@ __device__ __forceinline__ double partials_warp(const double* p, int n) {
     return slot_tree(v);
 }
 
-// Block sums of N values per thread in FP32-pair arithmetic (off the FP64 pipe), as FP64 in
-// out[0..N) of thread 0's choice: warp c finishes value c.
+// Block sums of N FP32 values per thread, added up in FP64, in out[0..N): warp c sums value c,
+// as warp_of_block_sum does.
 template <int N>
-__device__ __forceinline__ void block_sums_dw(const float (&v)[N], double* out) {
-    __shared__ DW s_w[N][kCoopThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void block_sums(const float (&v)[N], double* out) {
+    __shared__ float s_v[N][kCoopThreads];
+    static_assert(kCoopThreads == 256, "eight values per lane");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-    for (int c = 0; c < N; c++) {
-        const DW w = warp_sum_dw(DW{v[c], 0.f});
-        if (lane == 0) s_w[c][warp] = w;
-    }
+    for (int c = 0; c < N; c++) s_v[c][tid] = v[c];
     __syncthreads();
     if (warp < N) {
-        const DW w = warp_sum_dw(lane < kCoopThreads / 32 ? s_w[warp][lane] : DW{0.f, 0.f});
-        if (lane == 0) out[warp] = dw_join(w);
+        double t[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) t[k] = (double)s_v[warp][lane + 32 * k];
+        const double s = warp_sum(((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7])));
+        if (lane == 0) out[warp] = s;
     }
     __syncthreads();
 }
@@ -575,7 +576,7 @@ __device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, i
         for (int qq = 0; qq < kQuads; qq++)
             if (q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x) < q.ncell) residual_quads<NC, 1>(a, q, c0, qq, acc);
     }
-    block_sums_dw<NC>(acc, part + c0);
+    block_sums<NC>(acc, part + c0);
 }
 
 template <int PH>
