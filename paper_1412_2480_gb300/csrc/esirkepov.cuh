@@ -189,52 +189,4 @@ __device__ __forceinline__ void deposit_rho(const GridDev& G, int i, double fx, 
     }
 }
 
-// The product's upper 64 bits, off by less than 3/4 either way (the lower halves' product
-// left out, its mean added).
-__device__ __forceinline__ unsigned long long mul_hi(unsigned long long x, unsigned long long y) {
-    const unsigned x0 = (unsigned)x, x1 = (unsigned)(x >> 32), y0 = (unsigned)y, y1 = (unsigned)(y >> 32);
-    const unsigned long long t = (unsigned long long)x1 * y0 + 0xC0000000ull;
-    const unsigned long long u = (unsigned long long)x0 * y1 + (unsigned)t;
-    return (unsigned long long)x1 * y1 + (t >> 32) + (u >> 32);
-}
-
-// An FP32 offset in [0, 1) as a whole number of 2^-40; false where it needs smaller units
-// (below 2^-17, and not zero).
-__device__ __forceinline__ bool offset_fixed(float f, unsigned long long& F) {
-    const unsigned b = __float_as_uint(f);
-    const int sh = (int)(b >> 23) - 110;
-    F = sh < 0 ? 0ull : (unsigned long long)((b & 0x7fffffu) | 0x800000u) << sh;
-    return sh >= 0 || b == 0u;
-}
-
-// The weights of an offset of F 2^-40 as whole numbers: of 2^-60 at orders 1 and 2, six
-// times the weight in 2^-58 at order 3. They add up to one exactly; each is within 4 units.
-template <int P>
-__device__ __forceinline__ void rho_weights_fixed(int i, unsigned long long F, int& base, unsigned long long w[P + 1]) {
-    constexpr unsigned long long one = 1ull << 40;
-    if constexpr (P == 1) {
-        base = i;
-        w[0] = (one - F) << 20;
-        w[1] = F << 20;
-    } else if constexpr (P == 2) {  // 1/2 (1/2 -+ d)^2 and the rest, d from the nearest node
-        const bool up = F >= one / 2;
-        base = up ? i : i - 1;
-        const unsigned long long hm = (up ? one / 2 + one : one / 2) - F, hp = one - hm;
-        w[0] = mul_hi(hm << 23, hm << 23) >> 3;
-        w[2] = mul_hi(hp << 23, hp << 23) >> 3;
-        w[1] = (1ull << 60) - w[0] - w[2];
-    } else {  // f^3, (1-f)^3, 4 - 6 f^2 + 3 f^3 and the rest
-        base = i - 1;
-        const unsigned long long f = F << 23, g = (one - F) << 23;  // of 2^-63
-        const unsigned long long f2 = mul_hi(f, f), f3 = mul_hi(f2 << 1, f), g3 = mul_hi(mul_hi(g, g) << 1, g);
-        w[3] = f3 >> 4;
-        w[0] = g3 >> 4;
-        w[1] = (1ull << 60) - 3 * (f2 >> 3) + 3 * (f3 >> 4);
-        w[2] = (6ull << 58) - w[0] - w[1] - w[3];
-    }
-}
-// the upper 64 bits of a product of two of them: units per full weight
-template <int P>
-constexpr double kRhoUnits = P == 3 ? 36.0 * 4503599627370496.0 : 72057594037927936.0;  // 36 x 2^52, 2^56
-
 }  // namespace pic

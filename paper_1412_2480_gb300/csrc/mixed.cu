@@ -36,6 +36,7 @@
 #include <mutex>
 #include <vector>
 
+#include "density_fixed.h"
 #include "esirkepov.cuh"
 #include "inject.cuh"
 #include "mixed.h"
@@ -1065,15 +1066,20 @@ __global__ void k_gather_overflow(long long n_over, int gs, Slots O, long long b
 // not asked for.
 //
 // In FP64 throughout the kernel was bound by that pipe (two lanes per cycle and SM, 28
-// operations per particle at order 2: 376 us for 8.4e6 particles). Here weights and their
-// products are 64-bit whole numbers, exact to 2^-56 of a full weight, and so are the sums in
-// the tile's window in shared memory; FP64 is left to the window's nodes when the block is
-// done, and to the offsets below 2^-17 that have smaller bits. A window's node holds up to
-// 256 full weights (113 at order 3); what wraps goes to the output at once. 1024 x 256 with 16
-// per cell, order 2 (8.4e6 particles, 101 MB): 376 -> 92 us, bound by instruction issue (69%
-// active: 64-bit products, carries) and the two atomics per node (3.0 wavefronts each).
-// Against exact sums the error is no larger than FP64's at any density from one particle per
-// cell (order 2, 16 per cell: 6e-17 against 3.2e-16, relative to the density's norm).
+// operations per particle at order 2: 376 us for 8.4e6 particles). Here contributions are whole
+// numbers that keep their relative accuracy (density_fixed.h), and so are the sums in the
+// tile's window in shared memory: 96 bits, which hold a contribution of 2^-34 to 53 places and
+// a sum of 256 full weights (what wraps goes to the output at once). FP64 is left to the
+// window's nodes when the block is done and to the particles that density_contributions
+// refuses (1% at order 2, 3.5% at order 3 of random ones), which wait until then: one of them
+// would cost its whole warp the FP64 path. So every node's density, also one that only the far
+// edges of shapes reach, is as accurate as a sum in FP64 or better (order 2, 16 per cell: 9e-17
+// against 3.2e-16, relative to the density's norm; 200 particles on 64 x 48 cells: 2e-16 of
+// each node at most, both).
+// 1024 x 256 with 16 per cell (8.4e6 particles, 101 MB), order 2: 118 us, bound by instruction
+// issue (64% active; 360 instructions per 32 particles) and by the three atomics per node (3.0
+// wavefronts each); order 3 216 us. With 64-bit sums, exact to 2^-56 of a full weight, they
+// were 106 and 199 us, but the sparse plasma's nodes were off by up to 1e-10 of themselves.
 struct DensityArgs {
     double q[2], w;
     double *rho, *mom;
@@ -1093,99 +1099,91 @@ __device__ __forceinline__ void density_node(const GridDev& G, int ix, int iy, d
 }
 
 struct DensityWin {
-    unsigned *lo, *hi;  // words of the sums, wx per row
-    int wx, X0, Y0;     // the window's row length and first node
+    unsigned* w;         // words of the sums: wx per row, then the next word's plane of nw
+    int wx, nw, X0, Y0;  // the window's row length, size and first node
     double unit;
     double* rho;
 };
 
-// the sums of window nodes k0 + (bit / 4) wx + bit % 4 passed 2^64 units
+// the sums of window nodes k0 + (bit / 4) wx + bit % 4 passed 2^96 units
 __device__ __noinline__ void density_wrapped(const GridDev& G, int k0, unsigned bits, int X0, int Y0, double unit,
                                              double* rho) {
     for (; bits; bits &= bits - 1) {
         const int n = __ffs(bits) - 1, k = k0 + (n >> 2) * G.wx + (n & 3);
-        density_node(G, X0 + k % G.wx, Y0 + k / G.wx, unit * 18446744073709551616.0, rho);
+        density_node(G, X0 + k % G.wx, Y0 + k / G.wx, unit * 79228162514264337593543950336.0, rho);
     }
 }
 
-// hi + 1 if l + v passes 2^32, else hi
-__device__ __forceinline__ unsigned carry_into(unsigned l, unsigned v, unsigned hi) {
-    unsigned r;
-    asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %3, 0;\n}\n" : "=r"(r) : "r"(l), "r"(v), "r"(hi));
-    return r;
+// v (of one or two words) and the carry of l + u
+__device__ __forceinline__ void carry_into(unsigned l, unsigned u, unsigned& v0, unsigned& v1) {
+    asm("{\n .reg .u32 t;\n add.cc.u32 t, %2, %3;\n addc.cc.u32 %0, %0, 0;\n addc.u32 %1, %1, 0;\n}\n"
+        : "+r"(v0), "+r"(v1)
+        : "r"(l), "r"(u));
+}
+__device__ __forceinline__ void carry_into(unsigned l, unsigned u, unsigned& v) {
+    asm("{\n .reg .u32 t;\n add.cc.u32 t, %1, %2;\n addc.u32 %0, %0, 0;\n}\n" : "+r"(v) : "r"(l), "r"(u));
 }
 
-// 64-bit sums of N neighbouring nodes, each from two 32-bit atomics: the one that sees a word
-// wrap carries. All low words, then all high ones: one wait for each, not for each node.
-// Returns which sums wrapped: none while the high words found are below 2^32 - 2^24 - 1, as
-// a contribution's is at most 2^24, and only then is each looked at.
-template <int N>
-__device__ __forceinline__ unsigned density_add(const DensityWin& W, int k, const unsigned long long v[N]) {
-    unsigned l[N], h[N], most = 0, wrapped = 0;
+// 96-bit sums of a row's nodes, each from three 32-bit atomics: the one that sees a word wrap
+// carries. All lowest words, then all middle and all highest ones: one wait for each, not for
+// each node. At order 1 the highest word gets carries only. Returns which sums wrapped: none
+// while the high words found are below 2^32 - 2^24 - 1, as a contribution's is at most 2^24 and
+// a carry, and only then is each looked at (at order 1 it would take 2^34 particles).
+template <int P>
+__device__ __forceinline__ unsigned density_add(const DensityWin& W, int k, const Words (&v)[P + 1]) {
+    unsigned l[P + 1], mid[P + 1], hi[P + 1], most = 0, wrapped = 0;
+    unsigned* w = W.w + k;
 #pragma unroll
-    for (int a = 0; a < N; a++) l[a] = atomicAdd(W.lo + k + a, (unsigned)v[a]);
+    for (int a = 0; a <= P; a++) l[a] = atomicAdd(w + a, v[a].w[0]);
+    w += W.nw;
 #pragma unroll
-    for (int a = 0; a < N; a++) {
-        l[a] = carry_into(l[a], (unsigned)v[a], (unsigned)(v[a] >> 32));
-        h[a] = atomicAdd(W.hi + k + a, l[a]);
+    for (int a = 0; a <= P; a++) {
+        mid[a] = v[a].w[1];
+        hi[a] = v[a].w[2];
+        if (P == 1) carry_into(l[a], v[a].w[0], mid[a]);  // (its contributions' middle word is below 2^31)
+        else carry_into(l[a], v[a].w[0], mid[a], hi[a]);
+        l[a] = atomicAdd(w + a, mid[a]);
     }
+    w += W.nw;
 #pragma unroll
-    for (int a = 0; a < N; a++) most = max(most, h[a]);
-    if (most >= 0xfeffffffu) {
+    for (int a = 0; a <= P; a++) {
+        carry_into(l[a], mid[a], hi[a]);
+        if (P == 1) {
+            if (hi[a]) atomicAdd(w + a, hi[a]);
+        } else {
+            l[a] = atomicAdd(w + a, hi[a]);
+            most = max(most, l[a]);
+        }
+    }
+    if (P > 1 && most >= 0xfeffffffu) {
 #pragma unroll
-        for (int a = 0; a < N; a++) wrapped |= h[a] + l[a] < h[a] ? 1u << a : 0u;
+        for (int a = 0; a <= P; a++) wrapped |= l[a] + hi[a] < l[a] ? 1u << a : 0u;
     }
     return wrapped;
 }
 
-// The weights of each axis add up to one, so the products of one column and one row (the
-// middle ones: the largest weight, at order 1 the lower node's) follow from the others by
-// subtraction: 4 products instead of 9 at order 2, and a particle's charge is exact. A
-// product a few units from zero may come out below it: cut there, but for the middle one's
-// own, which is at least 2^8 units.
 template <int P>
-__device__ __forceinline__ void density_window(const GridDev& G, const DensityWin& W, int i, unsigned long long fx,
-                                               int j, unsigned long long fy) {
-    constexpr int C = P == 1 ? 0 : 1;
-    constexpr int one = P == 3 ? 3 : 0;  // the weights' sum is 2^60, at order 3 6 x 2^58
-    int bx, by;
-    unsigned long long X[P + 1], Y[P + 1];
-    rho_weights_fixed<P>(i, fx, bx, X);
-    rho_weights_fixed<P>(j, fy, by, Y);
-    const int k0 = by * W.wx + bx;
-    const auto whole = [&](unsigned long long w) { return one ? (w >> 5) * 3 : w >> 4; };  // w times the sum
-    const auto cut = [](unsigned long long v) { return (long long)v < 0 ? 0ull : v; };
-    unsigned long long mid[P + 1];  // the middle row
+__device__ __forceinline__ bool density_window(const GridDev& G, const DensityWin& W, int i, unsigned Fx, int j,
+                                               unsigned Fy) {
     unsigned wrapped = 0;
-#pragma unroll
-    for (int a = 0; a <= P; a++) mid[a] = whole(X[a]);
-#pragma unroll
-    for (int b = 0; b <= P; b++) {
-        if (b == C) continue;
-        unsigned long long v[P + 1];
-        v[C] = whole(Y[b]);
-#pragma unroll
-        for (int a = 0; a <= P; a++) {
-            if (a == C) continue;
-            v[a] = mul_hi(X[a], Y[b]);
-            v[C] -= v[a];
-            mid[a] -= v[a];
-        }
-        v[C] = cut(v[C]);
-        mid[C] -= v[C];
-        wrapped |= density_add<P + 1>(W, k0 + b * W.wx, v) << 4 * b;
-    }
-#pragma unroll
-    for (int a = 0; a <= P; a++)
-        if (a != C) mid[a] = cut(mid[a]);
-    wrapped |= density_add<P + 1>(W, k0 + C * W.wx, mid) << 4 * C;
+    int k0 = 0;
+    const bool ok = density_contributions<P>(i, Fx, j, Fy, [&](int bx, int by, int r, const Words (&v)[P + 1]) {
+        k0 = by * W.wx + bx;
+        wrapped |= density_add<P>(W, k0 + r * W.wx, v) << 4 * r;
+    });
     if (wrapped) density_wrapped(G, k0, wrapped, W.X0, W.Y0, W.unit, W.rho);
+    return ok;
 }
 
-template <int P>
+constexpr int kDensityRare = 256;  // particles of a block kept for the end
+
+// MOM: with the momentum. (Not a test in the loop: its FP64 instructions then went through the
+// pipe without effect, 6 per 32 particles: 138 instead of 118 us.)
+template <int P, bool MOM>
 __global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int nbins, const DensityArgs d) {
-    extern __shared__ unsigned dens_win[];  // [2][wx * wy]: low and high words
-    __shared__ double s_m[3][256];
+    extern __shared__ unsigned dens_win[];  // [3][wx * wy]: words of the sums
+    __shared__ long long s_rare[kDensityRare];
+    __shared__ int s_nrare;
     const GridDev& G = a.grids[g];
     const DevStatus* st = a.st;
     const int par = (int)st->parity;
@@ -1202,15 +1200,19 @@ __global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int n
         const long long bin = 2ll * t + s;
         const double q = s ? d.q[1] : d.q[0];
         double* rho = q != 0.0 ? d.rho : nullptr;
-        if (!(d.mom || rho)) return;
+        if (!(MOM || rho)) return;
         const unsigned* B = par ? a.buf[1] : a.buf[0];
         const float* F = reinterpret_cast<const float*>(B);
         const int* cnt = (par ? a.cnt[1] : a.cnt[0]) + ((long long)G.tile_first * 2 + bin) * kSegs;
         const int X0 = t % G.ntx * G.tx, Y0 = t / G.ntx * G.ty, NW = G.wx * G.wy;
         const int nx = G.nx, ny = G.ny, tx = G.tx, ty = G.ty;
-        const DensityWin W{dens_win, dens_win + NW, G.wx, X0 - 2, Y0 - 2, q / kRhoUnits<P>, rho};
+        // a unit of the words (density_fixed.h)
+        const double unit = P == 1 ? q / 4611686018427387904.0
+                                   : q * ((P == 3 ? 4.0 / 9.0 : 1.0) / 309485009821345068724781056.0);
+        const DensityWin W{dens_win, G.wx, NW, X0 - 2, Y0 - 2, unit, rho};
         if (rho)
-            for (int k = tid; k < 2 * NW; k += 256) dens_win[k] = 0u;
+            for (int k = tid; k < 3 * NW; k += 256) dens_win[k] = 0u;
+        if (tid == 0) s_nrare = 0;
         __syncthreads();
         long long base = G.bin_off + bin * bin_stride(G);
         for (int k = 0; k < kSegs; k++) {
@@ -1226,22 +1228,36 @@ __global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int n
                     else if (i > tx + 2) i -= nx;
                     if (j < 1) j += ny;
                     else if (j > ty + 2) j -= ny;
-                    unsigned long long Fx, Fy;
-                    const bool fine = offset_fixed(fx, Fx) && offset_fixed(fy, Fy);
-                    if (fine && i >= 1 && i <= tx + 2 && j >= 1 && j <= ty + 2)
-                        density_window<P>(G, W, i, Fx, j, Fy);
-                    else
-                        density_global<P>(G, c, fx, fy, q, rho);
+                    unsigned Fx, Fy;
+                    const bool fine = fixed_offset(__float_as_uint(fx), Fx) & fixed_offset(__float_as_uint(fy), Fy);
+                    if (!(fine && i >= 1 && i <= tx + 2 && j >= 1 && j <= ty + 2 && density_window<P>(G, W, i, Fx, j, Fy))) {
+                        const int e = atomicAdd(&s_nrare, 1);
+                        if (e < kDensityRare) s_rare[e] = base + v;
+                        else density_global<P>(G, c, fx, fy, q, rho);
+                    }
                 }
-                if (d.mom) momentum(F, base + v);
+                if (MOM) momentum(F, base + v);
             }
             base += lim;
         }
         if (rho) {
             __syncthreads();
+            // (kept for now: a warp of them costs what one of them would have cost its warp)
+            for (int e = tid; e < min(s_nrare, kDensityRare); e += 256) {
+                const long long k = s_rare[e];
+                density_global<P>(G, (int)B[aos(k, 0)], F[aos(k, 1)], F[aos(k, 2)], q, rho);
+            }
             for (int k = tid; k < NW; k += 256) {
-                const unsigned long long v = (unsigned long long)W.hi[k] << 32 | W.lo[k];
-                if (v) density_node(G, W.X0 + k % G.wx, W.Y0 + k / G.wx, W.unit * (double)v, rho);
+                // the sum's leading 64 bits: one conversion and one product in FP64, the power
+                // of two into the exponent
+                const unsigned w0 = W.w[k], w1 = W.w[NW + k], w2 = W.w[2 * NW + k];
+                const int lead = clz32(w2), e = 32 - lead;  // (e = 0: w2 = 0)
+                const u64 v = e ? (u64)__funnelshift_l(w1, w2, lead) << 32 | __funnelshift_l(w0, w1, lead) : (u64)w1 << 32 | w0;
+                if (v) {
+                    const double x = W.unit * (double)v;
+                    density_node(G, W.X0 + k % G.wx, W.Y0 + k / G.wx,
+                                 __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x)), rho);
+                }
             }
         }
     } else {
@@ -1254,17 +1270,23 @@ __global__ void __launch_bounds__(256) k_density(const MixedArgs a, int g, int n
             const double q = gs & 1 ? d.q[1] : d.q[0];
             if (d.rho && q != 0.0)
                 density_global<P>(G, (int)O.p[aos(k, 0)], F[aos(k, 1)], F[aos(k, 2)], q, d.rho);
-            if (d.mom) momentum(F, k);
+            if (MOM) momentum(F, k);
         }
     }
-    if (!d.mom) return;
+    if constexpr (MOM) {
+        __shared__ double s_m[3][256];
 #pragma unroll
-    for (int c = 0; c < 3; c++) s_m[c][tid] = m[c];
-    __syncthreads();
-    if (tid >= 96) return;
-    const double t = warp_of_block_sum(s_m[tid >> 5]);
-    if ((tid & 31) == 0 && t != 0.0) atomicAdd(d.mom + (tid >> 5), d.w * t);
+        for (int c = 0; c < 3; c++) s_m[c][tid] = m[c];
+        __syncthreads();
+        if (tid >= 96) return;
+        const double t = warp_of_block_sum(s_m[tid >> 5]);
+        if ((tid & 31) == 0 && t != 0.0) atomicAdd(d.mom + (tid >> 5), d.w * t);
+    }
 }
+
+using DensityKernel = void (*)(const MixedArgs, int, int, const DensityArgs);
+constexpr DensityKernel kDensityKernels[3][2] = {  // [order - 1][with momentum]
+    {k_density<1, false>, k_density<1, true>}, {k_density<2, false>, k_density<2, true>}, {k_density<3, false>, k_density<3, true>}};
 
 __global__ void k_unstage(long long n, GridDev G, PartArrays S, double* out) {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1818,6 +1840,11 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<1>, 1);
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<2>, 2);
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<3>, 3);
+    // (the densities' window at its largest: the same value from every handle)
+    const int dens = 3 * kMaxWinCells * (int)sizeof(unsigned);
+    for (const auto& k : kDensityKernels)
+        for (int mom = 0; mom < 2; mom++)
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k[mom], cudaFuncAttributeMaxDynamicSharedMemorySize, dens);
     if (rc == PIC_OK && e == cudaSuccess) {
         rc = alloc_bins(m, cap, capo, 0, err);
         if (rc == PIC_OK) e = cudaDeviceSynchronize();
@@ -1996,13 +2023,10 @@ int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, d
     // 1024 x 256, 16 per cell: 92 us against 98 with the short parts).
     const long long chunk = nbins * std::max(1ll, G.cap / 5120) < 8 * 152 ? 2560 : 5120;
     const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / chunk)));
-    const size_t sm = d.rho ? (size_t)2 * G.wx * G.wy * sizeof(unsigned) : 0;
+    const size_t sm = d.rho ? (size_t)3 * G.wx * G.wy * sizeof(unsigned) : 0;
     const MixedArgs a = make_args(m, 0);
-    switch (G.order) {
-    case 1: k_density<1><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
-    case 2: k_density<2><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
-    default: k_density<3><<<nb, 256, sm, st>>>(a, g, nbins, d); break;
-    }
+    const DensityKernel kern = kDensityKernels[G.order - 1][mom ? 1 : 0];
+    kern<<<nb, 256, sm, st>>>(a, g, nbins, d);
     MCK(cudaGetLastError());
     return PIC_OK;
 }
