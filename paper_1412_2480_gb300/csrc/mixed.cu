@@ -40,10 +40,12 @@
 #include "esirkepov.cuh"
 #include "inject.cuh"
 #include "mixed.h"
+#include "tile_plan.h"
 
 namespace pic {
 
 constexpr int kTileThreads = 256;
+static_assert(kTileThreads == kPartUnit, "parts of whole rounds of a CTA");
 constexpr double kBinSlack = 1.25;  // stayer capacity over the expected particles of a tile
 constexpr int kNbr = 8;          // outboxes per bin, one per neighbouring tile
 constexpr int kSegs = 1 + kNbr;  // count slots per bin: [0] stayers, [1 + o] outbox o
@@ -111,6 +113,7 @@ struct MixedState {
     int resident[4] = {0, 0, 0, 0}; // CTAs of each order's launch the device holds at once
     int pblocks[4] = {0, 0, 0, 0};  // persistent CTAs of each order's launch
     std::vector<long long> n;     // live particles [2 g + species]
+    std::vector<double> expect;   // particles of a tile of simulation g, both species, on average
     unsigned long long* injected = nullptr;  // device [2 ngrids]: pairs added by the injector
     int inject_grids = 0;         // simulations with an injector
     long long inject_threads = 0; // rows x most pairs per row, over those simulations
@@ -597,11 +600,14 @@ k_push_tile(const MixedArgs a) {
         }
         __syncthreads();
         // this item's range [lo, hi) of the tile's particles: species 0, padded to whole
-        // chunks, then species 1; the last part takes what is left
+        // chunks, then species 1; parts of the planned size, or equal ones where the tile
+        // holds more than was planned for
         const int v1 = (s_start[0][kSegs] + 31) & ~31;
         const int vend = v1 + s_start[1][kSegs];
-        const int lo = part * G.pchunk;
-        const int hi = part == parts - 1 ? vend : min(vend, lo + G.pchunk);
+        const int share = ((vend + parts - 1) / parts + kPartUnit - 1) / kPartUnit * kPartUnit;
+        const int chunk = max(G.pchunk, share);
+        const int lo = (int)min((long long)vend, (long long)part * chunk);
+        const int hi = part == parts - 1 ? vend : min(vend, lo + chunk);
         if (lo >= hi) continue;  // (uniform over the CTA) nothing to push, no current to add
         // The window, one node per thread and round: its wrapped (or mirrored) cell once for
         // all six components, whose loads are all in flight together.
@@ -1548,45 +1554,22 @@ int gather_species(MixedState* m, int g, int par, int s, PartArrays& S, long lon
     return PIC_OK;
 }
 
-// The tile kernels' work items. An item is a tile, or one of `parts` equal parts of its
-// particles where whole tiles are too few, or too long, to fill the device evenly. Each
-// part stages the field window and adds its own current window, and the parts of a tile
-// take their slots of the next buffer from the tile's counters in global memory. The
-// current is an integer sum and its rounding follows the tile's population, so the result
-// does not depend on the split.
-//
-// The split minimises (rounds + 0.4) (n / parts + 500) [x 1.04 if parts > 1], rounds =
-// tiles x parts / resident CTAs (1 in all where they fit at once): an item costs its n /
-// parts particles and its window, worth about 500 particles (8 us of one CTA, measured
-// from 4 to 8 parts of 2048 x 512 cells); a launch of several rounds ends, on average, in
-// a partly empty one; counters in global memory cost 4%. Measured (tile kernel per step,
-// us, one part / the chosen split / twice it): 128 x 128 cells, 100 per cell 1046 / 158
-// (14) / 171; 64 x 64, 8 per cell 75 / 21 (32) / 21; 1413 x 247, 50 per cell 989 / 971
-// (5) / 978; twelve scan simulations 1347 / 1176 (3) / 1243; 2048 x 512, 32 per cell 2698
-// (1, chosen) / 2666 (2) / 2881 (4).
+// The tile kernels' work items (tile_plan.h): the wanted size from the particles there are, the
+// parts of a tile from those its bins have room for.
 int plan_items(MixedState* m, std::string& err) {
     std::vector<int2> items;
     for (int P = 1; P <= 3; P++) {
         m->item_first[P] = (int)items.size();
-        const double tiles = m->order_n[P], resident = std::max(m->resident[P], 1);
-        double mean = 0.0;  // particles per tile that the bins are sized for
+        double mean = 0.0;
         for (int g = 0; g < m->ngrids; g++)
-            if (m->G[g].order == P) mean += m->G[g].cap * (2.0 / kBinSlack) * m->G[g].ntiles / tiles;
-        double part = mean, best = -1.0;  // particles per item
-        for (int p = 1; p <= 256 && (p == 1 || mean / p >= kTileThreads); p++) {
-            const double rounds = tiles * p / resident;
-            const double cost = (rounds <= 1.0 ? 1.0 : rounds + 0.4) * (mean / p + 500.0) * (p > 1 ? 1.04 : 1.0);
-            if (best < 0.0 || cost < best) {
-                best = cost;
-                part = mean / p;
-            }
-        }
+            if (m->G[g].order == P) mean += m->expect[g] * m->G[g].ntiles / m->order_n[P];
+        const double size = split_size(m->order_n[P], std::max(m->resident[P], 1), mean);
         for (int g = 0; g < m->ngrids; g++) {
             GridDev& G = m->G[g];
             if (G.order != P) continue;
-            const double n = G.cap * (2.0 / kBinSlack);
-            G.parts = (int)std::max(1.0, std::min(256.0, std::floor(n / part + 0.5)));
-            G.pchunk = ((int)std::ceil(n / G.parts) + kTileThreads - 1) / kTileThreads * kTileThreads;
+            const TileSplit t = split_tile(G.cap * (2.0 / kBinSlack), m->expect[g], size);
+            G.parts = t.parts;
+            G.pchunk = t.pchunk;
         }
         for (int q = m->order_first[P]; q < m->order_first[P] + m->order_n[P]; q++)
             for (int part = 0; part < m->G[m->host_tile_grid[m->tlist[q]]].parts; part++)
@@ -1651,6 +1634,8 @@ int gather_all(MixedState* m, int par, Staged& A, cudaStream_t st, std::string& 
 int place_all(MixedState* m, int par, Staged& A, std::vector<long long> cap, std::vector<long long> capo,
               cudaStream_t st, std::string& err) {
     int rc = PIC_OK;
+    for (int g = 0; g < m->ngrids; g++)  // (a species that is still to be loaded is like the other)
+        if (const long long n = std::max(A.n[2 * g], A.n[2 * g + 1])) m->expect[g] = 2.0 * n / m->G[g].ntiles;
     for (int attempt = 0; attempt < 8; attempt++) {
         rc = alloc_bins(m, cap, capo, st, err);
         if (rc) return rc;
@@ -1754,6 +1739,7 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         m->smem[D.order] = std::max(m->smem[D.order], sm);
         const double slack = q.bin_slack > 0 ? q.bin_slack : kBinSlack;
         cap[g] = round32((double)q.ppc * D.tx * D.ty * slack + 64.0);
+        m->expect.push_back(round32((double)q.ppc * D.tx * D.ty * kBinSlack + 64.0) * (2.0 / kBinSlack));
         capo[g] = round32((double)q.ppc * std::max(D.tx, D.ty) * 1.5 + 32.0);
         expect += 2ll * q.ppc * (long long)q.nx * q.ny;
     }

@@ -55,7 +55,7 @@ struct GridDev {
     long long cap;        // layered capacity rcap * cpt_pad per (tile, species) bin
     long long capo;       // capacity of each of the 8 outboxes of a bin
     long long bin_off;    // first particle slot of this simulation's bins
-    int parts, pchunk;    // work items per tile, particles of each (the last takes the rest)
+    int parts, pchunk;    // work items per tile, particles of each (tile_plan.h)
     // MIXED32 current: 64-bit fixed point, J = (double)Jfix * jinv
     double jscale, jinv;
     // MIXED32 push constants, formed once on the host from the FP64 parameters (the FP64
