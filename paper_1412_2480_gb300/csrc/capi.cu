@@ -1467,7 +1467,7 @@ int pic_spectrum(pic_sim* s, int32_t which, double* out, size_t len) {
     const double* src = nullptr;
     if (int rc = field_source(s, which, &src)) return rc;
     double* dout = nullptr;
-    CK(temp_alloc((void**)&dout, nc * sizeof(double), s->stream));
+    CK(scratch_alloc((void**)&dout, nc * sizeof(double), s->stream));
     int rc = spectrum_2d(src, G.nx, G.ny, dout, s->stream, s->err);
     cudaError_t e = cudaSuccess;
     if (rc == PIC_OK) e = cudaMemcpyAsync(out, dout, nc * sizeof(double), cudaMemcpyDefault, s->stream);
@@ -1547,11 +1547,11 @@ int pic_particles(pic_sim* s, int32_t sp, double* out, int64_t n) {
     }
     const GridDev& G = s->hgrids[0];
     // positions in physical units: straight into a caller's array on this device, else
-    // through a temporary of the library's pool
+    // through a temporary
     double* t = nullptr;
     cudaError_t e = cudaSuccess;
     const bool direct = on_device(s, out, 5 * (long long)n);
-    if (!direct) e = temp_alloc((void**)&t, 2 * (size_t)n * sizeof(double), s->stream);
+    if (!direct) e = scratch_alloc((void**)&t, 2 * (size_t)n * sizeof(double), s->stream);
     double* pos = direct ? out : t;
     if (e == cudaSuccess) {
         k_unload_fp64<<<(unsigned)((n + 255) / 256), 256, 0, s->stream>>>(n, s->pa[sp][0], s->pa[sp][1], G.dx, G.dy,
@@ -1575,7 +1575,7 @@ int pic_conservation(pic_sim* s, double* out, int32_t n_out) {
     // results (momentum, charge, max and sum of squares of the residual), block partials
     const int nb = (int)std::min<long long>(152, (G.ncell + 255) / 256);
     double* d = nullptr;
-    CK(temp_alloc((void**)&d, (6 + 3 * (size_t)nb) * sizeof(double), s->stream));
+    CK(scratch_alloc((void**)&d, (6 + 3 * (size_t)nb) * sizeof(double), s->stream));
     cudaError_t e = cudaMemsetAsync(d, 0, 3 * sizeof(double), s->stream);
     int rc = PIC_OK;
     double h[6] = {0, 0, 0, 0, 0, 0};

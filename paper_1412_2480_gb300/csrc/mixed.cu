@@ -1698,6 +1698,12 @@ cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, st);
 }
 
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+    if (bytes <= kScratchKept) return temp_alloc(p, bytes, st);
+    *p = nullptr;
+    return cudaMallocAsync(p, bytes, st);
+}
+
 void temp_free(void* p, cudaStream_t st) {
     if (p) cudaFreeAsync(p, st);
 }

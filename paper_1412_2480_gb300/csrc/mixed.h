@@ -14,8 +14,13 @@ namespace pic {
 
 struct MixedState;
 
-// Temporaries of the library's stream-ordered pool (mixed.cu).
+// Temporaries of the library's stream-ordered pool (mixed.cu), which keeps what it was given for
+// the next load or re-sort. Those of read-backs and diagnostics (scratch_alloc) are in it up
+// to kScratchKept bytes each; larger ones come from the device's default pool and go back to the
+// device. temp_free releases either.
+constexpr size_t kScratchKept = 64u << 20;
 cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st);
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
 void temp_free(void* p, cudaStream_t st);
 
 // Choose tiles and allocate bins for ngrids simulations (fills the tile fields of the

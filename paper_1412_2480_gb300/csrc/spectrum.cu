@@ -328,7 +328,7 @@ int spectrum_2d(const double* F, int nx, int ny, double* out, cudaStream_t st, s
     const Plan px = make_plan(nx), py = make_plan(ny);
     const int np = nx / 2 + 1;
     double2* W = nullptr;  // half spectrum, then the roots of both lengths
-    const cudaError_t ea = temp_alloc((void**)&W, ((size_t)np * ny + nx + ny) * sizeof(double2), st);
+    const cudaError_t ea = scratch_alloc((void**)&W, ((size_t)np * ny + nx + ny) * sizeof(double2), st);
     if (ea != cudaSuccess) {
         cudaGetLastError();
         err = std::string("spectrum scratch: ") + cudaGetErrorString(ea);
