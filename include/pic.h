@@ -98,9 +98,10 @@ extern "C" {
                               reduce the error by 4e3 at least. A simulation asking for
                               cg_rtol < 1e-13 keeps the CG (the pairs resolve about 1e-14 of
                               ||b||), and so does a handle with a grid whose nx is no
-                              multiple of 4 (the graph-driven loop's passes in one kernel). The same FP64-class test ||r|| <= rtol ||b|| ends the
-                              solve either way. NO_GRAPH, NO_COOP, EXPLICIT and CG_INNER are
-                              per handle: every simulation of a batch gives the same. */
+                              multiple of 4 (the graph-driven loop's passes in one kernel).
+                              The same FP64-class test ||r|| <= rtol ||b|| ends the solve
+                              either way. NO_GRAPH, NO_COOP, EXPLICIT and CG_INNER are per
+                              handle: every simulation of a batch gives the same. */
 
 /* ---- x boundaries ----
  * PIC_BC_WALLS closes the box in x with two perfectly conducting walls at x = 0 and
@@ -464,8 +465,10 @@ PIC_API const char* pic_last_error(const pic_sim* s);
 /* ---- bounded device-side waits -----------------------------------------------------
  * The paper has no counterpart: these are services of this library for testing its
  * failure paths. Every wait inside the library's kernels is bounded. The grid barriers
- * of the cooperative PCG (a persistent kernel whose blocks meet through global memory)
- * poll at most 2^22 times; the tensor-core completion waits of the network's kernels
+ * and grid-wide sums of the cooperative PCG (one kernel whose blocks meet through global
+ * memory: every FP64 handle's, pic_field_solve_noalloc's, and a MIXED32 handle's without
+ * PIC_NO_COOP and with at most 64 simulations) poll at most 2^22 times;
+ * the tensor-core completion waits of the network's kernels
  * at most 2^24 times. A wait that runs out makes the kernel record the failure and
  * return (a tensor-core wait that gave up first waits, with the default bound, for the
  * matrix operations it has in flight, and only then frees its tensor memory); the call
@@ -473,8 +476,11 @@ PIC_API const char* pic_last_error(const pic_sim* s);
  *
  * These calls lower the bound so that a test can make the waits run out on purpose:
  * spins >= 1 polls per wait, 0 restores the default. pic_set_wait_limit applies to the
- * handle's cooperative solve (MIXED32) from the next step on; a handle that solves
- * without it is unaffected. pic_cnn_set_wait_limit applies to the network's next calls
+ * handle's cooperative solve, FP64 or MIXED32, from the next step on; a handle that
+ * solves without it (PIC_NO_COOP, more than 64 simulations, PIC_EXPLICIT) is unaffected,
+ * and so is one whose grid is so small that one block solves it. After PIC_ETIMEOUT the
+ * fields of the failed step are not a solution of Eq. (7), as after PIC_ECG_NOCONV.
+ * pic_cnn_set_wait_limit applies to the network's next calls
  * (forward, gradient, training). Both return PIC_OK or PIC_EINVAL (spins < 0). */
 PIC_API int pic_set_wait_limit(pic_sim* s, int32_t spins);
 PIC_API int pic_cnn_set_wait_limit(pic_cnn* c, int32_t spins);
