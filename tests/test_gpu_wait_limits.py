@@ -52,7 +52,7 @@ def test_waits_run_out_and_the_handle_goes_on(sizes, precision, graph):
 
 
 def test_one_block_waits_for_nobody():
-    h = _handle([(8, 8)], pic.PIC_FP64)
+    h = _handle([(9, 9)], pic.PIC_MIXED32)  # (the FP64 PCG spreads 64 cells over two blocks)
     try:
         pic.pic_set_wait_limit(h, 1)
         pic.pic_step(h, 2)
