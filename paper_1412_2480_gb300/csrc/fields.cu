@@ -483,7 +483,7 @@ __device__ bool grid_sum(double v, double scale, bool inv, double out[2], double
                 if (all_arrived(seen, epoch, gridDim.x)) break;
                 if (++it > limit) {
                     ok = 0;
-                    atomicExch(timeout, 1u);
+                    atomicAdd(timeout, 1u);
                     break;
                 }
             }

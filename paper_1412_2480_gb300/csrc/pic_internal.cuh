@@ -106,7 +106,7 @@ struct DevStatus {
     unsigned long long ovf_count[2]; // MIXED32: particles in each overflow list
     unsigned long long loop_iters[2]; // PCG loop iterations run: [0] CG (inner) iterations,
                                       // [1] FP64 refinements (MIXED32 outer iterations)
-    unsigned int sync_timeout;        // a grid barrier of the cooperative solve ran out
+    unsigned int sync_timeout;        // waits of the cooperative solve that ran out
     unsigned int spin_limit;          // polls of a grid-barrier wait before it gives up (0: 2^22)
 };
 
@@ -316,7 +316,7 @@ static __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned 
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
             if (all_arrived(seen, epoch, nblocks)) break;
             if (++it > limit) {
-                atomicExch(timeout, 1u);
+                atomicAdd(timeout, 1u);
                 ok = 0;
                 break;
             }

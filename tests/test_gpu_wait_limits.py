@@ -59,3 +59,21 @@ def test_one_block_waits_for_nobody():
         assert 0 < pic.pic_moments(h)["cg_rel_resid"] <= 1e-10
     finally:
         pic.pic_free(h)
+
+
+@pytest.mark.parametrize("sizes,precision", [([(128, 128)], pic.PIC_FP64), ([(258, 130)], pic.PIC_MIXED32),
+                                             ([(256, 128)], pic.PIC_MIXED32)])
+def test_every_wait_that_runs_out_is_reported(sizes, precision):
+    h = _handle(sizes, precision)
+    try:
+        pic.pic_set_wait_limit(h, 1)
+        for k in range(3):
+            with pytest.raises(pic.PicError) as e:
+                pic.pic_step(h, 2)
+            assert e.value.code == pic.PIC_ETIMEOUT, (k, e.value)
+            assert pic.pic_moments(h)["step"] == k + 1
+        pic.pic_set_wait_limit(h, 0)
+        pic.pic_step(h, 2)
+        assert 0 < pic.pic_moments(h)["cg_rel_resid"] <= 1e-10
+    finally:
+        pic.pic_free(h)
