@@ -58,3 +58,22 @@ def test_gradients_against_64_bit_sums(nimg, nx, ny):
         gb = grad[b0:b0 + co].astype(np.float64)
         assert np.all(gb[3:] == 0.0)
         assert np.abs(gb[:3] / b - 1.0).max() <= (12 + 5 + 3) * 2.0 ** -24 + joins
+
+
+def test_gradient_after_a_wait_that_ran_out_is_the_same_to_the_bit():
+    rng = np.random.default_rng(5)
+    x, t = (rng.standard_normal((2, 3, 64, 64)).astype(np.float32) for _ in range(2))
+    c = pic.pic_cnn_create()
+    try:
+        pic.pic_cnn_set_params(c, (rng.standard_normal(pic.PIC_CNN_NPARAMS) * 0.05).astype(np.float32))
+        want, loss = pic.pic_cnn_gradient(c, x, t)
+        pic.pic_cnn_set_wait_limit(c, 1)
+        with pytest.raises(pic.PicError) as e:
+            pic.pic_cnn_gradient(c, -2 * x, t)
+        assert e.value.code == pic.PIC_ETIMEOUT, e.value
+        pic.pic_cnn_set_wait_limit(c, 0)
+        got, loss2 = pic.pic_cnn_gradient(c, x, t)
+        np.testing.assert_array_equal(got, want)
+        assert loss2 == pytest.approx(loss, rel=1e-12)
+    finally:
+        pic.pic_cnn_free(c)
