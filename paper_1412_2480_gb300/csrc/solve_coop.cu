@@ -1186,7 +1186,11 @@ int coop_create(CoopSolve* cs, const GridDev* hg, int ngrids, bool cg_inner, std
     cs->rsplit = 3 * cs->nchunks <= 2 * nsm ? 3 : 1;
     const size_t smem = coop_smem(*cs);
     const CoopKernel kern = coop_kernel(*cs);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the attribute belongs to the kernel and other handles may need more: only ever raised)
+    cudaFuncAttributes fa{};
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kCoopThreads, smem);
     if (e == cudaSuccess && (!coop || occ < 1)) {
         *cs = CoopSolve{};
