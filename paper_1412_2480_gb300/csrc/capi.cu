@@ -1573,7 +1573,9 @@ int pic_conservation(pic_sim* s, double* out, int32_t n_out) {
     if (!out || n_out < 1) return fail(s, PIC_EINVAL, "out is NULL");
     const GridDev& G = s->hgrids[s->sel];
     // results (momentum, charge, max and sum of squares of the residual), block partials
-    const int nb = (int)std::min<long long>(152, (G.ncell + 255) / 256);
+    int nsm = 0;
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device));
+    const int nb = (int)std::min<long long>(std::min(nsm, 256), (G.ncell + 255) / 256);  // (k_gauss_end: 256 at most)
     double* d = nullptr;
     CK(scratch_alloc((void**)&d, (6 + 3 * (size_t)nb) * sizeof(double), s->stream));
     cudaError_t e = cudaMemsetAsync(d, 0, 3 * sizeof(double), s->stream);

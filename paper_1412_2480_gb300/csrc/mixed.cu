@@ -111,6 +111,7 @@ struct MixedState {
     int* work = nullptr;          // device [4]: work counter of each order's launch
     size_t smem[4] = {0, 0, 0, 0};  // dynamic shared memory of each order's launch
     int resident[4] = {0, 0, 0, 0}; // CTAs of each order's launch the device holds at once
+    int nsm = 0;                  // SMs of the device
     int pblocks[4] = {0, 0, 0, 0};  // persistent CTAs of each order's launch
     std::vector<long long> n;     // live particles [2 g + species]
     std::vector<double> expect;   // particles of a tile of simulation g, both species, on average
@@ -1813,9 +1814,9 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
     int rc = PIC_OK;
     // Shared-memory opt-in: only ever raised, since the attribute belongs to the kernel
     // and other handles in the process may need more than this one.
-    int dev = 0, nsm = 152;
+    int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->nsm, cudaDevAttrMultiProcessorCount, dev);
     auto setup = [&](auto kern, int P) {
         if (m->order_n[P] == 0) return cudaSuccess;
         cudaFuncAttributes fa{};
@@ -1826,7 +1827,7 @@ int mixed_create(MixedState** out, const pic_params* p, int ngrids, GridDev* G,
         if (r == cudaSuccess)
             r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kTileThreads, m->smem[P]);
         if (r == cudaSuccess && nb < 1) r = cudaErrorInvalidConfiguration;
-        m->resident[P] = nb * nsm;
+        m->resident[P] = nb * m->nsm;
         return r;
     };
     if (rc == PIC_OK && e == cudaSuccess) e = setup(k_push_tile<1>, 1);
@@ -1934,9 +1935,9 @@ void mixed_enqueue(MixedState* m, cudaStream_t st, int part) {
     if (part == 0) {
         const long long nj2 = (3 * m->ntot + 1) / 2;
         const int ncnt = m->ntiles_total * (2 * kSegs + 1);
-        const unsigned nb = (unsigned)std::min<long long>(8 * 152, std::max<long long>(1, (nj2 + 255) / 256));
+        const unsigned nb = (unsigned)std::min<long long>(8 * m->nsm, std::max<long long>(1, (nj2 + 255) / 256));
         k_mixed_begin<<<nb, 256, 0, st>>>(make_args(m, 0), m->ngrids, nj2, ncnt, m->work);
-        k_push_overflow<<<152, kTileThreads, 0, st>>>(make_args(m, 0));
+        k_push_overflow<<<m->nsm, kTileThreads, 0, st>>>(make_args(m, 0));
     } else if (part == 1) {
         for (int P = 1; P <= 3; P++) {
             if (m->order_n[P] == 0) continue;
@@ -2013,7 +2014,7 @@ int mixed_rho_momentum(MixedState* m, int g, const double q_s[2], double* rho, d
     // zeroing and its nodes' FP64, below a tenth of the block's time; half as many where that
     // leaves fewer than the eight blocks that an SM holds (512 x 256, 8 per cell: 30 -> 22 us;
     // 1024 x 256, 16 per cell: 92 us against 98 with the short parts).
-    const long long chunk = nbins * std::max(1ll, G.cap / 5120) < 8 * 152 ? 2560 : 5120;
+    const long long chunk = nbins * std::max(1ll, G.cap / 5120) < 8 * m->nsm ? 2560 : 5120;
     const dim3 nb((unsigned)nbins + 1, (unsigned)std::max(1ll, std::min(64ll, G.cap / chunk)));
     const size_t sm = d.rho ? (size_t)3 * G.wx * G.wy * sizeof(unsigned) : 0;
     const MixedArgs a = make_args(m, 0);
