@@ -1,6 +1,7 @@
-// fields.cu -- the implicit field solve of the particle cycle, FP64 throughout:
-//   right-hand side of Eq. (7), PCG iterations on [1 - (theta c dt)^2 Lap] dB = b, and
-//   the E, B update from Eqs. (5)-(6).
+// fields.cu -- the implicit field solve of the particle cycle: right-hand side of Eq. (7),
+//   PCG iterations on [1 - (theta c dt)^2 Lap] dB = b, and the E, B update from Eqs. (5)-(6).
+//   FP64 for PIC_FP64; for PIC_MIXED32 the right-hand side and the updates in FP32 pairs, the
+//   inner CG in FP32, its refinements in FP64 (solve_coop.cu holds the other form of it).
 //
 // One thread per cell handles the three components of every vector. Reductions use
 // per-block partials and a "last block finishes" step per simulation (fixed summation

@@ -11,26 +11,29 @@
 // slots sit at its own offsets.
 //
 // Per step (inside the captured step graph):
-//   0. k_mixed_begin clears the current and the next buffer's counts; k_push_overflow: particles parked in the overflow list (no room
-//      in a bin; normally none) are pushed straight from global memory;
+//   0. k_mixed_begin clears the current and the next buffer's counts; k_push_overflow:
+//      particles parked in the overflow list (no room in a bin; normally none) are pushed
+//      straight from global memory;
 //   1. k_push_tile<P>, one persistent launch per shape order P present: each CTA takes
-//      the next tile of that order, or part of a tile, from a device work counter (tiles
-//      listed largest first, so uneven simulations balance across the SMs), stages the FP32 field window
-//      (tile + 2 cells below, 3 above, in x and y) into shared memory and zeroes a
-//      fixed-point current window of the same size. Its particles are its own stayer segment plus the eight
-//      neighbours' outboxes addressed to it. Warps run independently (no block barrier in
-//      the particle loop): each gathers E^n, B^n, pushes (Boris), moves and deposits
-//      J^{n+1/2} (Esirkepov) with native integer shared-memory atomics, then writes each
-//      particle to the next buffer's stayer segment or to the outbox of the neighbour it
-//      moved into, taking slots from warp-aggregated counters. The current
-//      window is added to the global fixed-point current at the end;
+//      the next tile of that order, or part of a tile (tile_plan.h), from a device work
+//      counter (tiles listed largest first, so uneven simulations balance across the
+//      SMs), stages the FP32 field window (tile + 2 cells below, 3 above, in x and y)
+//      into shared memory and zeroes a fixed-point current window of the same size. Its
+//      particles are its own stayer segment plus the eight neighbours' outboxes addressed
+//      to it. Warps run independently (no block barrier in the particle loop): each
+//      gathers E^n, B^n, pushes (Boris), moves and deposits J^{n+1/2} (Esirkepov) with
+//      native integer shared-memory atomics, then writes each particle to the next
+//      buffer's stayer segment or to the outbox of the neighbour it moved into, taking
+//      slots from warp-aggregated counters. The current window is added to the global
+//      fixed-point current at the end;
 //   2. k_mixed_end, after the field update: the buffers swap.
-// No global atomics are needed in steady state and no migration kernel runs. A particle
-// found outside its tile is pushed with the same arithmetic and the same current
-// rounding on global memory, so results never depend on bin capacity; a particle that
-// finds no room goes to the overflow list and the host re-sorts with larger bins after
-// the pic_step call. Count slots record every particle sent to a segment, parked ones
-// included; readers clamp them to the segment's capacity.
+// No migration kernel runs, and in steady state global atomics only add the windows and,
+// where a tile is split, take slots (one per warp and destination). A particle found
+// outside its tile is pushed with the same arithmetic and the same current rounding on
+// global memory, so results never depend on bin capacity; a particle that finds no room
+// goes to the overflow list and the host re-sorts with larger bins after the pic_step
+// call. Count slots record every particle sent to a segment, parked ones included;
+// readers clamp them to the segment's capacity.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -221,10 +224,12 @@ __device__ __forceinline__ void fixed_split(float x, float jlb, int& hi, int& lo
 }
 
 // Two contributions at once (the same four roundings each): two FP32 operations per issue
-// slot. At order 3 (48 to 65 contributions per particle) instruction issue bounds the tile
-// kernel: 8192 x 512 with 4 per cell 4837 -> 4530 us per step, a twelve-run scan of all
-// orders 1190 -> 1150. At order 2 the shared-memory data path bounds it (84% of its rate,
-// most of it bank conflicts of the atomics) and 2048 x 512 stays at 2.69 ms.
+// slot. At order 3 (48 to 65 contributions per particle, 16 warps per SM) instructions and
+// their latency bound the tile kernel (issue 61% active, shared-memory data path 68%): half
+// full 8192 x 512 with 16 per cell and species 4837 -> 4530 us per step, a twelve-run scan of
+// all orders 1190 -> 1150. At order 2 issue (70%) and the data path (73% in a cold beam, 78%
+// in a hot plasma, most of it bank conflicts of the atomics) bound it together and 2048 x 512
+// stays at 2.69 ms.
 __device__ __forceinline__ void fixed_split2(float x0, float x1, F2 jlb2, int hi[2], int lo[2]) {
     const F2 m = f2_dup(kMagic), x = f2(x0, x1);
     const F2 xr = add2(x, m);

@@ -37,7 +37,8 @@ int mixed_load(MixedState* m, int g, int sp, const double* x, const double* y, c
 // overflow-list push, 1 = tile kernels, 2 = the injector's pairs, 3 = its end (buffer
 // swap, PCG statistics).
 void mixed_enqueue(MixedState* m, cudaStream_t s, int part);
-// Host bookkeeping around a pic_step call (re-bin when bins overflowed).
+// Host bookkeeping around a pic_step call: lost bins are refused before it, overflowed ones
+// sorted anew after it.
 int mixed_before_steps(MixedState* m, cudaStream_t s, std::string& err);
 // hs: the device status as it is after the steps
 int mixed_after_steps(MixedState* m, const DevStatus& hs, cudaStream_t s, std::string& err);

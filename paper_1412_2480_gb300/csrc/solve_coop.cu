@@ -21,13 +21,13 @@
 // which keep A symmetric positive definite), so m steps of the three-term Chebyshev
 // recurrence on that interval reduce every error component by 1/T_m(sigma),
 // sigma = c0 / (2 (cx + cy)) >= 5/4 here, with no inner products. Step k at a cell needs
-// step k-1 at its four neighbours, so a tile of 32 x 64 cells loaded with a halo of 12
-// >= m - 1 cells in shared memory computes all m steps by itself (the halo's outer ring
-// goes stale one cell per step and never reaches the interior) and adds its interior's
-// correction to x. m is chosen per refinement from the reduction it needs (as the CG's
+// step k-1 at its four neighbours, so a tile of 32 x TY cells (TY = 64, 32 or 16, by how
+// many tiles the grid has) loaded with a halo of 12 >= m - 1 cells in shared memory
+// computes all m steps by itself (the halo's outer ring goes stale one cell per step and
+// never reaches the interior) and adds its interior's correction to x. m is chosen per refinement from the reduction it needs (as the CG's
 // inner tolerance is), at most 13 (1/T_13(2) = 7e-8 at CFL 1, theta 1/2, near the FP32
 // floor). During the solve x is held as FP32 pairs and the residual pass runs in pair
-// arithmetic (dword.cuh), so no FP64 instruction is spent inside a refinement; x is
+// arithmetic (dword.cuh), so a cell costs no FP64 instruction inside a refinement; x is
 // joined back to FP64 at the end. A refinement costs two grid barriers (tiles,
 // residual) instead of two per inner iteration. PIC_CG_INNER, or a simulation's
 // cg_rtol below 1e-13, keeps the CG. Every nx is a multiple of 4 here; the other grids'
@@ -600,8 +600,8 @@ __device__ __forceinline__ void chunk_phase(const CoopArgs& a, const ChunkC& q, 
 //                  d_k = rho_k rho_{k-1} d_{k-1} + (2 rho_k / delta) t_k,  e_{k+1} = e_k + d_k.
 // The window holds the tile and kChebHalo >= m - 1 cells around it (wrapped
 // periodically; at a wall the columns beyond it are dead and the wall's images are
-// applied exactly). Thread tid < 224 owns window column tid % 56 and the 22-row strip
-// tid / 56: r sc, d and e of its cells stay in registers; e also goes to shared memory
+// applied exactly). Thread tid < 224 owns window column tid % 56 and the strip tid / 56 of
+// 22, 14 or 10 rows (kRows): r sc, d and e of its cells stay in registers; e also goes to shared memory
 // each step (two buffers, one barrier per step) for the neighbouring columns and the
 // strips above and below. The ring of ghost cells around the window stays zero.
 
