@@ -162,10 +162,10 @@ __device__ __forceinline__ double partials_warp(const double* p, int n) {
 }
 
 // Block sums of N FP32 values per thread, added up in FP64, in out[0..N): warp c sums value c,
-// as warp_of_block_sum does.
+// as warp_of_block_sum does. s_v: N x 256 floats of shared memory (the tiles' staging area, idle
+// then: 4 KB more per CTA would take the L1 cache a step down).
 template <int N>
-__device__ __forceinline__ void block_sums(const float (&v)[N], double* out) {
-    __shared__ float s_v[N][kCoopThreads];
+__device__ __forceinline__ void block_sums(const float (&v)[N], double* out, float (*s_v)[kCoopThreads]) {
     static_assert(kCoopThreads == 256, "eight values per lane");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
@@ -564,7 +564,8 @@ __device__ __forceinline__ void residual_quads(const CoopArgs& a, const ChunkC& 
 
 // Components c0 .. c0 + NC - 1 of a chunk's pair residual and their partial sums.
 template <int NC>
-__device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, int g, int ch, int c0, double* part) {
+__device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, int g, int ch, int c0, double* part,
+                                           float (*s_v)[kCoopThreads]) {
     const ChunkC q = chunk_consts(a, s, g, ch, 0);
     float acc[NC];
 #pragma unroll
@@ -576,7 +577,7 @@ __device__ __forceinline__ void pair_chunk(const CoopArgs& a, const GState& s, i
         for (int qq = 0; qq < kQuads; qq++)
             if (q.l0 + 4 * (qq * kCoopThreads + (int)threadIdx.x) < q.ncell) residual_quads<NC, 1>(a, q, c0, qq, acc);
     }
-    block_sums<NC>(acc, part + c0);
+    block_sums<NC>(acc, part + c0, s_v);
 }
 
 template <int PH>
@@ -830,13 +831,15 @@ __global__ void __launch_bounds__(kCoopThreads, CHEB ? 2 : 4) k_mp_coop(const __
     // and component either way, from one accumulator per thread and component.
     auto pair_pass = [&]() {
         double* part = a.part_dw + (size_t)pbuf * 3 * a.nchunks;
+        static_assert(2 * ChebTile<TY>::kInterior >= 3 * kCoopThreads, "staging area holds the sums");
+        float(*s_v)[kCoopThreads] = reinterpret_cast<float(*)[kCoopThreads]>(ew + 2 * ChebTile<TY>::kCells);
         const int nitems = a.nchunks * a.rsplit;
         for (int it = blockIdx.x; it < nitems; it += nb) {
             const int ch = it / a.rsplit;
             const int g = __ldg(a.chunk_grid + ch);
             if (!(gs[g].active && gs[g].dw)) continue;  // uniform over the CTA
-            if (a.rsplit == 3) pair_chunk<1>(a, gs[g], g, ch, it - 3 * ch, part + 3 * (size_t)ch);
-            else pair_chunk<3>(a, gs[g], g, ch, 0, part + 3 * (size_t)ch);
+            if (a.rsplit == 3) pair_chunk<1>(a, gs[g], g, ch, it - 3 * ch, part + 3 * (size_t)ch, s_v);
+            else pair_chunk<3>(a, gs[g], g, ch, 0, part + 3 * (size_t)ch, s_v);
         }
     };
     // One pass over this CTA's chunks of the simulations taking part in `ph`, with
