@@ -15,9 +15,9 @@
 // What bounds it is the FP64 pipe (two lanes per cycle and SM here), so the work is cut
 // where the result allows it: twiddles come from a table of the N-th roots of unity made
 // once per call (a sincospi per element was three quarters of the operations); the field
-// is real, so two rows go through one complex transform, only the columns p <= nx/2 are
-// transformed and the others' amplitudes are |F^(nx - p, ny - q)|; the direct sums fold
-// index l with N - l, and take several rows (columns) per root. 1024 x 256: 328 -> 56 us.
+// is real, so only the columns p <= nx/2 are transformed and the others' amplitudes are
+// |F^(nx - p, ny - q)|; the direct sums fold index l with N - l, and take several rows
+// (columns) per root. 1024 x 256: 328 -> 68 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -106,7 +106,8 @@ __device__ __forceinline__ void dft_small(double2 v[R], const double2* __restric
             double2 e = v[0], o = make_double2(0.0, 0.0);
 #pragma unroll
             for (int j = 1; j <= H; j++) {
-                const double2 w = __ldg(tw + (j * k) % R * (n / R));  // (cos, -sin)
+                double2 w = __ldg(tw + (j * k) % R * (n / R));  // (cos, -sin)
+                if (R == 3) w.x = -0.5;  // (a third is no FP64 number, nor then the table's root)
                 e.x += a[j - 1].x * w.x;
                 e.y += a[j - 1].y * w.x;
                 o.x -= b[j - 1].y * w.y;
@@ -171,23 +172,19 @@ __device__ __forceinline__ void fft_smem(double2* buf, const Plan& p, const doub
 // The half spectrum of the rows lies column by column: W[p ny + m] = row m's DFT at p, 0 <=
 // p <= nx/2, so a column is contiguous.
 
-// Rows 2 b and 2 b + 1 as the real and imaginary part of one transform along x.
+// A row as the real part of a transform along x. (Two rows as the real and imaginary part of
+// one, 93 -> 81 us for 1024 x 256, 872 -> 635 for 8192 x 512, take an addition more per value:
+// the spectrum was 4 to 13% further from the exact one than from transforms of real rows.)
 template <int T, int NMAX>
 __global__ void __launch_bounds__(T, 1) k_fft_rows(const double* __restrict__ F, int nx, int ny, const Plan p,
                                                 const double2* __restrict__ tw, double2* __restrict__ W) {
     extern __shared__ double2 sbuf[];
-    const int m = 2 * blockIdx.x;
-    const bool pair = m + 1 < ny;
+    const int m = blockIdx.x;
     const double* f0 = F + (long long)m * nx;
-    for (int l = threadIdx.x; l < nx; l += T) sbuf[l] = make_double2(f0[l], pair ? f0[nx + l] : 0.0);
+    for (int l = threadIdx.x; l < nx; l += T) sbuf[l] = make_double2(f0[l], 0.0);
     __syncthreads();
     fft_smem<T, NMAX>(sbuf, p, tw);
-    for (int k = threadIdx.x; k <= nx / 2; k += T) {
-        const double2 z = sbuf[k], y = sbuf[k == 0 ? 0 : nx - k];  // Z(k), Z(n - k)
-        double2* w = W + (long long)k * ny + m;
-        w[0] = make_double2(0.5 * (z.x + y.x), 0.5 * (z.y - y.y));
-        if (pair) w[1] = make_double2(0.5 * (z.y + y.y), 0.5 * (y.x - z.x));
-    }
+    for (int k = threadIdx.x; k <= nx / 2; k += T) W[(long long)k * ny + m] = sbuf[k];
 }
 
 // |.| * scale at wave number (p, q) and at its conjugate (nx - p, ny - q).
@@ -344,9 +341,9 @@ int spectrum_2d(const double* F, int nx, int ny, double* out, cudaStream_t st, s
     if (px.direct)
         k_dft_rows<<<dim3(blocks(np, kDftThreads), blocks(ny, kDftLines)), kDftThreads, 0, st>>>(F, nx, ny, twx, W);
     else if (nx <= kShort)
-        k_fft_rows<256, kShort><<<blocks(ny, 2), 256, nx * sizeof(double2), st>>>(F, nx, ny, px, twx, W);
+        k_fft_rows<256, kShort><<<(unsigned)ny, 256, nx * sizeof(double2), st>>>(F, nx, ny, px, twx, W);
     else
-        k_fft_rows<1024, kMaxN><<<blocks(ny, 2), 1024, nx * sizeof(double2), st>>>(F, nx, ny, px, twx, W);
+        k_fft_rows<1024, kMaxN><<<(unsigned)ny, 1024, nx * sizeof(double2), st>>>(F, nx, ny, px, twx, W);
     if (py.direct)
         k_dft_cols<<<dim3(blocks(ny / 2 + 1, kDftThreads), blocks(np, kDftCols)), kDftThreads, 0, st>>>(W, nx, ny, twy,
                                                                                                    scale, out);
